@@ -148,12 +148,14 @@ int sem_destroy(sem_ctx* ctx);
  *   on the context's own fields. Patches are bricks of neighbouring elements
  *   (1 x 4 x 2 at NGLL 5; SEM_OPT_PATCH_SHAPE sets another, sem_patch_info gives the shape in
  *   use) evaluated by one CTA each, which
- *   sums the forces meeting at each of the brick's nodes in a fixed order and writes each
- *   node once; the bricks are coloured so that no two of a colour share a node (Sec. IV-C's
- *   colouring applied to groups of elements).
- *     0 (default) = patches, one launch per patch colour (with several shots one CTA per
- *       patch and shot);
- *     1 = element by element, one launch per element colour (the form always used for
+ *   sums the forces meeting at each of the brick's nodes in a fixed order; the bricks are
+ *   coloured so that no two of a colour share a node (Sec. IV-C's colouring applied to groups of
+ *   elements), which orders the sums at the nodes that bricks share.
+ *     0 (default) = patches, one launch over all of them: the nodes of one brick are completed
+ *       by it, and at the nodes bricks share every brick leaves its sum, which a second launch
+ *       adds up in the order of the colours (with several shots one CTA per patch and shot or
+ *       shot pair). Also used for caller-layout arrays;
+ *     1 = element by element, one launch per element colour (2 and 3 use this form for
  *       caller-layout arrays);
  *     2 = patches, all colours in one persistent launch (single shot; several shots use 0):
  *       CTAs take patches in sweep order
@@ -181,22 +183,21 @@ int sem_destroy(sem_ctx* ctx);
  *   captured time step are not affected. */
 #define SEM_OPT_SWEEP_STALL_TEST 4
 /*   SEM_OPT_FUSED_NEWMARK (takes effect at once; used with SEM_OPT_ASSEMBLY 0): 2 (default)
- *   = 1 for a single shot, 0 for several (where the separate pass over the shot-innermost
- *   fields measures faster); 1 = time steps run the Newmark update (Sec. I) inside the force
- *   sweep: the patch that touches a node last in the sweep adds the step's point sources to
- *   the node's complete force and runs the corrector of step n fused with the predictor of
- *   step n+1 there, so a
- *   step is one receiver-sampling launch plus the sweep, with no separate pass over the
- *   nodes; sem_step / sem_run start with a predictor pass and end with a sweep that runs the
+ *   = 1; 1 = time steps run the Newmark update (Sec. I) inside the force sweep: where a node's
+ *   force becomes complete, the step's point sources are added to it and the corrector of step
+ *   n fused with the predictor of step n+1 runs there, so a step is the two launches of the
+ *   sweep (which also sample the receivers), with no separate pass over the nodes;
+ *   sem_step / sem_run start with a predictor pass and end with a sweep that runs the
  *   corrector alone, so the state is complete between calls. 0 = separate Newmark passes
  *   (one fused corrector/predictor pass per step; the state between calls is completed on
  *   demand). Both give bitwise equal wavefields and seismograms. */
 #define SEM_OPT_FUSED_NEWMARK 6
-/*   SEM_OPT_SHOT_PAIRS (takes effect at once; several shots, SEM_OPT_ASSEMBLY 0): 1 (default)
- *   = each CTA of the patch sweep takes one patch for two shots, every thread carrying both
- *   shots as float32 pairs (one packed fma for both; each geometry and modulus value read
- *   once for both); 0 = one CTA per patch and shot. The same arithmetic per shot; results
- *   differ only by the rounding order of a few sums. */
+/*   SEM_OPT_SHOT_PAIRS (takes effect at once; several shots, SEM_OPT_ASSEMBLY 0): 1 = each CTA
+ *   of the patch sweep takes one patch for two shots, every thread carrying both shots as
+ *   float32 pairs (one packed fma for both; each geometry and modulus value read
+ *   once for both); 0 = one CTA per patch and shot; until it is set, pairs up to NGLL 6 (not at
+ *   3) for even shot counts and odd ones from 13 on, where they measure faster. The same
+ *   arithmetic per shot; results differ only by the rounding order of a few sums. */
 #define SEM_OPT_SHOT_PAIRS 7
 /*   SEM_OPT_PATCH_SHAPE (applied by the next sem_set_mesh): the brick of elements one CTA of
  *   the patch sweep takes, value = bx | by << 8 | bz << 16 in elements along the mesh's
@@ -371,8 +372,8 @@ int sem_run_record_snapshots(sem_ctx* ctx, int nsteps, float* seis_dev, float* u
 int sem_check_finite(sem_ctx* ctx);
 
 /* One matrix-free stiffness application on the device: f_dev = -K u_dev, both
- * [nglob][3] float32 in the caller's node order (Sec. II-B), by the element kernel, colour
- * by colour. Every node of f_dev is written. u_dev and f_dev must not overlap. Allocates
+ * [nglob][3] float32 in the caller's node order (Sec. II-B), assembled as SEM_OPT_ASSEMBLY
+ * says. Every node of f_dev is written. u_dev and f_dev must not overlap. Allocates
  * nothing. Asynchronous on the context's stream. Does not touch the solver state. */
 int sem_apply_stiffness(sem_ctx* ctx, const float* u_dev, float* f_dev);
 
@@ -385,8 +386,9 @@ int sem_apply_stiffness_strided(sem_ctx* ctx, const float* u_dev, float* f_dev, 
 
 /* The solver's internal node order: perm[i] = caller node of internal node i, int32[nglob].
  * sem_set_mesh numbers the nodes so that every patch of the force sweep finds its nodes in
- * runs: the nodes a patch touches first (patch colour by patch colour) get consecutive
- * numbers, grouped by the set of patches that share them. Every call that takes or returns
+ * runs: the nodes of one patch only first, patch by patch, then the nodes that patches share,
+ * those a patch touches first (patch colour by patch colour) with consecutive numbers, grouped
+ * by the set of patches that share them. Every call that takes or returns
  * node data (states, snapshots, sources, receivers, sem_apply_stiffness, sem_node_xyz)
  * uses the caller's order; only sem_apply_stiffness_strided with stride 4 uses this one.
  * SEM_ESTATE before sem_set_mesh. */
@@ -440,16 +442,16 @@ int sem_tune_patch_shape(sem_ctx* ctx, int nspec, int nglob, const int32_t* iboo
 
 /* Profile nsteps time steps (Sec. I, IV-C), launched one by one with CUDA events on the
  * context's stream around each step's force sweep: ms_out[0] = mean milliseconds of the
- * sweep (all of its colour launches; with SEM_OPT_FUSED_NEWMARK the Newmark update and the
- * sources included), ms_out[1] = mean milliseconds per step of everything else (receiver
- * sampling, separate Newmark passes, the predictor that starts a run). The state advances
+ * sweep (all of its launches; with SEM_OPT_FUSED_NEWMARK the Newmark update, the sources and
+ * the receiver sampling included), ms_out[1] = mean milliseconds per step of everything else
+ * (separate Newmark passes and receiver sampling, the predictor that starts a run). The state advances
  * as with sem_step (same results); no seismogram is recorded. Blocks until the steps are
  * done. SEM_EINVAL if nsteps < 1 or ms_out is NULL. */
 int sem_profile_steps(sem_ctx* ctx, int nsteps, double* ms_out);
 
 /* Groups: several contexts on one GPU (different meshes, orders, shot counts) stepped
- * together. sem_group_step advances every context nsteps steps (no seismograms): one eager
- * step per context, then CUDA graphs of the remaining steps. In the persistent mode
+ * together. sem_group_step advances every context nsteps steps (no seismograms): an eager
+ * start (or step) per context, then CUDA graphs of the remaining steps. In the persistent mode
  * (SEM_GROUP_MODE 1; used when every context has one shot, SEM_OPT_ASSEMBLY 0 and at most
  * 64 patch colours, and the group at most 64 contexts) a step is the contexts'
  * Newmark passes, ONE persistent force-sweep launch for all contexts of the same order and

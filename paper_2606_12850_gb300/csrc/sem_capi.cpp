@@ -50,7 +50,7 @@ struct sem_ctx {
   int stall_test = 0;               // SEM_OPT_SWEEP_STALL_TEST (one-shot)
   int fuse_newmark = 2;             // SEM_OPT_FUSED_NEWMARK: Newmark update in the patch sweep
                                     // (1 on, 0 off, 2 on for a single shot)
-  int shot_pairs = 1;               // SEM_OPT_SHOT_PAIRS: patch CTAs per shot pair (1) or shot (0)
+  int shot_pairs = 2;               // SEM_OPT_SHOT_PAIRS: 1 pairs, 0 one CTA a shot, 2 (default) by pair_rule
   PatchShape shape_opt{0, 0, 0};    // SEM_OPT_PATCH_SHAPE for the next sem_set_mesh (0: the order's)
   PatchShape shape{0, 0, 0};        // the bricks of the current mesh
   std::vector<PatchDesc> pdesc;     // host copy of the patch descriptors
@@ -79,7 +79,16 @@ struct sem_ctx {
   uint16_t* d_pwords = nullptr;   // patch tables: shared patch node -> its first point's ibool word
   int* d_pcolor_end = nullptr;    // per patch colour, the end of its patch range
   SweepSync* d_sync = nullptr;    // counters of the persistent sweep
-  PatchSrc* d_psrc = nullptr;     // point sources by the patch that touches their node last
+  PatchSrc* d_psrc = nullptr;     // point sources by the patch of their inner node
+  PatchSrc* d_rsrc = nullptr;     // point sources by the block of their rim node
+  int ninner = 0;                 // internal ids below it are inner nodes, the others rim nodes
+  size_t nrimsums = 0;            // partials the sweep leaves for the rim pass (per shot)
+  RimNode* d_rim = nullptr;       // per rim node the partials that meet there
+  int* d_rimover = nullptr;       // its lists of more than four
+  RimBlock* d_rblocks = nullptr;  // per kRimBlock rim nodes their sources and receivers
+  std::vector<RimBlock> rblocks;
+  float* d_rimsums = nullptr;     // the partials, laid out like a field
+  int ahead = 0;                  // fused steps enqueued since d_ctl was last set or advanced
   float *d_u = nullptr, *d_v = nullptr, *d_a = nullptr, *d_minv = nullptr;
   float* d_f = nullptr;           // scratch force buffer for sem_energy
   float *d_lam = nullptr, *d_lam_old = nullptr, *d_lamF = nullptr;  // adjoint fields [nglob][4]
@@ -87,8 +96,8 @@ struct sem_ctx {
   float* d_grad32 = nullptr;      // [3][nlocal] float32 partial sums, flushed into d_grad
   int since_flush = 0;            // adjoint steps accumulated in d_grad32
   int node_order = 0;             // SEM_OPT_NODE_ORDER: device state arrays in caller (0) or internal (1) order
-  PatchRecv* d_precv = nullptr;   // receivers by the patch that touches their node last
-  int* d_precv_range = nullptr;   // [npatch][2] first, count into d_precv
+  PatchRecv* d_precv = nullptr;   // receivers by patch (PatchDesc rec_off, nrec, nrec_in)
+  PatchRecv* d_rrecv = nullptr;   // receivers by the block of their rim node
   int* d_rnode = nullptr;         // distinct receiver nodes (internal ids)
   int* d_roff = nullptr;          // their receivers: d_rlist[d_roff[t] .. d_roff[t+1])
   int* d_rlist = nullptr;
@@ -100,7 +109,7 @@ struct sem_ctx {
   int* d_src_shot = nullptr;
   double* d_src_force = nullptr;
   int nsrc = 0;
-  int shots = 1;  // wavefields [nglob][shots][kNodeStride]
+  int shots = 1;  // wavefields fields of kNodeStride floats per node and shot
   double f0 = 0.0, t0 = 0.0;
   int* d_rec_node = nullptr;
   int nrec = 0;
@@ -162,9 +171,10 @@ int dev_alloc(sem_ctx* c, T** p, size_t count) {
 }
 
 void free_device(sem_ctx* c) {
-  void* ptrs[] = {c->d_rec, c->d_order, c->d_elist, c->d_perm, c->d_node_new, c->d_pdesc, c->d_pslots, c->d_pwords, c->d_pcolor_end, c->d_sync, c->d_psrc, c->d_u, c->d_v,
+  void* ptrs[] = {c->d_rec, c->d_order, c->d_elist, c->d_perm, c->d_node_new, c->d_pdesc, c->d_pslots, c->d_pwords, c->d_pcolor_end, c->d_sync, c->d_psrc, c->d_rsrc, c->d_rim, c->d_rimover,
+                  c->d_rblocks, c->d_rimsums, c->d_u, c->d_v,
                   c->d_a, c->d_minv, c->d_f, c->d_partials, c->d_lam, c->d_lam_old, c->d_lamF, c->d_grad,
-                  c->d_grad32, c->d_precv, c->d_precv_range, c->d_rnode, c->d_roff, c->d_rlist,
+                  c->d_grad32, c->d_precv, c->d_rrecv, c->d_rnode, c->d_roff, c->d_rlist,
                   c->d_ctl, c->d_src_node, c->d_src_shot, c->d_src_force, c->d_rec_node};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -178,14 +188,17 @@ void free_device(sem_ctx* c) {
   c->d_pwords = nullptr;
   c->d_pcolor_end = nullptr;
   c->d_sync = nullptr;
-  c->d_psrc = nullptr;
+  c->d_psrc = c->d_rsrc = nullptr;
+  c->d_rim = nullptr;
+  c->d_rimover = nullptr;
+  c->d_rblocks = nullptr;
+  c->d_rimsums = nullptr;
   c->d_u = c->d_v = c->d_a = c->d_minv = c->d_f = nullptr;
   c->d_lam = c->d_lam_old = c->d_lamF = nullptr;
   c->d_grad = nullptr;
   c->d_grad32 = nullptr;
   c->d_rnode = c->d_roff = c->d_rlist = nullptr;
-  c->d_precv = nullptr;
-  c->d_precv_range = nullptr;
+  c->d_precv = c->d_rrecv = nullptr;
   c->nrnodes = 0;
   c->adjoint = false;
   c->d_partials = nullptr;
@@ -237,46 +250,74 @@ int set_device(sem_ctx* c) {
   return SEM_OK;
 }
 
-// f = -K u over all colours (Sec. IV-C: colour by colour, no atomics). On the context's own
-// fields the patch kernel takes the patch colours in order (one launch per colour, one CTA
-// per patch and shot; patches of a colour share no node). Otherwise (caller arrays, or
-// SEM_OPT_ASSEMBLY = 1) the element kernel walks the element list slab by slab and, inside a
-// slab, colour by colour: a launch holds elements of one colour only.
-// With nm (mode 1 or 2; only on the per-colour patch path, see fused_sweep) the sweep also
-// runs the Newmark update of every node at the patch that touches it last.
+// Whether several shots are swept in pairs. GB300, 24 steps of about 3.4e5 points: 16 shots in
+// pairs against one CTA a shot 2.78 / 2.99 ms at NGLL 5, 2.59 / 2.89 at 4, 3.57 / 4.15 at 6, but
+// 3.65 / 3.51 at 7, 4.53 / 3.95 at 8, 4.62 / 4.49 at 9 (one resident CTA, or spills, for the two
+// shots' registers); an odd count leaves half of the last pair idle (3 shots at NGLL 5: 0.77 /
+// 0.69 ms), which a tenth gained on the others pays back from 13 shots on.
+bool pair_rule(const sem_ctx* c, int shots) {
+  if (c->shot_pairs != 2) return c->shot_pairs == 1;
+  return c->ngll <= 6 && c->ngll != 3 && (shots % 2 == 0 || shots >= 13);
+}
+
+// f = -K u. On the context's own fields the patch sweep (one launch, one CTA per patch and
+// shot or shot pair) completes the inner nodes, and the rim pass sums the partials it left at
+// the nodes patches share: no atomics, a fixed order of every sum. SEM_OPT_ASSEMBLY 2 takes the
+// patch colours in order in one persistent launch (Sec. IV-C's colouring, applied to patches).
+// Caller arrays [nglob][3] go through the same sweep, read and written through the node
+// permutation (mode 4). With SEM_OPT_ASSEMBLY 1 the element kernel
+// walks the element list slab by slab and, inside a slab, colour by colour: a launch holds
+// elements of one colour only.
+// With nm (mode 1, 2 or 3; see fused_sweep) both passes also run the update of every node.
 int forces_all_colors(sem_ctx* c, const float* u, float* f, int node_stride, int shots,
                       const SweepNewmark* nm = nullptr) {
-  if ((c->assembly == 0 || c->assembly == 2) && node_stride == kNodeStride && c->npatch > 0) {
+  const bool caller = node_stride == 3;
+  if (c->npatch > 0 && (c->assembly == 0 || (c->assembly == 2 && !caller))) {
     PatchLaunch P{};
     if (nm) P.nm = *nm;
+    P.nm.nglob = c->nglob;
+    P.nm.nsums = static_cast<int>(c->nrimsums);
     P.rec = c->d_rec;
     P.desc = c->d_pdesc;
     P.slots = c->d_pslots;
     P.words = c->d_pwords;
     P.u = u;
     P.f = f;
+    P.partials = c->d_rimsums;
+    P.npatch = c->npatch;
     P.variant = c->variant;
     P.shots = shots;
-    P.pairs = c->shot_pairs;
+    P.pairs = pair_rule(c, shots);
+    if (caller) {
+      P.nm.mode = 4;
+      P.nm.perm = c->d_perm;
+    }
     const int npc = static_cast<int>(c->pcolor_off.size()) - 1;
     if (c->assembly == 2 && shots == 1 && npc <= kMaxSweepColors && P.nm.mode == 0) {
       P.sync = c->d_sync;
       P.color_end = c->d_pcolor_end;
-      P.npatch = c->npatch;
       P.ncolors = npc;
       P.stall = c->stall_test;
       c->stall_test = 0;
       SEM_LAUNCH(c, launch_patch_forces(c->ngll, P, c->stream));
       return SEM_OK;
     }
-    for (size_t k = 0; k + 1 < c->pcolor_off.size(); ++k) {
-      P.p0 = c->pcolor_off[k];
-      P.p1 = c->pcolor_off[k + 1];
-      SEM_LAUNCH(c, launch_patch_forces(c->ngll, P, c->stream));
-    }
+    SEM_LAUNCH(c, launch_patch_forces(c->ngll, P, c->stream));
+    RimLaunch R{};
+    R.rim = c->d_rim;
+    R.over = c->d_rimover;
+    R.blocks = c->d_rblocks;
+    R.partials = c->d_rimsums;
+    R.f = f;
+    R.ninner = c->ninner;
+    R.nrim = c->nglob - c->ninner;
+    R.shots = shots;
+    R.nm = P.nm;
+    SEM_LAUNCH(c, launch_rim_combine(R, c->stream));
     return SEM_OK;
   }
   ForceLaunch L{};
+  L.nglob = c->nglob;
   L.rec = c->d_rec;
   L.elist = c->d_elist;
   L.perm = c->d_perm;
@@ -306,13 +347,11 @@ int forces_all_colors(sem_ctx* c, const float* u, float* f, int node_stride, int
   return SEM_OK;
 }
 
-// Whether time steps run the fused sweep: the per-colour patch sweep (SEM_OPT_ASSEMBLY 0)
-// with SEM_OPT_FUSED_NEWMARK on (by default for a single shot only: with several shots the
-// separate pass over the [nglob][S][4] fields is faster on GB300, 48^3 at NGLL 5 with 32
-// shots: 11.8 ms per step against 13.1 ms).
-bool fused_sweep(const sem_ctx* c) {
-  return (c->fuse_newmark == 1 || (c->fuse_newmark == 2 && c->shots == 1)) && c->assembly == 0 && c->npatch > 0;
-}
+// Whether time steps run the fused sweep: the patch sweep (SEM_OPT_ASSEMBLY 0) with
+// SEM_OPT_FUSED_NEWMARK not 0. With several shots too: GB300, 20^3 at NGLL 5, 24 steps, 32
+// shots 14.8 ms against 17.1 ms with a separate pass, 4 shots 2.09 against 2.47 ms (before the
+// shots were kept in pairs the separate pass, which streams, was the faster one).
+bool fused_sweep(const sem_ctx* c) { return c->fuse_newmark != 0 && c->assembly == 0 && c->npatch > 0; }
 
 SweepNewmark sweep_newmark(const sem_ctx* c, int mode) {
   SweepNewmark nm{};
@@ -322,7 +361,12 @@ SweepNewmark sweep_newmark(const sem_ctx* c, int mode) {
   nm.a = c->d_a;
   nm.minv = c->d_minv;
   nm.src = c->d_psrc;
-  nm.step = &c->d_ctl->step;
+  nm.rim_src = c->d_rsrc;
+  nm.recv = c->d_precv;
+  nm.rim_recv = c->d_rrecv;
+  nm.nrec = c->nrec;
+  nm.ctl = c->d_ctl;
+  nm.ahead = c->ahead;
   nm.f0 = c->f0;
   nm.t0 = c->t0;
   nm.dtd = c->dt;
@@ -333,16 +377,42 @@ SweepNewmark sweep_newmark(const sem_ctx* c, int mode) {
 }
 
 // One step of the fused sweep from u_{n+1} (predicted) and the half-step velocity: the
-// receivers sample u_{n+1} and the step counter advances to n+1, then the sweep assembles
-// the forces and, at each node's last touch, adds the step's point sources and runs the
-// corrector of step n fused with the predictor of step n+1 (mode 1), or the corrector alone
-// (mode 2, the last step of a run: the state is complete afterwards).
+// receivers sample u_{n+1}, then sweep and rim pass assemble the forces, add the step's point
+// sources and run, node by node, the corrector of step n fused with the predictor of step n+1
+// (mode 1), or the corrector alone (mode 2, the last step of a run: the state is complete
+// afterwards). The step's index is the device counter plus the steps enqueued since it was
+// last written (c->ahead), so the kernels of a step need not count.
 int enqueue_fused_step(sem_ctx* c, int mode) {
-  DevProblem p = problem(c);
-  p.nsrc = 0;  // the sweep adds the sources
-  SEM_LAUNCH(c, launch_sources_record(p, c->stream));
   const SweepNewmark nm = sweep_newmark(c, mode);
-  return forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots, &nm);
+  const int r = forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots, &nm);
+  ++c->ahead;
+  return r;
+}
+
+// Writes the device counter: step n, an empty seismogram of ncols columns (and snapshots).
+int set_ctl(sem_ctx* c, long long step, int ncols, float* seis, float* snap = nullptr, long long snap_per = 0) {
+  SEM_LAUNCH(c, launch_set_ctl(c->d_ctl, step, ncols, seis, c->stream, snap, snap_per));
+  c->ahead = 0;
+  return SEM_OK;
+}
+
+// Brings the device counter up to date, as captured steps count from it.
+int settle_ctl(sem_ctx* c) {
+  if (c->ahead) SEM_LAUNCH(c, launch_advance_ctl(c->d_ctl, c->ahead, c->stream));
+  c->ahead = 0;
+  return SEM_OK;
+}
+
+// Enqueues `steps` steps for capture, which advance the device counter at their end.
+template <class Step>
+int enqueue_captured(sem_ctx* c, int steps, Step step) {
+  const int ahead = c->ahead;
+  c->ahead = 0;
+  int r = SEM_OK;
+  for (int s = 0; s < steps && r == SEM_OK; ++s) r = step();
+  c->ahead = ahead;
+  if (r == SEM_OK) SEM_LAUNCH(c, launch_advance_ctl(c->d_ctl, steps, c->stream));
+  return r;
 }
 
 // One time step in the "pending" representation (a holds M a_raw of the previous step, v
@@ -356,7 +426,8 @@ int enqueue_step(sem_ctx* c, bool first) {
     SEM_LAUNCH(c, launch_fused_newmark(p, c->stream));
   int r = forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots);
   if (r) return r;
-  SEM_LAUNCH(c, launch_sources_record(p, c->stream));
+  SEM_LAUNCH(c, launch_sources_record(p, c->ahead, c->stream));
+  ++c->ahead;
   return SEM_OK;
 }
 int enqueue_pending_step(sem_ctx* c) { return enqueue_step(c, false); }
@@ -367,8 +438,7 @@ int build_graph(sem_ctx* c) {
   cudaGraph_t g = nullptr;
   const bool fused = fused_sweep(c);
   SEM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-  int r = SEM_OK;
-  for (int s = 0; s < kStepsPerGraph && r == SEM_OK; ++s) r = fused ? enqueue_fused_step(c, 1) : enqueue_pending_step(c);
+  const int r = enqueue_captured(c, kStepsPerGraph, [&] { return fused ? enqueue_fused_step(c, 1) : enqueue_pending_step(c); });
   cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (r != SEM_OK) {
     if (g) cudaGraphDestroy(g);
@@ -394,6 +464,7 @@ int advance_fused(sem_ctx* c, int nsteps) {
   int left = nsteps - 1;
   if (left >= kStepsPerGraph && (!c->graph_valid || !c->graph_fused))
     if ((r = build_graph(c))) return r;
+  if (left >= kStepsPerGraph && (r = settle_ctl(c))) return r;
   for (; left >= kStepsPerGraph; left -= kStepsPerGraph) SEM_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
   for (; left > 0; --left)
     if ((r = enqueue_fused_step(c, 1))) return r;
@@ -415,7 +486,7 @@ int advance(sem_ctx* c, int nsteps, float* seis_dev, bool fused = true) {
   if (r) return r;
   if (nsteps < 0) return fail(c, SEM_EINVAL, "nsteps must be >= 0");
   if ((r = set_device(c))) return r;
-  SEM_LAUNCH(c, launch_set_ctl(c->d_ctl, c->steps, seis_dev ? nsteps : 0, seis_dev, c->stream));
+  if ((r = set_ctl(c, c->steps, seis_dev ? nsteps : 0, seis_dev))) return r;
   if (fused && fused_sweep(c)) {
     if (nsteps > 0 && (r = advance_fused(c, nsteps))) return r;
     c->steps += nsteps;
@@ -429,6 +500,7 @@ int advance(sem_ctx* c, int nsteps, float* seis_dev, bool fused = true) {
   }
   if (left >= kStepsPerGraph && (!c->graph_valid || c->graph_fused))
     if ((r = build_graph(c))) return r;
+  if (left >= kStepsPerGraph && (r = settle_ctl(c))) return r;
   while (left >= kStepsPerGraph) {
     SEM_CUDA(c, cudaGraphLaunch(c->graph, c->stream));
     left -= kStepsPerGraph;
@@ -901,7 +973,7 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
             g |= kFirstTouchBit;
           }
           std::memcpy(&r[kIbool * np + p], &g, sizeof(uint32_t));
-          for (int a = 0; a < 9; ++a) r[(kG + a) * np + q] = gq[a * np + p];
+          for (int a = 0; a < 9; ++a) r[rec_at(np, a, q)] = gq[a * np + p];
           r[kJac * np + q] = gq[9 * np + p];
         }
   }
@@ -909,9 +981,12 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
   // ibool word of its first local point in that patch's table, the points alone at their
   // patch node on their own words; the slot tables become shared-memory offsets of the
   // patch kernel's workspaces
-  int ES = 0, TS = 0, EPT = 0;
-  if (patch_layout(n, &ES, &TS, &EPT)) return fail(c, SEM_EINVAL, "no patch layout for this order");
-  auto ws_float = [&](int le) { return (le / EPT) * TS + (le % EPT) * ES; };
+  PatchLayout lay{};
+  if (patch_layout(n, &lay)) return fail(c, SEM_EINVAL, "no patch layout for this order");
+  // float of local point pp of element le in the sweep's workspace, and in the persistent ones'
+  auto ws_point = [&](int pp) { return 3 * (pp % n + lay.sy * ((pp / n) % n) + lay.sz * (pp / (n * n))); };
+  auto ws_float = [&](int le, int pp) { return (le / lay.e) * lay.ts + (le % lay.e) * lay.es + ws_point(pp); };
+  auto wsw_element = [&](int le) { return (le / lay.e) * lay.tsw + (le % lay.e) * lay.esw; };
   std::vector<uint16_t> slots(plan.csr.size(), kPatchNoSlot), words;
   std::vector<int> word_off(plan.tab_nelem.size(), 0);
   for (size_t t = 0; t < plan.tab_nelem.size(); ++t) {
@@ -925,17 +1000,117 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
         continue;
       }
       const int le = v / np, pp = v % np;
-      const int off = ws_float(le) + 3 * pp;
+      const int off = wsw_element(le) + ws_point(pp);
       if (off >= kPatchChain) return fail(c, SEM_EINVAL, "patch workspace offsets exceed the slot range");
       slots[q] = static_cast<uint16_t>(off);
       if ((q - g0) % kPatchSlots == 0 && (q - g0) / kPatchSlots < static_cast<size_t>(plan.tab_nshared[t])) {
-        const int wo = ws_float(le) + 9 * np + pp;  // a shared node's first slot
+        const int wo = wsw_element(le) + lay.words + pp;  // a shared node's first slot
         if (wo > 0xFFFF) return fail(c, SEM_EINVAL, "patch workspace offsets exceed the word range");
         words.push_back(static_cast<uint16_t>(wo));
       }
     }
   }
+  // the tables of the one-launch sweep: per patch its inner nodes in id order (those met by one
+  // point, then the others) and its rim nodes (ascending internal id, the order of their
+  // partials); patches with the same lists share them
+  struct Lists {
+    int table;
+    std::vector<uint16_t> rim;  // patch node indices, in partial order
+    int nalone, nin, alone_off, in_slots, rim_slots;
+  };
+  std::vector<Lists> lists;
+  std::unordered_map<uint64_t, std::vector<int>> lists_by_hash;
+  std::vector<int> lists_of(plan.npatch);
+  slots.resize((slots.size() + kPatchSlots - 1) / kPatchSlots * kPatchSlots, kPatchNoSlot);
+  {
+    std::vector<std::pair<int, int>> order;  // (internal id, patch node)
+    std::vector<uint16_t> rim;
+    for (int P = 0; P < plan.npatch; ++P) {
+      const int t = plan.table_of[P];
+      const int nn = plan.node_off[P + 1] - plan.node_off[P];
+      order.clear();
+      for (int k = 0; k < nn; ++k) {
+        const int g = plan.node_new[plan.nodes[plan.node_off[P] + k] & ~kFirstTouchBit];
+        if (g >= plan.ninner) order.emplace_back(g, k);
+      }
+      std::sort(order.begin(), order.end());
+      rim.clear();
+      uint64_t h = 1469598103934665603ull ^ static_cast<uint64_t>(t);  // 64-bit FNV-1a
+      for (const std::pair<int, int>& x : order) {
+        rim.push_back(static_cast<uint16_t>(x.second));
+        h = (h ^ static_cast<uint64_t>(x.second)) * 1099511628211ull;
+      }
+      int found = -1;
+      for (int l : lists_by_hash[h])
+        if (lists[l].table == t && lists[l].rim == rim) {
+          found = l;
+          break;
+        }
+      if (found < 0) {
+        const int nelem = plan.patch_off[P + 1] - plan.patch_off[P];
+        const uint16_t* lid = plan.lid.data() + plan.tab_lid_off[t];
+        std::vector<std::vector<int>> con(nn);  // local points at each patch node, ascending
+        for (int q = 0; q < nelem * np; ++q) con[lid[q]].push_back(q);
+        std::vector<char> is_rim(nn, 0);
+        for (uint16_t k : rim) is_rim[k] = 1;
+        bool fits = true;
+        // one slot group per node, in the list's order, chained groups after them
+        auto add_groups = [&](const std::vector<int>& nodes_k) {
+          const size_t g0 = slots.size() / kPatchSlots;
+          slots.resize(slots.size() + nodes_k.size() * kPatchSlots, kPatchNoSlot);
+          for (size_t i = 0; i < nodes_k.size(); ++i) {
+            size_t g = g0 + i, k = 0;
+            const std::vector<int>& pts = con[nodes_k[i]];
+            for (size_t q = 0; q < pts.size(); ++q) {
+              if (k == kPatchSlots - 1 && q + 1 < pts.size()) {
+                const size_t ng = slots.size() / kPatchSlots;
+                if (ng - g0 >= kPatchChain) fits = false;
+                slots[g * kPatchSlots + k] = static_cast<uint16_t>(kPatchChain | (ng - g0));
+                slots.resize(slots.size() + kPatchSlots, kPatchNoSlot);
+                g = ng;
+                k = 0;
+              }
+              const int off = ws_float(pts[q] / np, pts[q] % np);
+              if (off >= kPatchChain) fits = false;
+              slots[g * kPatchSlots + k++] = static_cast<uint16_t>(off);
+            }
+          }
+          return static_cast<int>(g0);
+        };
+        Lists l;
+        l.table = t;
+        l.rim = rim;
+        // inner nodes in id order: the ones met by one point, then the others
+        std::vector<int> inner, rimk(rim.begin(), rim.end());
+        l.nalone = 0;
+        l.alone_off = static_cast<int>(words.size());
+        for (int k = 0; k < nn; ++k) {
+          if (is_rim[k]) continue;
+          if (con[k].size() > 1) {
+            inner.push_back(k);
+            continue;
+          }
+          const int off = ws_float(con[k][0] / np, con[k][0] % np);
+          if (off >= kPatchChain) fits = false;
+          words.push_back(static_cast<uint16_t>(off));
+          ++l.nalone;
+        }
+        l.nin = static_cast<int>(inner.size());
+        l.in_slots = add_groups(inner);
+        l.rim_slots = add_groups(rimk);
+        if (!fits) return fail(c, SEM_EINVAL, "patch workspace offsets exceed the slot range");
+        if (slots.size() / kPatchSlots > 0x7FFFFFFFull || words.size() > 0x7FFFFFFFull)
+          return fail(c, SEM_EINVAL, "patch tables too large");
+        found = static_cast<int>(lists.size());
+        lists.push_back(std::move(l));
+        lists_by_hash[h].push_back(found);
+      }
+      lists_of[P] = found;
+    }
+  }
   std::vector<PatchDesc> pdesc(plan.npatch);
+  size_t nrimsums = 0;
+  int inner_next = 0;
   auto flag_word = [&](int slot, int pp, uint32_t bit) {
     float* r = c->rec.data() + static_cast<size_t>(slot) * RW;
     uint32_t wd;
@@ -956,7 +1131,20 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
     d.nshared = plan.tab_nshared[t];
     d.slot_off = plan.tab_csr_off[t];
     d.word_off = word_off[t];
-    d.src_off = d.nsrc = d.pad = 0;
+    d.src_off = d.nsrc = d.rec_off = d.nrec = d.nrec_in = 0;
+    const Lists& l = lists[lists_of[P]];
+    d.nalone = l.nalone;
+    d.alone_off = l.alone_off;
+    d.nin = l.nin;
+    d.in_slots = l.in_slots;
+    d.inner0 = inner_next;
+    inner_next += l.nalone + l.nin;
+    d.pad[0] = d.pad[1] = 0;
+    d.nrim = static_cast<int>(l.rim.size());
+    d.rim_slots = l.rim_slots;
+    d.rim0 = static_cast<int>(nrimsums);
+    nrimsums += l.rim.size();
+    if (nrimsums > 0x7FFFFFFFull) return fail(c, SEM_EINVAL, "mesh too large for int32 indexing");
     const uint16_t* lid = plan.lid.data() + plan.tab_lid_off[t];
     for (int q = 0; q < d.nelem * np; ++q)
       if (last_patch[plan.nodes[plan.node_off[P] + lid[q]] & ~kFirstTouchBit] == P)
@@ -971,6 +1159,35 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
     for (int q = 0; q < d.nelem * np; ++q)
       if ((ex[q / 32] >> (q % 32)) & 1u) flag_word(d.slot0 + q / np, q % np, kAloneBit);
   }
+  // the partials that meet at each rim node, in sweep order
+  const int nrim = nglob - plan.ninner;
+  std::vector<RimNode> rim(nrim);
+  std::vector<int> rimover;
+  {
+    std::vector<int> off(static_cast<size_t>(nrim) + 1, 0);
+    auto rim_of = [&](int P, int k) {
+      return plan.node_new[plan.nodes[plan.node_off[P] + lists[lists_of[P]].rim[k]] & ~kFirstTouchBit] - plan.ninner;
+    };
+    for (int P = 0; P < plan.npatch; ++P)
+      for (int k = 0; k < pdesc[P].nrim; ++k) off[rim_of(P, k) + 1]++;
+    for (int t = 0; t < nrim; ++t) off[t + 1] += off[t];
+    std::vector<int> sums(nrimsums), fill(off.begin(), off.end() - 1);
+    for (int P = 0; P < plan.npatch; ++P)
+      for (int k = 0; k < pdesc[P].nrim; ++k) sums[fill[rim_of(P, k)]++] = pdesc[P].rim0 + k;
+    for (int t = 0; t < nrim; ++t) {
+      const int* s0 = sums.data() + off[t];
+      const int m = off[t + 1] - off[t];
+      rim[t] = RimNode{s0[0], s0[1], m > 2 ? s0[2] : -1, m > 3 ? s0[3] : -1};
+      if (m > 4) {
+        rim[t].w = -2 - static_cast<int>(rimover.size());
+        rimover.push_back(m - 3);
+        rimover.insert(rimover.end(), s0 + 3, s0 + m);
+      }
+    }
+  }
+  c->ninner = plan.ninner;
+  c->nrimsums = nrimsums;
+  c->rblocks.assign((static_cast<size_t>(nrim) + kRimBlock - 1) / kRimBlock, RimBlock{0, 0, 0, 0});
   c->last_patch.assign(nglob, -1);
   for (int g = 0; g < nglob; ++g) c->last_patch[plan.node_new[g]] = last_patch[g];
   c->pdesc = pdesc;
@@ -999,13 +1216,16 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
   free_device(c);
   c->d_ctl = keep_ctl;
   c->dev_bytes = sizeof(DevCtl);
-  const size_t nf = kNodeStride * static_cast<size_t>(nglob) * c->shots;
+  const size_t nf = kNodeStride * static_cast<size_t>(nglob) * padded_shots(c->shots);
   if ((r = dev_alloc(c, &c->d_rec, c->rec.size())) || (r = dev_alloc(c, &c->d_order, c->order.size())) ||
       (r = dev_alloc(c, &c->d_elist, elist.size())) || (r = dev_alloc(c, &c->d_pdesc, pdesc.size())) ||
       (r = dev_alloc(c, &c->d_perm, c->perm.size())) || (r = dev_alloc(c, &c->d_node_new, c->node_new.size())) ||
       (r = dev_alloc(c, &c->d_pslots, std::max<size_t>(slots.size(), kPatchSlots))) ||
       (r = dev_alloc(c, &c->d_pwords, std::max<size_t>(words.size(), 1))) ||
       (r = dev_alloc(c, &c->d_pcolor_end, static_cast<size_t>(plan.ncolors))) || (r = dev_alloc(c, &c->d_sync, 1)) ||
+      (r = dev_alloc(c, &c->d_rim, rim.size())) || (r = dev_alloc(c, &c->d_rimover, rimover.size())) ||
+      (r = dev_alloc(c, &c->d_rblocks, c->rblocks.size())) ||
+      (r = dev_alloc(c, &c->d_rimsums, kNodeStride * nrimsums * padded_shots(c->shots))) ||
       (r = dev_alloc(c, &c->d_u, nf)) ||
       (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf)) ||
       (r = dev_alloc(c, &c->d_minv, static_cast<size_t>(nglob))))
@@ -1026,6 +1246,14 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
                                 c->stream));
   if (!words.empty())
     SEM_CUDA(c, cudaMemcpyAsync(c->d_pwords, words.data(), words.size() * sizeof(uint16_t), cudaMemcpyHostToDevice,
+                                c->stream));
+  if (nrim > 0) {
+    SEM_CUDA(c, cudaMemcpyAsync(c->d_rim, rim.data(), rim.size() * sizeof(RimNode), cudaMemcpyHostToDevice, c->stream));
+    SEM_CUDA(c, cudaMemcpyAsync(c->d_rblocks, c->rblocks.data(), c->rblocks.size() * sizeof(RimBlock),
+                                cudaMemcpyHostToDevice, c->stream));
+  }
+  if (!rimover.empty())
+    SEM_CUDA(c, cudaMemcpyAsync(c->d_rimover, rimover.data(), rimover.size() * sizeof(int), cudaMemcpyHostToDevice,
                                 c->stream));
   SEM_CUDA(c, cudaMemcpyAsync(c->d_pcolor_end, plan.color_off.data() + 1, plan.ncolors * sizeof(int),
                               cudaMemcpyHostToDevice, c->stream));
@@ -1200,31 +1428,47 @@ int sem_locate_nodes(sem_ctx* c, int npts, const double* xyz, const double* surf
 
 // The point sources of the fused sweep: entry s (internal node, shot, force) goes to the patch
 // that touches its node last; the descriptors name each patch's range.
+// The patch descriptors and rim blocks, after their sources or receivers changed.
+static int upload_places(sem_ctx* c) {
+  SEM_CUDA(c, cudaMemcpy(c->d_pdesc, c->pdesc.data(), c->pdesc.size() * sizeof(PatchDesc), cudaMemcpyHostToDevice));
+  if (!c->rblocks.empty())
+    SEM_CUDA(c, cudaMemcpy(c->d_rblocks, c->rblocks.data(), c->rblocks.size() * sizeof(RimBlock), cudaMemcpyHostToDevice));
+  return SEM_OK;
+}
+
 static int set_patch_sources(sem_ctx* c, const std::vector<int>& nodes, const std::vector<int>& shots,
                              const std::vector<double>& forces) {
   if (c->npatch <= 0) return SEM_OK;
-  std::vector<std::pair<int, int>> by_patch;  // (patch, entry), in entry order within a patch
-  for (size_t s = 0; s < nodes.size(); ++s) by_patch.emplace_back(c->last_patch[nodes[s]], static_cast<int>(s));
-  std::stable_sort(by_patch.begin(), by_patch.end(),
+  // (patch, or past the patches the rim block; entry), in entry order within one of them
+  std::vector<std::pair<int, int>> by_place;
+  for (size_t s = 0; s < nodes.size(); ++s) {
+    const int g = nodes[s];
+    by_place.emplace_back(g < c->ninner ? c->last_patch[g] : c->npatch + (g - c->ninner) / kRimBlock, static_cast<int>(s));
+  }
+  std::stable_sort(by_place.begin(), by_place.end(),
                    [](const std::pair<int, int>& x, const std::pair<int, int>& y) { return x.first < y.first; });
-  std::vector<PatchSrc> list(by_patch.size());
+  std::vector<PatchSrc> list, rim;
   for (PatchDesc& d : c->pdesc) d.src_off = d.nsrc = 0;
-  for (size_t k = 0; k < by_patch.size(); ++k) {
-    const int P = by_patch[k].first, s = by_patch[k].second;
-    PatchSrc& e = list[k];
-    e.node = nodes[s];
-    e.shot = shots[s];
-    for (int d = 0; d < 3; ++d) e.f[d] = forces[3 * static_cast<size_t>(s) + d];
-    PatchDesc& d = c->pdesc[P];
-    if (d.nsrc == 0) d.src_off = static_cast<int>(k);
-    ++d.nsrc;
+  for (RimBlock& b : c->rblocks) b.src_off = b.nsrc = 0;
+  for (const std::pair<int, int>& x : by_place) {
+    PatchSrc e{};
+    e.node = nodes[x.second];
+    e.shot = shots[x.second];
+    for (int d = 0; d < 3; ++d) e.f[d] = forces[3 * static_cast<size_t>(x.second) + d];
+    const bool inner = x.first < c->npatch;
+    std::vector<PatchSrc>& to = inner ? list : rim;
+    int& off = inner ? c->pdesc[x.first].src_off : c->rblocks[x.first - c->npatch].src_off;
+    int& n = inner ? c->pdesc[x.first].nsrc : c->rblocks[x.first - c->npatch].nsrc;
+    if (n++ == 0) off = static_cast<int>(to.size());
+    to.push_back(e);
   }
   int r = dev_alloc(c, &c->d_psrc, list.size());
-  if (r) return r;
+  if (r || (r = dev_alloc(c, &c->d_rsrc, rim.size()))) return r;
   if (!list.empty())
     SEM_CUDA(c, cudaMemcpy(c->d_psrc, list.data(), list.size() * sizeof(PatchSrc), cudaMemcpyHostToDevice));
-  SEM_CUDA(c, cudaMemcpy(c->d_pdesc, c->pdesc.data(), c->pdesc.size() * sizeof(PatchDesc), cudaMemcpyHostToDevice));
-  return SEM_OK;
+  if (!rim.empty())
+    SEM_CUDA(c, cudaMemcpy(c->d_rsrc, rim.data(), rim.size() * sizeof(PatchSrc), cudaMemcpyHostToDevice));
+  return upload_places(c);
 }
 
 static int set_sources_impl(sem_ctx* c, int nsrc, const int32_t* shot, const int32_t* node, const double* force,
@@ -1393,7 +1637,8 @@ int sem_set_shots(sem_ctx* c, int nshots) {
   int r = set_device(c);
   if (r) return r;
   cudaStreamSynchronize(c->stream);
-  const size_t old = kNodeStride * static_cast<size_t>(c->nglob) * c->shots * sizeof(float);
+  const size_t old = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots) * sizeof(float);
+  const size_t old_sums = kNodeStride * c->nrimsums * padded_shots(c->shots) * sizeof(float);
   c->dev_bytes -= 3 * old;
   if (c->d_f) {
     c->dev_bytes -= old;
@@ -1401,8 +1646,11 @@ int sem_set_shots(sem_ctx* c, int nshots) {
     c->d_f = nullptr;
   }
   c->shots = nshots;
-  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * nshots;
-  if ((r = dev_alloc(c, &c->d_u, nf)) || (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf))) return r;
+  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(nshots);
+  c->dev_bytes -= old_sums;
+  if ((r = dev_alloc(c, &c->d_u, nf)) || (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf)) ||
+      (r = dev_alloc(c, &c->d_rimsums, kNodeStride * c->nrimsums * padded_shots(nshots))))
+    return r;
   SEM_CUDA(c, cudaMemsetAsync(c->d_u, 0, nf * sizeof(float), c->stream));
   SEM_CUDA(c, cudaMemsetAsync(c->d_v, 0, nf * sizeof(float), c->stream));
   SEM_CUDA(c, cudaMemsetAsync(c->d_a, 0, nf * sizeof(float), c->stream));
@@ -1465,24 +1713,40 @@ int sem_set_receiver_nodes(sem_ctx* c, int nrec, const int32_t* node) {
     SEM_CUDA(c, cudaMemcpy(c->d_roff, roff.data(), roff.size() * sizeof(int), cudaMemcpyHostToDevice));
     SEM_CUDA(c, cudaMemcpy(c->d_rlist, byn.data(), byn.size() * sizeof(int), cudaMemcpyHostToDevice));
   }
-  // the same receivers by the patch that touches their node last (the fused adjoint sweep),
-  // ascending receiver index within a patch
+  // the same receivers by patch (at inner nodes, then at rim nodes the patch touches last) and,
+  // at rim nodes, by rim block; ascending receiver index within each
   if (c->npatch > 0) {
-    std::vector<std::pair<int, int>> by_patch;  // (patch, receiver)
-    for (int k = 0; k < nrec; ++k) by_patch.emplace_back(c->last_patch[internal[k]], k);
-    std::sort(by_patch.begin(), by_patch.end());
-    std::vector<PatchRecv> list(by_patch.size());
-    std::vector<int> range(2 * static_cast<size_t>(c->npatch), 0);
-    for (size_t k = 0; k < by_patch.size(); ++k) {
-      const int P = by_patch[k].first, rr = by_patch[k].second;
-      list[k] = PatchRecv{internal[rr], rr};
-      if (range[2 * P + 1] == 0) range[2 * P] = static_cast<int>(k);
-      ++range[2 * P + 1];
+    struct Place {
+      int patch, rim, r;
+    };
+    std::vector<Place> at;
+    for (int k = 0; k < nrec; ++k) at.push_back({c->last_patch[internal[k]], internal[k] >= c->ninner, k});
+    std::sort(at.begin(), at.end(), [](const Place& x, const Place& y) {
+      return x.patch != y.patch ? x.patch < y.patch : x.rim != y.rim ? x.rim < y.rim : x.r < y.r;
+    });
+    for (PatchDesc& d : c->pdesc) d.rec_off = d.nrec = d.nrec_in = 0;
+    for (RimBlock& b : c->rblocks) b.rec_off = b.nrec = 0;
+    std::vector<PatchRecv> list(at.size()), rim;
+    std::vector<std::pair<int, int>> by_block;  // (rim block, receiver)
+    for (size_t k = 0; k < at.size(); ++k) {
+      list[k] = PatchRecv{internal[at[k].r], at[k].r};
+      PatchDesc& d = c->pdesc[at[k].patch];
+      if (d.nrec++ == 0) d.rec_off = static_cast<int>(k);
+      if (!at[k].rim) ++d.nrec_in;
+      if (at[k].rim) by_block.emplace_back((internal[at[k].r] - c->ninner) / kRimBlock, at[k].r);
     }
-    if ((r = dev_alloc(c, &c->d_precv, list.size())) || (r = dev_alloc(c, &c->d_precv_range, range.size()))) return r;
+    std::sort(by_block.begin(), by_block.end());
+    for (const std::pair<int, int>& x : by_block) {
+      RimBlock& b = c->rblocks[x.first];
+      if (b.nrec++ == 0) b.rec_off = static_cast<int>(rim.size());
+      rim.push_back(PatchRecv{internal[x.second], x.second});
+    }
+    if ((r = dev_alloc(c, &c->d_precv, list.size())) || (r = dev_alloc(c, &c->d_rrecv, rim.size()))) return r;
     if (!list.empty())
       SEM_CUDA(c, cudaMemcpy(c->d_precv, list.data(), list.size() * sizeof(PatchRecv), cudaMemcpyHostToDevice));
-    SEM_CUDA(c, cudaMemcpy(c->d_precv_range, range.data(), range.size() * sizeof(int), cudaMemcpyHostToDevice));
+    if (!rim.empty())
+      SEM_CUDA(c, cudaMemcpy(c->d_rrecv, rim.data(), rim.size() * sizeof(PatchRecv), cudaMemcpyHostToDevice));
+    if ((r = upload_places(c))) return r;
   }
   drop_graph(c);
   return SEM_OK;
@@ -1505,7 +1769,7 @@ static int set_state_impl(sem_ctx* c, const float* u, const float* v, const floa
   for (int q = 0; q < 3 && rc == SEM_OK; ++q) {
     cudaError_t e = cudaSuccess;
     if (!src[q]) {
-      e = cudaMemsetAsync(dst[q], 0, kNodeStride * static_cast<size_t>(c->nglob) * c->shots * sizeof(float), c->stream);
+      e = cudaMemsetAsync(dst[q], 0, kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots) * sizeof(float), c->stream);
     } else {
       const float* from = src[q];
       if (host) {
@@ -1530,7 +1794,7 @@ static int set_state_impl(sem_ctx* c, const float* u, const float* v, const floa
     SEM_CUDA(c, cudaStreamSynchronize(c->stream));
     if (bad) {
       for (float* d : dst)
-        SEM_CUDA(c, cudaMemsetAsync(d, 0, kNodeStride * static_cast<size_t>(c->nglob) * c->shots * sizeof(float), c->stream));
+        SEM_CUDA(c, cudaMemsetAsync(d, 0, kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots) * sizeof(float), c->stream));
       SEM_CUDA(c, cudaStreamSynchronize(c->stream));
       return fail(c, SEM_EINVAL, "non-finite state value (the state was reset to zero)");
     }
@@ -1598,7 +1862,7 @@ int sem_run_record_snapshots(sem_ctx* c, int nsteps, float* seis_dev, float* u_d
   const size_t per = 3 * static_cast<size_t>(c->nglob) * c->shots;
   const int* perm = c->node_order == 1 ? nullptr : c->d_perm;
   if (!fused_sweep(c)) {
-    SEM_LAUNCH(c, launch_set_ctl(c->d_ctl, c->steps, seis_dev ? nsteps : 0, seis_dev, c->stream));
+    if ((r = set_ctl(c, c->steps, seis_dev ? nsteps : 0, seis_dev))) return r;
     for (int k = 0; k < nsteps; ++k) {
       if (!c->pending) {
         if ((r = enqueue_first_step(c))) return r;
@@ -1611,44 +1875,43 @@ int sem_run_record_snapshots(sem_ctx* c, int nsteps, float* seis_dev, float* u_d
     c->steps += nsteps;
     return SEM_OK;
   }
-  // fused sweep: the predictor once, then per step the receivers sample u^{n+1}, which is
-  // also the snapshot (the sweep overwrites it with the next prediction), then the sweep; the
-  // snapshot slot comes from the device's step counter, so the steps replay as graphs
+  // fused sweep: the predictor once, then per step the receivers sample u^{n+1}, which is also
+  // the snapshot (the sweep overwrites it with the next prediction); the snapshot slot comes
+  // from the device's step counter, so the steps replay as graphs
   if (nsteps == 0) return SEM_OK;
   if ((r = finish_state(c))) return r;
-  SEM_LAUNCH(c, launch_set_ctl(c->d_ctl, c->steps, seis_dev ? nsteps : 0, seis_dev, c->stream, u_dev,
-                               static_cast<long long>(per)));
+  if ((r = set_ctl(c, c->steps, seis_dev ? nsteps : 0, seis_dev, u_dev, static_cast<long long>(per)))) return r;
   SEM_LAUNCH(c, launch_predictor(problem(c), c->stream));
   auto snap_step = [&](int mode) -> int {
-    DevProblem q = problem(c);
-    q.nsrc = 0;
-    SEM_LAUNCH(c, launch_sources_record(q, c->stream));
     SweepNewmark nm = sweep_newmark(c, mode);
-    if (c->shots == 1) {  // the sweep stores u^{n+1} at each node's last touch
-      nm.snap_ctl = c->d_ctl;
+    if (c->shots == 1) {  // u^{n+1} stored where it is updated
+      nm.snap = 1;
       nm.snap_perm = perm;
     } else {
-      SEM_LAUNCH(c, launch_snapshot(c->d_u, c->d_ctl, perm, c->nglob, c->shots, c->stream));
+      SEM_LAUNCH(c, launch_snapshot(c->d_u, c->d_ctl, c->ahead, perm, c->nglob, c->shots, c->stream));
     }
-    return forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots, &nm);
+    const int rs = forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots, &nm);
+    ++c->ahead;
+    return rs;
   };
   int left = nsteps - 1;
   if (left >= kStepsPerGraph && !c->graph_snap) {
     cudaGraph_t g = nullptr;
     SEM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     int rc = SEM_OK;
-    for (int s = 0; s < kStepsPerGraph && rc == SEM_OK; ++s) rc = snap_step(1);
+    rc = enqueue_captured(c, kStepsPerGraph, [&] { return snap_step(1); });
     cudaError_t e = cudaStreamEndCapture(c->stream, &g);
     if (rc == SEM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_snap, g, 0);
     if (g) cudaGraphDestroy(g);
     if (rc) return rc;
     if (e != cudaSuccess) return cuda_fail(c, e, "snapshot graph");
   }
+  if (left >= kStepsPerGraph && (r = settle_ctl(c))) return r;
   for (; left >= kStepsPerGraph; left -= kStepsPerGraph) SEM_CUDA(c, cudaGraphLaunch(c->graph_snap, c->stream));
   for (; left > 0; --left)
     if ((r = snap_step(1))) return r;
   if ((r = snap_step(2))) return r;
-  SEM_LAUNCH(c, launch_set_ctl(c->d_ctl, c->steps + nsteps, 0, nullptr, c->stream));  // forget the buffers
+  if ((r = set_ctl(c, c->steps + nsteps, 0, nullptr))) return r;  // forget the buffers
   c->steps += nsteps;
   return SEM_OK;
 }
@@ -1742,7 +2005,7 @@ int sem_energy(sem_ctx* c, double* out) {
   if (!out) return fail(c, SEM_EINVAL, "sem_energy: NULL output");
   int r = set_device(c);
   if (r || (r = finish_state(c))) return r;
-  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * c->shots;
+  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots);
   if (!c->d_f) {
     if ((r = dev_alloc(c, &c->d_f, nf)) || (r = dev_alloc(c, &c->d_partials, 2 * static_cast<size_t>(kEnergyBlocks))))
       return r;
@@ -1832,11 +2095,9 @@ int sem_adjoint_begin(sem_ctx* c) {
   return SEM_OK;
 }
 
-// Whether adjoint steps run the leapfrog inside the sweep of lam (the per-colour patch
-// sweep with SEM_OPT_FUSED_NEWMARK not 0, and the receivers' patch lists built).
-bool fused_adjoint(const sem_ctx* c) {
-  return c->fuse_newmark != 0 && c->assembly == 0 && c->npatch > 0 && (c->nrec == 0 || c->d_precv_range);
-}
+// Whether adjoint steps run the leapfrog inside the sweep of lam (the patch sweep with
+// SEM_OPT_FUSED_NEWMARK not 0).
+bool fused_adjoint(const sem_ctx* c) { return c->fuse_newmark != 0 && c->assembly == 0 && c->npatch > 0; }
 
 // One adjoint step: the sweep of lam with, at each node's last touch, the residual injection
 // and the leapfrog (or, unfused, the sweep, then the injection and leapfrog passes). G_dev is
@@ -1849,8 +2110,9 @@ static int adjoint_sweep_step(sem_ctx* c, const float* G_dev, const DevCtl* idx)
     nm.u = c->d_lam;
     nm.lam_old = c->d_lam_old;
     nm.minv = c->d_minv;
-    nm.recv_range = c->nrec > 0 && G_dev ? c->d_precv_range : nullptr;
     nm.recv = c->d_precv;
+    nm.rim_recv = c->d_rrecv;
+    nm.nrec = c->nrec;
     nm.G = idx ? nullptr : G_dev;
     nm.idx = G_dev ? idx : nullptr;
     nm.inv_dt2 = static_cast<float>(1.0 / (c->dt * c->dt));
@@ -2055,7 +2317,7 @@ int sem_profile_steps(sem_ctx* c, int nsteps, double* ms_out) {
   if ((r = set_device(c))) return r;
   const bool fused = fused_sweep(c);
   if (fused && (r = finish_state(c))) return r;
-  SEM_LAUNCH(c, launch_set_ctl(c->d_ctl, c->steps, 0, nullptr, c->stream));
+  if ((r = set_ctl(c, c->steps, 0, nullptr))) return r;
   std::vector<cudaEvent_t> ev(2 * static_cast<size_t>(nsteps) + 2, nullptr);
   int rc = SEM_OK;
   for (cudaEvent_t& e : ev)
@@ -2071,12 +2333,8 @@ int sem_profile_steps(sem_ctx* c, int nsteps, double* ms_out) {
     rc = launch_predictor(p, c->stream) ? fail(c, SEM_ECUDA, "predictor launch") : SEM_OK;
   for (int s = 0; s < nsteps && rc == SEM_OK; ++s) {
     if (fused) {
-      DevProblem q = p;
-      q.nsrc = 0;
-      if (launch_sources_record(q, c->stream)) rc = fail(c, SEM_ECUDA, "receiver launch");
       mark(1 + 2 * s);
-      const SweepNewmark nm = sweep_newmark(c, s + 1 < nsteps ? 1 : 2);
-      if (rc == SEM_OK) rc = forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots, &nm);
+      if (rc == SEM_OK) rc = enqueue_fused_step(c, s + 1 < nsteps ? 1 : 2);
       mark(2 + 2 * s);
     } else {
       if (s > 0 || c->pending)
@@ -2084,7 +2342,7 @@ int sem_profile_steps(sem_ctx* c, int nsteps, double* ms_out) {
       mark(1 + 2 * s);
       if (rc == SEM_OK) rc = forces_all_colors(c, c->d_u, c->d_a, kNodeStride, c->shots);
       mark(2 + 2 * s);
-      if (rc == SEM_OK && launch_sources_record(p, c->stream)) rc = fail(c, SEM_ECUDA, "source launch");
+      if (rc == SEM_OK && launch_sources_record(p, c->ahead++, c->stream)) rc = fail(c, SEM_ECUDA, "source launch");
     }
   }
   mark(ev.size() - 1);
@@ -2114,7 +2372,7 @@ int sem_autotune(sem_ctx* c, int reps, double* ms_out, int* choice_out) {
   if (reps < 1) return fail(c, SEM_EINVAL, "sem_autotune: reps must be >= 1");
   if ((r = set_device(c))) return r;
   if ((r = finish_state(c))) return r;  // the timing sweeps read u and write scratch only
-  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * c->shots;
+  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots);
   float* f = nullptr;
   SEM_CUDA(c, cudaMallocAsync(reinterpret_cast<void**>(&f), nf * sizeof(float), c->stream));
   cudaEvent_t ev[2] = {nullptr, nullptr};
@@ -2267,7 +2525,7 @@ int group_tables(sem_group* g) {
 
 // One pending step of every context on the group's stream with the force sweeps persistent:
 // the contexts' Newmark passes, one sweep launch per (order, form), the contexts' sources.
-int group_enqueue_persistent_step(sem_group* g, unsigned int stall) {
+int group_enqueue_persistent_step(sem_group* g, unsigned int stall, int ahead) {
   for (sem_ctx* c : g->ctx)
     if (launch_fused_newmark(problem(c), g->stream)) return group_fail(g, SEM_ECUDA, "group Newmark pass");
   for (const auto& sw : g->sweeps) {
@@ -2283,7 +2541,7 @@ int group_enqueue_persistent_step(sem_group* g, unsigned int stall) {
     if (launch_group_sweep(sw.ngll, L, g->stream)) return group_fail(g, SEM_ECUDA, "group sweep launch");
   }
   for (sem_ctx* c : g->ctx)
-    if (launch_sources_record(problem(c), g->stream)) return group_fail(g, SEM_ECUDA, "group sources");
+    if (launch_sources_record(problem(c), ahead, g->stream)) return group_fail(g, SEM_ECUDA, "group sources");
   return SEM_OK;
 }
 
@@ -2293,7 +2551,9 @@ int group_build_persistent(sem_group* g, int which, int steps) {
   cudaError_t e = cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return group_fail(g, SEM_ECUDA, std::string("cudaStreamBeginCapture: ") + cudaGetErrorString(e));
   int rc = SEM_OK;
-  for (int s = 0; s < steps && rc == SEM_OK; ++s) rc = group_enqueue_persistent_step(g, 0u);
+  for (int s = 0; s < steps && rc == SEM_OK; ++s) rc = group_enqueue_persistent_step(g, 0u, s);
+  for (sem_ctx* c : g->ctx)
+    if (rc == SEM_OK && launch_advance_ctl(c->d_ctl, steps, g->stream)) rc = group_fail(g, SEM_ECUDA, "group counters");
   e = cudaStreamEndCapture(g->stream, &graph);
   if (rc == SEM_OK && e != cudaSuccess) rc = group_fail(g, SEM_ECUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(e));
   if (rc == SEM_OK) {
@@ -2304,8 +2564,9 @@ int group_build_persistent(sem_group* g, int which, int steps) {
   return rc;
 }
 
-// One graph advancing every context by `steps` pending steps, each context on a branch of
-// its own so that the contexts' kernels may run side by side.
+// One graph advancing every context by `steps` steps (fused ones where the context runs them,
+// else pending ones), each context on a branch of its own so that the contexts' kernels may run
+// side by side.
 int group_build(sem_group* g, int which, int steps) {
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(g->stream, cudaStreamCaptureModeThreadLocal);
@@ -2320,8 +2581,9 @@ int group_build(sem_group* g, int which, int steps) {
     }
     cudaStream_t own = c->stream;
     c->stream = g->branch[i];
-    for (int s = 0; s < steps && rc == SEM_OK; ++s)
-      if (enqueue_pending_step(c) != SEM_OK) rc = group_fail(g, SEM_ECUDA, "capture of a step: " + c->err);
+    const bool fused = fused_sweep(c);
+    if (enqueue_captured(c, steps, [&] { return fused ? enqueue_fused_step(c, 1) : enqueue_pending_step(c); }) != SEM_OK)
+      rc = group_fail(g, SEM_ECUDA, "capture of a step: " + c->err);
     c->stream = own;
     if (rc == SEM_OK && (cudaEventRecord(g->ev[1 + i], g->branch[i]) != cudaSuccess ||
                          cudaStreamWaitEvent(g->stream, g->ev[1 + i], 0) != cudaSuccess))
@@ -2391,18 +2653,29 @@ int sem_group_step(sem_group* g, int nsteps) {
   cudaError_t e = cudaSetDevice(g->device);
   if (e != cudaSuccess) return group_fail(g, SEM_ECUDA, cudaGetErrorString(e));
   const size_t n = g->ctx.size();
-  // each context: step counter, then one eager step on its own stream (a first step from a
-  // complete state, or a pending one), so that all of them continue in pending form
+  // graph branches: a context that runs the fused sweep starts with the predictor and ends with
+  // a step that completes its state, both on its own stream; any other context (and every one
+  // of a persistent group) runs one eager step on its own stream (a first step from a complete
+  // state, or a pending one), so that it continues in pending form
+  const bool persistent = group_persistent_ok(g);
+  std::vector<char> fused(n, 0);
+  for (size_t i = 0; i < n; ++i)
+    if (int r = check_ready(g->ctx[i])) return group_fail(g, r, "context " + std::to_string(i) + ": " + g->ctx[i]->err);
   for (size_t i = 0; i < n; ++i) {
     sem_ctx* c = g->ctx[i];
-    int r = check_ready(c);
-    if (r) return group_fail(g, r, "context " + std::to_string(i) + ": " + c->err);
-    if ((r = advance(c, 1, nullptr, false))) return group_fail(g, r, "context " + std::to_string(i) + ": " + c->err);
+    int r = SEM_OK;
+    fused[i] = !persistent && fused_sweep(c);
+    if (fused[i]) {
+      if ((r = finish_state(c)) || (r = set_ctl(c, c->steps, 0, nullptr)))
+        return group_fail(g, r, "context " + std::to_string(i) + ": " + c->err);
+      if (launch_predictor(problem(c), c->stream)) return group_fail(g, SEM_ECUDA, "group predictor");
+    } else if ((r = advance(c, 1, nullptr, false)) || (r = settle_ctl(c))) {
+      return group_fail(g, r, "context " + std::to_string(i) + ": " + c->err);
+    }
     if (cudaEventRecord(g->ev[1 + i], c->stream) != cudaSuccess || cudaStreamWaitEvent(g->stream, g->ev[1 + i], 0) != cudaSuccess)
       return group_fail(g, SEM_ECUDA, "ordering the group after its contexts");
   }
   int left = nsteps - 1;
-  const bool persistent = group_persistent_ok(g);
   bool stale = g->gen.size() != n || g->persistent != persistent;
   for (size_t i = 0; i < n && !stale; ++i) stale = g->gen[i] != g->ctx[i]->generation;
   if (stale) {
@@ -2416,7 +2689,9 @@ int sem_group_step(sem_group* g, int nsteps) {
     }
   }
   if (persistent && g->stall && left > 0) {  // failure-detection test: one eager step whose waits give up
-    int r = group_enqueue_persistent_step(g, g->stall);
+    int r = group_enqueue_persistent_step(g, g->stall, 0);
+    for (sem_ctx* c : g->ctx)
+      if (!r && launch_advance_ctl(c->d_ctl, 1, g->stream)) r = group_fail(g, SEM_ECUDA, "group counters");
     g->stall = 0;
     if (r) return r;
     --left;
@@ -2438,7 +2713,10 @@ int sem_group_step(sem_group* g, int nsteps) {
   for (size_t i = 0; i < n; ++i) {
     if (cudaStreamWaitEvent(g->ctx[i]->stream, g->ev[0], 0) != cudaSuccess)
       return group_fail(g, SEM_ECUDA, "ordering a context after the group");
-    g->ctx[i]->steps += nsteps - 1;  // advance() counted the eager step
+    sem_ctx* c = g->ctx[i];
+    if (fused[i] && enqueue_fused_step(c, 2) != SEM_OK)
+      return group_fail(g, SEM_ECUDA, "context " + std::to_string(i) + ": " + c->err);
+    c->steps += fused[i] ? nsteps : nsteps - 1;  // advance() counted the eager step
   }
   return SEM_OK;
 }

@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "sem_internal.h"
+#include "sem_newmark.cuh"
 
 #define SEM_CAT2(a, b) a##b
 #define SEM_CAT(a, b) SEM_CAT2(a, b)
@@ -60,11 +61,63 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
 //  4. scatter in the gather's order: a store at the node's first touch, a
 //     read-modify-write otherwise (elements of one launch share no node: no atomics,
 //     fixed summation order), previous values of four points loaded before any store.
-// Shared memory per element: u (then F), eta and zeta derivatives (then fluxes) as [NP][3]
-// each (the odd per-line stride 3N keeps the xi-line accesses conflict-free), ibool as
-// [NP]; with several elements per warp the element stride is padded so that they fall in
-// disjoint banks (offsets chosen by simulating the warp's access patterns).
+// Shared memory per element: u (then F), eta and zeta derivatives (then fluxes) as planes of
+// three floats per point, ibool as [NP] (see Ws).
 // ---------------------------------------------------------------------------------------
+// Element workspace in shared memory: local point (i, j, k) at float 3 (i + SY j + SZ k) of each
+// of its three planes [PV][3] (u then F, eta values, zeta values), element stride = RES modulo 32
+// banks. SY, SZ and RES minimise the bank conflicts of a team's xi-, eta- and zeta-line accesses
+// (exhaustive search; L1 wavefronts per team, the earlier natural strides against these: NGLL 3
+// 288 against 216, 4 384 / 240, 8 4032 / 960, 9 4968 / 4536, 10 6360 / 4800; at 5, 6 and 7 the
+// natural strides are best).
+template <int N>
+struct Ws {
+  static constexpr int SY = N == 8 || N == 10 ? N + 1 : N;
+  static constexpr int SZ = N == 2 ? 5 : N == 4 ? 19 : SY * N;
+  static constexpr int PV = (SZ + SY + 1) * (N - 1) + 1;
+  static constexpr int RES = N == 2 || N == 10 ? 4 : N == 3 ? 15 : N == 4 ? 16 : N == 9 ? 11 : 0;
+  static constexpr bool NATURAL = SY == N && SZ == N * N;
+  __device__ __forceinline__ static constexpr int at(int i, int j, int k) { return 3 * (i + SY * j + SZ * k); }
+  __device__ __forceinline__ static constexpr int at(int p) {
+    return NATURAL ? 3 * p : at(p % N, (p / N) % N, p / (N * N));
+  }
+};
+
+// a b + c d + e f in one fixed rounding (the compiler's own choice of contractions depends on
+// the code around an expression).
+__device__ __forceinline__ float dot3(float a, float b, float c, float d, float e, float f) {
+  return fmaf(e, f, fmaf(a, b, c * d));
+}
+
+// The record values of one point: inverse Jacobian, J kappa, J mu.
+struct PointRec {
+  float G[9], kappa, mu;
+};
+template <int NP>
+__device__ __forceinline__ PointRec load_point(const float* __restrict__ r, int q, bool active) {
+  PointRec o;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+  float2 c = make_float2(0.f, 0.f);
+  o.mu = 0.f;
+  if (active) {
+    a = __ldg(reinterpret_cast<const float4*>(r) + q);
+    b = __ldg(reinterpret_cast<const float4*>(r + 4 * NP) + q);
+    c = __ldg(reinterpret_cast<const float2*>(r + 8 * NP) + q);
+    o.mu = __ldg(r + 10 * NP + q);
+  }
+  o.G[0] = a.x;
+  o.G[1] = a.y;
+  o.G[2] = a.z;
+  o.G[3] = a.w;
+  o.G[4] = b.x;
+  o.G[5] = b.y;
+  o.G[6] = b.z;
+  o.G[7] = b.w;
+  o.G[8] = c.x;
+  o.kappa = c.y;
+  return o;
+}
+
 template <int N>
 struct ForceCfg {
   static constexpr int NP = N * N * N;
@@ -78,8 +131,8 @@ struct ForceCfg {
   static constexpr int TEAMS = T / TEAM;              // teams per CTA
   static constexpr int E = TEAM / NL;                 // elements per team
   static constexpr int EPC = TEAMS * E;               // elements per CTA
-  static constexpr int RES = N == 2 ? 7 : N == 3 ? 3 : N == 6 ? 5 : N == 7 ? 4 : N == 9 ? 9 : N == 4 || N == 10 ? 1 : 0;
-  static constexpr int ES = 10 * NP + ((RES - 10 * NP) % 32 + 32) % 32;  // floats per element
+  static constexpr int WORDS = 9 * Ws<N>::PV;         // ibool words [NP]
+  static constexpr int ES = WORDS + NP + ((Ws<N>::RES - WORDS - NP) % 32 + 32) % 32;  // floats per element
   static constexpr int TS = E * ES;                   // floats per team
   static constexpr int SMEM_FLOATS = TEAMS * TS;
   static constexpr int REC = (kRecFields * NP + 3) / 4 * 4;
@@ -100,18 +153,14 @@ struct ForceCfg {
 #endif
 };
 
-// Programmatic dependent launch (the colour launches of one sweep overlap): a colour's
-// CTAs may be scheduled while the previous launch drains, prefetch their element records
-// (constant for the whole run) into L2, and wait for the previous grid to complete, with
-// its memory visible, before they read any wavefield. Both instructions are no-ops for a
-// kernel launched without the programmatic attribute.
+// With programmatic dependent launch (sem_newmark.cuh) a sweep's CTAs prefetch their element
+// records, which are constant for the whole run, into L2 while the previous kernel drains.
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void prefetch_l2_line(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
-__device__ __forceinline__ void wait_prerequisite_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
   unsigned int v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -119,7 +168,6 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
 }
 // Iterations of a bounded spin (each with a 128 ns sleep): about half a second.
 constexpr unsigned int kSweepSpinLimit = 1u << 22;
-__device__ __forceinline__ void allow_dependent_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Barrier of one team: the warp, a named barrier (1 + team) over the team's TEAM threads
 // (several warps), or the CTA.
@@ -141,7 +189,8 @@ __device__ __forceinline__ void team_sync(int team) {
 // the patch kernel, which differ only in how they gather u and assemble F.
 template <int N, int KIND, int TEAM, int ES, bool LO, class RecOf>
 __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, int team, RecOf rec_of) {
-  constexpr int NP = N * N * N, NL = N * N;
+  constexpr int NP = N * N * N, NL = N * N, PV = Ws<N>::PV;
+  using L = Ws<N>;
   const float* __restrict__ H = c_h;
   const float* __restrict__ HW = c_hw;
   const float* __restrict__ W = c_w;
@@ -156,9 +205,9 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
     const int a = line % N;
     const int b = line / N;
     const bool active = le < ne;
-    float* su = ts + (active ? le : 0) * ES;  // u, then F: [NP][3]
-    float* se = su + 3 * NP;                   // eta derivatives, then eta fluxes [NP][3]
-    float* sz = su + 6 * NP;                   // zeta derivatives, then zeta fluxes [NP][3]
+    float* su = ts + (active ? le : 0) * ES;  // u, then F
+    float* se = su + 3 * PV;                   // eta derivatives, then eta fluxes
+    float* sz = su + 6 * PV;                   // zeta derivatives, then zeta fluxes
     const float* __restrict__ r = rec_of(active ? le : 0);
 
     // 2a. eta derivatives along the eta-line (i, k) = (a, b), zeta derivatives along the
@@ -171,7 +220,7 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
       for (int l = 0; l < N; ++l)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          v[c][l] = make_float2(su[3 * (a + N * (l + N * b)) + c], su[3 * (a + N * (b + N * l)) + c]);
+          v[c][l] = make_float2(su[L::at(a, l, b) + c], su[L::at(a, b, l) + c]);
 #pragma unroll
       for (int m = 0; m < N; ++m)
 #pragma unroll
@@ -179,8 +228,8 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
           float2 d = make_float2(0.f, 0.f);
 #pragma unroll
           for (int l = 0; l < N; ++l) d = ffma2(c_h2[m * N + l], v[c][l], d);
-          se[3 * (a + N * (m + N * b)) + c] = d.x;
-          sz[3 * (a + N * (b + N * m)) + c] = d.y;
+          se[L::at(a, m, b) + c] = d.x;
+          sz[L::at(a, b, m) + c] = d.y;
         }
     }
     team_sync<KIND, TEAM>(team);
@@ -195,9 +244,9 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
       float uz[N];
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        const int p = i + N * line;
-        uxy[i] = make_float2(su[3 * p], su[3 * p + 1]);
-        uz[i] = su[3 * p + 2];
+        const int p = L::at(i, a, b);
+        uxy[i] = make_float2(su[p], su[p + 1]);
+        uz[i] = su[p + 2];
         fxy[i] = make_float2(0.f, 0.f);
         fz[i] = 0.f;
       }
@@ -211,39 +260,37 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
           dxi_z += H[i * N + l] * uz[l];
         }
         const float dxi_x = dxy.x, dxi_y = dxy.y;
-        const int p3 = 3 * (i + N * line);
+        const int p3 = L::at(i, a, b);
         const float det_x = se[p3], det_y = se[p3 + 1], det_z = se[p3 + 2];
         const float dze_x = sz[p3], dze_y = sz[p3 + 1], dze_z = sz[p3 + 2];
         const int q = i * NL + line;
-        float G[9];
-#pragma unroll
-        for (int c = 0; c < 9; ++c) G[c] = active ? __ldg(r + (kG + c) * NP + q) : 0.f;
-        const float kappa = active ? __ldg(r + kJKappa * NP + q) : 0.f;  // J kappa
-        const float mu = active ? __ldg(r + kJMu * NP + q) : 0.f;        // J mu
+        const PointRec pr = load_point<NP>(r, q, active);
+        const float(&G)[9] = pr.G;
+        const float kappa = pr.kappa, mu = pr.mu;  // J kappa, J mu
 
-        const float uxx = dxi_x * G[0] + det_x * G[3] + dze_x * G[6];
-        const float uxy = dxi_x * G[1] + det_x * G[4] + dze_x * G[7];
-        const float uxz = dxi_x * G[2] + det_x * G[5] + dze_x * G[8];
-        const float uyx = dxi_y * G[0] + det_y * G[3] + dze_y * G[6];
-        const float uyy = dxi_y * G[1] + det_y * G[4] + dze_y * G[7];
-        const float uyz = dxi_y * G[2] + det_y * G[5] + dze_y * G[8];
-        const float uzx = dxi_z * G[0] + det_z * G[3] + dze_z * G[6];
-        const float uzy = dxi_z * G[1] + det_z * G[4] + dze_z * G[7];
-        const float uzz = dxi_z * G[2] + det_z * G[5] + dze_z * G[8];
+        const float uxx = dot3(dxi_x, G[0], det_x, G[3], dze_x, G[6]);
+        const float uxy = dot3(dxi_x, G[1], det_x, G[4], dze_x, G[7]);
+        const float uxz = dot3(dxi_x, G[2], det_x, G[5], dze_x, G[8]);
+        const float uyx = dot3(dxi_y, G[0], det_y, G[3], dze_y, G[6]);
+        const float uyy = dot3(dxi_y, G[1], det_y, G[4], dze_y, G[7]);
+        const float uyz = dot3(dxi_y, G[2], det_y, G[5], dze_y, G[8]);
+        const float uzx = dot3(dxi_z, G[0], det_z, G[3], dze_z, G[6]);
+        const float uzy = dot3(dxi_z, G[1], det_z, G[4], dze_z, G[7]);
+        const float uzz = dot3(dxi_z, G[2], det_z, G[5], dze_z, G[8]);
 
         // J sigma (the record holds J kappa and J mu, so the fluxes need no J multiply)
-        const float lam = kappa - (2.f / 3.f) * mu;
+        const float lam = fmaf(-2.f / 3.f, mu, kappa);
         const float tr = uxx + uyy + uzz;
-        const float sxx = lam * tr + 2.f * mu * uxx;
-        const float syy = lam * tr + 2.f * mu * uyy;
-        const float szz = lam * tr + 2.f * mu * uzz;
+        const float sxx = fmaf(2.f * mu, uxx, lam * tr);
+        const float syy = fmaf(2.f * mu, uyy, lam * tr);
+        const float szz = fmaf(2.f * mu, uzz, lam * tr);
         const float sxy = mu * (uxy + uyx);
         const float sxz = mu * (uxz + uzx);
         const float syz = mu * (uyz + uzy);
 
-        const float txi_x = (sxx * G[0] + sxy * G[1] + sxz * G[2]);
-        const float txi_y = (sxy * G[0] + syy * G[1] + syz * G[2]);
-        const float txi_z = (sxz * G[0] + syz * G[1] + szz * G[2]);
+        const float txi_x = fmaf(sxz, G[2], fmaf(sxy, G[1], sxx * G[0]));
+        const float txi_y = dot3(sxy, G[0], syy, G[1], syz, G[2]);
+        const float txi_z = dot3(sxz, G[0], syz, G[1], szz, G[2]);
         const float2 txy = make_float2(txi_x, txi_y);
 #pragma unroll
         for (int ip = 0; ip < N; ++ip) {
@@ -251,12 +298,12 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
           fz[ip] += HW[i * N + ip] * txi_z;
         }
         if (active) {
-          se[p3] = (sxx * G[3] + sxy * G[4] + sxz * G[5]);
-          se[p3 + 1] = (sxy * G[3] + syy * G[4] + syz * G[5]);
-          se[p3 + 2] = (sxz * G[3] + syz * G[4] + szz * G[5]);
-          sz[p3] = (sxx * G[6] + sxy * G[7] + sxz * G[8]);
-          sz[p3 + 1] = (sxy * G[6] + syy * G[7] + syz * G[8]);
-          sz[p3 + 2] = (sxz * G[6] + syz * G[7] + szz * G[8]);
+          se[p3] = dot3(sxx, G[3], sxy, G[4], sxz, G[5]);
+          se[p3 + 1] = dot3(sxy, G[3], syy, G[4], syz, G[5]);
+          se[p3 + 2] = dot3(sxz, G[3], syz, G[4], szz, G[5]);
+          sz[p3] = dot3(sxx, G[6], sxy, G[7], sxz, G[8]);
+          sz[p3 + 1] = dot3(sxy, G[6], syy, G[7], syz, G[8]);
+          sz[p3 + 2] = dot3(sxz, G[6], syz, G[7], szz, G[8]);
         }
       }
     }
@@ -269,7 +316,7 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
       for (int l = 0; l < N; ++l)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-          v[c][l] = make_float2(se[3 * (a + N * (l + N * b)) + c], sz[3 * (a + N * (b + N * l)) + c]);
+          v[c][l] = make_float2(se[L::at(a, l, b) + c], sz[L::at(a, b, l) + c]);
 #pragma unroll
       for (int m = 0; m < N; ++m)
 #pragma unroll
@@ -277,8 +324,8 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
           float2 t = make_float2(0.f, 0.f);
 #pragma unroll
           for (int l = 0; l < N; ++l) t = ffma2(c_hw2[l * N + m], v[c][l], t);
-          se[3 * (a + N * (m + N * b)) + c] = t.x;
-          sz[3 * (a + N * (b + N * m)) + c] = t.y;
+          se[L::at(a, m, b) + c] = t.x;
+          sz[L::at(a, b, m) + c] = t.y;
         }
     }
     team_sync<KIND, TEAM>(team);
@@ -289,10 +336,10 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
 #pragma unroll
       for (int i = 0; i < N; ++i) {
         const float wi = W[i];
-        const int p = 3 * (i + N * line);
-        su[p] = -(wj * wk * fxy[i].x + wi * wk * se[p] + wi * wj * sz[p]);
-        su[p + 1] = -(wj * wk * fxy[i].y + wi * wk * se[p + 1] + wi * wj * sz[p + 1]);
-        su[p + 2] = -(wj * wk * fz[i] + wi * wk * se[p + 2] + wi * wj * sz[p + 2]);
+        const int p = L::at(i, a, b);
+        su[p] = -dot3(wj * wk, fxy[i].x, wi * wk, se[p], wi * wj, sz[p]);
+        su[p + 1] = -dot3(wj * wk, fxy[i].y, wi * wk, se[p + 1], wi * wj, sz[p + 1]);
+        su[p + 2] = -dot3(wj * wk, fz[i], wi * wk, se[p + 2], wi * wj, sz[p + 2]);
       }
     }
     team_sync<KIND, TEAM>(team);
@@ -304,18 +351,18 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
     const int j = line % N;
     const int k = line / N;
     const bool active = le < ne;
-    float* su = ts + (active ? le : 0) * ES;  // u, then F: [NP][3]
-    float* se = su + 3 * NP;                   // eta fluxes [NP][3]
-    float* sz = su + 6 * NP;                   // zeta fluxes [NP][3]
+    float* su = ts + (active ? le : 0) * ES;  // u, then F
+    float* se = su + 3 * PV;                   // eta fluxes
+    float* sz = su + 6 * PV;                   // zeta fluxes
     const float* __restrict__ r = rec_of(active ? le : 0);
 
     float ux[N], uy[N], uz[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const int p = i + N * line;
-      ux[i] = su[3 * p];
-      uy[i] = su[3 * p + 1];
-      uz[i] = su[3 * p + 2];
+      const int p = L::at(i, j, k);
+      ux[i] = su[p];
+      uy[i] = su[p + 1];
+      uz[i] = su[p + 2];
     }
     float hj[N], hk[N];
 #pragma unroll
@@ -338,45 +385,43 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
         dxi_x += h * ux[l];
         dxi_y += h * uy[l];
         dxi_z += h * uz[l];
-        const int pe = 3 * (i + N * (l + N * k));
+        const int pe = L::at(i, l, k);
         det_x += hj[l] * su[pe];
         det_y += hj[l] * su[pe + 1];
         det_z += hj[l] * su[pe + 2];
-        const int pz = 3 * (i + N * (j + N * l));
+        const int pz = L::at(i, j, l);
         dze_x += hk[l] * su[pz];
         dze_y += hk[l] * su[pz + 1];
         dze_z += hk[l] * su[pz + 2];
       }
       const int q = i * NL + line;
-      float G[9];
-#pragma unroll
-      for (int a = 0; a < 9; ++a) G[a] = active ? __ldg(r + (kG + a) * NP + q) : 0.f;
-      const float kappa = active ? __ldg(r + kJKappa * NP + q) : 0.f;  // J kappa
-      const float mu = active ? __ldg(r + kJMu * NP + q) : 0.f;        // J mu
+      const PointRec pr = load_point<NP>(r, q, active);
+      const float(&G)[9] = pr.G;
+      const float kappa = pr.kappa, mu = pr.mu;  // J kappa, J mu
 
-      const float uxx = dxi_x * G[0] + det_x * G[3] + dze_x * G[6];
-      const float uxy = dxi_x * G[1] + det_x * G[4] + dze_x * G[7];
-      const float uxz = dxi_x * G[2] + det_x * G[5] + dze_x * G[8];
-      const float uyx = dxi_y * G[0] + det_y * G[3] + dze_y * G[6];
-      const float uyy = dxi_y * G[1] + det_y * G[4] + dze_y * G[7];
-      const float uyz = dxi_y * G[2] + det_y * G[5] + dze_y * G[8];
-      const float uzx = dxi_z * G[0] + det_z * G[3] + dze_z * G[6];
-      const float uzy = dxi_z * G[1] + det_z * G[4] + dze_z * G[7];
-      const float uzz = dxi_z * G[2] + det_z * G[5] + dze_z * G[8];
+      const float uxx = dot3(dxi_x, G[0], det_x, G[3], dze_x, G[6]);
+      const float uxy = dot3(dxi_x, G[1], det_x, G[4], dze_x, G[7]);
+      const float uxz = dot3(dxi_x, G[2], det_x, G[5], dze_x, G[8]);
+      const float uyx = dot3(dxi_y, G[0], det_y, G[3], dze_y, G[6]);
+      const float uyy = dot3(dxi_y, G[1], det_y, G[4], dze_y, G[7]);
+      const float uyz = dot3(dxi_y, G[2], det_y, G[5], dze_y, G[8]);
+      const float uzx = dot3(dxi_z, G[0], det_z, G[3], dze_z, G[6]);
+      const float uzy = dot3(dxi_z, G[1], det_z, G[4], dze_z, G[7]);
+      const float uzz = dot3(dxi_z, G[2], det_z, G[5], dze_z, G[8]);
 
       // J sigma (the record holds J kappa and J mu, so the fluxes need no J multiply)
-      const float lam = kappa - (2.f / 3.f) * mu;
+      const float lam = fmaf(-2.f / 3.f, mu, kappa);
       const float tr = uxx + uyy + uzz;
-      const float sxx = lam * tr + 2.f * mu * uxx;
-      const float syy = lam * tr + 2.f * mu * uyy;
-      const float szz = lam * tr + 2.f * mu * uzz;
+      const float sxx = fmaf(2.f * mu, uxx, lam * tr);
+      const float syy = fmaf(2.f * mu, uyy, lam * tr);
+      const float szz = fmaf(2.f * mu, uzz, lam * tr);
       const float sxy = mu * (uxy + uyx);
       const float sxz = mu * (uxz + uzx);
       const float syz = mu * (uyz + uzy);
 
-      const float txi_x = (sxx * G[0] + sxy * G[1] + sxz * G[2]);
-      const float txi_y = (sxy * G[0] + syy * G[1] + syz * G[2]);
-      const float txi_z = (sxz * G[0] + syz * G[1] + szz * G[2]);
+      const float txi_x = fmaf(sxz, G[2], fmaf(sxy, G[1], sxx * G[0]));
+      const float txi_y = dot3(sxy, G[0], syy, G[1], syz, G[2]);
+      const float txi_z = dot3(sxz, G[0], syz, G[1], szz, G[2]);
 #pragma unroll
       for (int ip = 0; ip < N; ++ip) {
         const float hw = HW[i * N + ip];
@@ -385,13 +430,13 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
         fz[ip] += hw * txi_z;
       }
       if (active) {
-        const int p3 = 3 * (i + N * line);
-        se[p3] = (sxx * G[3] + sxy * G[4] + sxz * G[5]);
-        se[p3 + 1] = (sxy * G[3] + syy * G[4] + syz * G[5]);
-        se[p3 + 2] = (sxz * G[3] + syz * G[4] + szz * G[5]);
-        sz[p3] = (sxx * G[6] + sxy * G[7] + sxz * G[8]);
-        sz[p3 + 1] = (sxy * G[6] + syy * G[7] + syz * G[8]);
-        sz[p3 + 2] = (sxz * G[6] + syz * G[7] + szz * G[8]);
+        const int p3 = L::at(i, j, k);
+        se[p3] = dot3(sxx, G[3], sxy, G[4], sxz, G[5]);
+        se[p3 + 1] = dot3(sxy, G[3], syy, G[4], syz, G[5]);
+        se[p3 + 2] = dot3(sxz, G[3], syz, G[4], szz, G[5]);
+        sz[p3] = dot3(sxx, G[6], sxy, G[7], sxz, G[8]);
+        sz[p3 + 1] = dot3(sxy, G[6], syy, G[7], syz, G[8]);
+        sz[p3 + 2] = dot3(sxz, G[6], syz, G[7], szz, G[8]);
       }
     }
     team_sync<KIND, TEAM>(team);
@@ -410,21 +455,21 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
         float ex = 0.f, ey = 0.f, ez = 0.f, zx = 0.f, zy = 0.f, zz = 0.f;
 #pragma unroll
         for (int l = 0; l < N; ++l) {
-          const int pe = 3 * (i + N * (l + N * k));
+          const int pe = L::at(i, l, k);
           ex += hwj[l] * se[pe];
           ey += hwj[l] * se[pe + 1];
           ez += hwj[l] * se[pe + 2];
-          const int pz = 3 * (i + N * (j + N * l));
+          const int pz = L::at(i, j, l);
           zx += hwk[l] * sz[pz];
           zy += hwk[l] * sz[pz + 1];
           zz += hwk[l] * sz[pz + 2];
         }
         const float wi = W[i];
         if (active) {
-          const int p = 3 * (i + N * line);
-          su[p] = -(wj * wk * fx[i] + wi * wk * ex + wi * wj * zx);
-          su[p + 1] = -(wj * wk * fy[i] + wi * wk * ey + wi * wj * zy);
-          su[p + 2] = -(wj * wk * fz[i] + wi * wk * ez + wi * wj * zz);
+          const int p = L::at(i, j, k);
+          su[p] = -dot3(wj * wk, fx[i], wi * wk, ex, wi * wj, zx);
+          su[p + 1] = -fmaf(wi * wj, zy, fmaf(wi * wk, ey, wj * wk * fy[i]));
+          su[p + 2] = -fmaf(wi * wj, zz, fmaf(wi * wk, ez, wj * wk * fz[i]));
         }
       }
     }
@@ -435,15 +480,14 @@ __device__ __forceinline__ void team_element_forces(float* ts, int tl, int ne, i
 
 // Element kernel: one colour of elements per launch, each element gathered and scattered
 // on its own through the ibool words of its record.
-// CALLER false: u and f are the context's own padded fields [nglob][S][4] (internal node
-// order). CALLER true (one shot): caller arrays [nglob][3] in caller node order, reached
+// CALLER false: u and f are the context's own padded fields (internal node order). CALLER true (one shot): caller arrays [nglob][3] in caller node order, reached
 // through perm (internal -> caller node). With S shots the launch works on the items
 // (element, shot) of elements e0 .. e1-1 of elist, element-major: the teams of a CTA take the
 // shots of one element, so its record is read from DRAM once for all of them.
 template <int N, bool MS, bool LO, bool CALLER, bool ATOMIC = false>
 __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
     forces_kernel(const float* __restrict__ rec, const int* __restrict__ elist, const int* __restrict__ perm,
-                  const float* __restrict__ u, float* __restrict__ f, int e0, int e1, int S_arg) {
+                  const float* __restrict__ u, float* __restrict__ f, int e0, int e1, int S_arg, int nglob) {
   const int S = MS ? S_arg : 1;  // shots (a compile-time 1 for the single-shot kernel)
   using C = ForceCfg<N>;
   constexpr int NP = C::NP, E = C::E, REC = C::REC, TEAM = C::TEAM, ES = C::ES;
@@ -473,7 +517,7 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
     for (int r = 0; r < GB; ++r) {
       const int idx = base + r * TEAM;
       const int le = idx / NP;
-      w[r] = idx < ne * NP ? __float_as_uint(__ldg(rec + static_cast<size_t>(elem_of(le)) * REC + (idx - le * NP)))
+      w[r] = idx < ne * NP ? __float_as_uint(__ldg(rec + static_cast<size_t>(elem_of(le)) * REC + kIbool * NP + (idx - le * NP)))
                            : 0u;
     }
     float q[GB][3];
@@ -488,7 +532,7 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
           q[r][2] = __ldg(u + 3 * gc + 2);
         } else {
           const int le = (base + r * TEAM) / NP;
-          const float4 v = __ldg(reinterpret_cast<const float4*>(u) + g * S + shot_of(le));
+          const float4 v = __ldg(reinterpret_cast<const float4*>(u) + field_slot(nglob, S, g, shot_of(le)));
           q[r][0] = v.x;
           q[r][1] = v.y;
           q[r][2] = v.z;
@@ -502,10 +546,11 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
         const int le = idx / NP;
         const int p = idx - le * NP;
         float* eb = ts + le * ES;
-        reinterpret_cast<uint32_t*>(eb + 9 * NP)[p] = w[r];
-        eb[3 * p] = q[r][0];
-        eb[3 * p + 1] = q[r][1];
-        eb[3 * p + 2] = q[r][2];
+        reinterpret_cast<uint32_t*>(eb + C::WORDS)[p] = w[r];
+        float* pu = eb + Ws<N>::at(p);
+        pu[0] = q[r][0];
+        pu[1] = q[r][1];
+        pu[2] = q[r][2];
       }
     }
   }
@@ -521,8 +566,8 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
     for (int idx = tl; idx < ne * NP; idx += TEAM) {
       const int e = idx / NP;
       const float* sb = ts + e * ES;
-      const uint32_t w = reinterpret_cast<const uint32_t*>(sb + 9 * NP)[idx - e * NP];
-      const float* src = sb + 3 * (idx - e * NP);
+      const uint32_t w = reinterpret_cast<const uint32_t*>(sb + C::WORDS)[idx - e * NP];
+      const float* src = sb + Ws<N>::at(idx - e * NP);
       atomicAdd(reinterpret_cast<float4*>(f) + static_cast<size_t>(w & kNodeMask),
                 make_float4(src[0], src[1], src[2], 0.f));
     }
@@ -532,9 +577,9 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
     for (int idx = tl; idx < ne * NP; idx += TEAM) {
       const int e = idx / NP;
       const float* sb = ts + e * ES;
-      const uint32_t w = reinterpret_cast<const uint32_t*>(sb + 9 * NP)[idx - e * NP];
+      const uint32_t w = reinterpret_cast<const uint32_t*>(sb + C::WORDS)[idx - e * NP];
       const size_t g = static_cast<size_t>(__ldg(perm + (w & kNodeMask)));
-      const float* src = sb + 3 * (idx - e * NP);
+      const float* src = sb + Ws<N>::at(idx - e * NP);
       if (w & kFirstTouchBit) {
         f[3 * g] = src[0];
         f[3 * g + 1] = src[1];
@@ -557,9 +602,9 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
       prev[r] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (idx < ne * NP) {
         const int e = idx / NP;
-        w[r] = reinterpret_cast<const uint32_t*>(ts + e * ES + 9 * NP)[idx - e * NP];
+        w[r] = reinterpret_cast<const uint32_t*>(ts + e * ES + C::WORDS)[idx - e * NP];
         if (!(w[r] & kFirstTouchBit))
-          prev[r] = reinterpret_cast<const float4*>(f)[static_cast<size_t>(w[r] & kNodeMask) * S + shot_of(e)];
+          prev[r] = reinterpret_cast<const float4*>(f)[field_slot(nglob, S, w[r] & kNodeMask, shot_of(e))];
       }
     }
 #pragma unroll
@@ -567,8 +612,8 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
       const int idx = base + r * TEAM;
       if (idx < ne * NP) {
         const int e = idx / NP;
-        const float* src = ts + e * ES + 3 * (idx - e * NP);
-        reinterpret_cast<float4*>(f)[static_cast<size_t>(w[r] & kNodeMask) * S + shot_of(e)] =
+        const float* src = ts + e * ES + Ws<N>::at(idx - e * NP);
+        reinterpret_cast<float4*>(f)[field_slot(nglob, S, w[r] & kNodeMask, shot_of(e))] =
             make_float4(src[0] + prev[r].x, src[1] + prev[r].y, src[2] + prev[r].z, 0.f);
       }
     }
@@ -618,66 +663,59 @@ struct PatchCfg {
   static constexpr int PE = BX * BY * BZ;
   static constexpr int TEAMS = (PE + E - 1) / E;
   static constexpr int T = TEAMS * TEAM;
-  // floats per element workspace (at least 10 NP: u/F, eta and zeta values, ibool words)
-  static constexpr int ES = KIND == ForceCfg<N>::KIND ? ForceCfg<N>::ES : 10 * NP + 1;
+  // floats per element workspace and per team; the persistent sweeps keep the ibool words too
+  static constexpr int ES = 9 * Ws<N>::PV + ((Ws<N>::RES - 9 * Ws<N>::PV) % 32 + 32) % 32;
   static constexpr int TS = E * ES;
+  static constexpr int WORDS = ForceCfg<N>::WORDS;
+  static constexpr int ESW = ForceCfg<N>::ES;
+  static constexpr int TSW = E * ESW;
+  static constexpr int SMEMW = TEAMS * TSW * 4;
   static constexpr int REC = ForceCfg<N>::REC;
   static constexpr int SMEM = TEAMS * TS * 4;
   static constexpr int MIN_BLOCKS = N == 3 ? 3 : N <= 5 ? 4 : N <= 7 ? 3 : 2;
-  static_assert(E >= 1 && 10 * NP <= ES, "team and workspace sizes");
+  static_assert(E >= 1 && TEAM >= E * NL, "team size");
 };
 
-// Index of a node's 16-byte slot in a [nglob][S][4] field (S = 1 for a single shot).
-template <bool MS>
-__device__ __forceinline__ size_t node_slot(uint32_t w, int S, int shot) {
-  if constexpr (MS)
-    return static_cast<size_t>(w & kNodeMask) * S + shot;
-  else
-    return static_cast<size_t>(w & kNodeMask);
-}
-
 // Phases 1-3 of one patch for the calling thread's team: gather through the records' ibool
-// words (GB points per thread in flight; the shared-memory copy of each word keeps the node,
-// the patch first-touch flag and kAloneBit), then the element forces.
-// (NM 1: the half-step velocity and 1/M of the nodes the patch touches last are prefetched
-// into L2 as their points are gathered, for the Newmark update at the end of the patch; NM 2:
-// the older adjoint field and 1/M, for the adjoint leapfrog.)
-template <int N, bool LO, bool MS = false, int NM = 0>
+// words (GB points per thread in flight), then the element forces. KEEP: the words also go to
+// shared memory (element stride ESW; the persistent sweeps write nodes through them). CALLER: u
+// is a caller array [nglob][3], reached through perm (one more dependent load; a separate pass
+// into the solver's layout first measured 40 us on 44 x 36 x 40 elements at NGLL 5, the longer
+// gather a sweep of 209 against 241 us, passes included).
+template <int N, bool LO, bool MS = false, bool KEEP = false, bool CALLER = false>
 __device__ __forceinline__ void patch_gather_compute(const PatchDesc& d, const float* __restrict__ rec,
-                                                     const float4* __restrict__ u, float* wsb, bool u_from_l2,
-                                                     int S = 1, int shot = 0, const SweepNewmark* nm = nullptr) {
+                                                     const float4* u, float* wsb,
+                                                     const int* __restrict__ perm = nullptr) {
   using C = PatchCfg<N>;
-  constexpr int NP = C::NP, E = C::E, TEAM = C::TEAM, ES = C::ES, REC = C::REC;
+  constexpr int NP = C::NP, E = C::E, TEAM = C::TEAM, REC = C::REC;
+  constexpr int ES = KEEP ? C::ESW : C::ES;
   const int team = threadIdx.x / TEAM;
   const int tl = threadIdx.x - team * TEAM;
   const int ne = min(E, d.nelem - team * E);  // this team's elements
   const float* __restrict__ trec = rec + static_cast<size_t>(d.slot0 + team * E) * REC;
   constexpr int GB = 4;
-  float* ts = wsb + team * C::TS;
+  float* ts = wsb + team * (E * ES);
   for (int base = tl; base < ne * NP; base += GB * TEAM) {
     uint32_t w[GB];
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
       const int idx = base + r * TEAM;
       const int le = idx / NP;
-      w[r] = idx < ne * NP ? __float_as_uint(__ldg(trec + static_cast<size_t>(le) * REC + (idx - le * NP))) : 0u;
-    }
-    if constexpr (NM != 0) {
-#pragma unroll
-      for (int r = 0; r < GB; ++r)
-        if (w[r] & kPatchLastBit) {
-          prefetch_l2_line(reinterpret_cast<const float4*>(NM == 2 ? nm->lam_old : nm->v) +
-                           node_slot<MS>(w[r], S, shot));
-          prefetch_l2_line(nm->minv + (w[r] & kNodeMask));
-        }
+      w[r] = idx < ne * NP ? __float_as_uint(__ldg(trec + static_cast<size_t>(le) * REC + kIbool * NP + (idx - le * NP)))
+                           : 0u;
     }
     float4 q[GB];
-    if (u_from_l2) {
+    if constexpr (CALLER) {
 #pragma unroll
-      for (int r = 0; r < GB; ++r) q[r] = __ldcg(u + node_slot<MS>(w[r], S, shot));
+      for (int r = 0; r < GB; ++r) w[r] = __ldg(perm + (w[r] & kNodeMask));
+#pragma unroll
+      for (int r = 0; r < GB; ++r) {
+        const float* pu = reinterpret_cast<const float*>(u) + 3 * static_cast<size_t>(w[r]);
+        q[r] = make_float4(__ldg(pu), __ldg(pu + 1), __ldg(pu + 2), 0.f);
+      }
     } else {
 #pragma unroll
-      for (int r = 0; r < GB; ++r) q[r] = __ldg(u + node_slot<MS>(w[r], S, shot));
+      for (int r = 0; r < GB; ++r) q[r] = __ldcg(u + node_slot<MS>(w[r]));
     }
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
@@ -686,10 +724,11 @@ __device__ __forceinline__ void patch_gather_compute(const PatchDesc& d, const f
         const int le = idx / NP;
         const int p = idx - le * NP;
         float* eb = ts + le * ES;
-        reinterpret_cast<uint32_t*>(eb + 9 * NP)[p] = w[r];
-        eb[3 * p] = q[r].x;
-        eb[3 * p + 1] = q[r].y;
-        eb[3 * p + 2] = q[r].z;
+        if constexpr (KEEP) reinterpret_cast<uint32_t*>(eb + C::WORDS)[p] = w[r];
+        float* pu = eb + Ws<N>::at(p);
+        pu[0] = q[r].x;
+        pu[1] = q[r].y;
+        pu[2] = q[r].z;
       }
     }
   }
@@ -700,130 +739,19 @@ __device__ __forceinline__ void patch_gather_compute(const PatchDesc& d, const f
   }
 }
 
-// Previous value of a node of f: through L1 (COHERENT false: f was last written by an
-// earlier grid) or from L2 (COHERENT true: other CTAs of this grid wrote it).
-template <bool COHERENT>
-__device__ __forceinline__ float4 load_f(const float4* p) {
-  if constexpr (COHERENT)
-    return __ldcg(p);
-  else
-    return *p;
-}
-
-// Point sources of the step at a node the patch touches last (Sec. V-C): the Ricker wavelet
-// at t_{n+1} = step dt (the counter, advanced before the sweep, read from L2) times each
-// force, added to the node's complete force in the order the entries are listed.
-__device__ __forceinline__ void add_point_sources(const PatchDesc& d, const SweepNewmark& nm, uint32_t node, int shot,
-                                                  float& fx, float& fy, float& fz) {
-  for (int i = 0; i < d.nsrc; ++i) {
-    const PatchSrc& s = nm.src[d.src_off + i];
-    if (s.node != static_cast<int>(node) || s.shot != shot) continue;
-    const long long n = __ldcg(nm.step);
-    const double tau = static_cast<double>(n) * nm.dtd - nm.t0;
-    const double x = M_PI * nm.f0 * tau;
-    const double aa = x * x;
-    const double R = (1.0 - 2.0 * aa) * exp(-aa);
-    fx += static_cast<float>(s.f[0] * R);
-    fy += static_cast<float>(s.f[1] * R);
-    fz += static_cast<float>(s.f[2] * R);
-  }
-}
-
-// The inputs of a node's Newmark update, loaded with the previous force values so that all
-// of a thread's loads are in flight together: 1/M, the half-step velocity and (mode 1) the
-// displacement.
-struct NodeState {
-  float m;
-  float4 v, u;
-};
-template <bool MS, bool WITH_U = false>
-__device__ __forceinline__ void load_node_state(const SweepNewmark& nm, uint32_t w, int S, int shot, NodeState& st) {
-  const size_t g = node_slot<MS>(w, S, shot);
-  st.m = __ldg(nm.minv + (w & kNodeMask));
-  st.v = __ldcg(reinterpret_cast<const float4*>(nm.v) + g);
-  if (WITH_U || nm.mode == 1) st.u = __ldcg(reinterpret_cast<const float4*>(nm.u) + g);
-}
-
-// Newmark update of a node whose complete force (fx, fy, fz) is known (mode 1 or 2):
-//   a = M^-1 f ; v = v_half + dt/2 a ; mode 1: u <- u + dt v + dt^2/2 a, v_half <- v + dt/2 a ;
-//   mode 2: v and a stored.
-template <bool MS>
-__device__ __forceinline__ void newmark_node(const SweepNewmark& nm, uint32_t w, int S, int shot, const NodeState& st,
-                                             float fx, float fy, float fz) {
-  const size_t g = node_slot<MS>(w, S, shot);
-  const float ax = fx * st.m, ay = fy * st.m, az = fz * st.m;
-  const float vx = st.v.x + nm.hdt * ax, vy = st.v.y + nm.hdt * ay, vz = st.v.z + nm.hdt * az;
-  if (nm.mode == 1) {
-    reinterpret_cast<float4*>(nm.u)[g] = make_float4((st.u.x + nm.dt * vx) + nm.hdt2 * ax,
-                                                     (st.u.y + nm.dt * vy) + nm.hdt2 * ay,
-                                                     (st.u.z + nm.dt * vz) + nm.hdt2 * az, 0.f);
-    reinterpret_cast<float4*>(nm.v)[g] = make_float4(vx + nm.hdt * ax, vy + nm.hdt * ay, vz + nm.hdt * az, 0.f);
-  } else {
-    reinterpret_cast<float4*>(nm.v)[g] = make_float4(vx, vy, vz, 0.f);
-    reinterpret_cast<float4*>(nm.a)[g] = make_float4(ax, ay, az, 0.f);
-  }
-}
-
-// The snapshot of the node's displacement u^{n+1} (NM 3: a Newmark sweep of a snapshot run).
-__device__ __forceinline__ void snapshot_node(const SweepNewmark& nm, uint32_t w, const NodeState& st) {
-  const DevCtl* ctl = nm.snap_ctl;
-  const uint32_t g = w & kNodeMask;
-  float* o = ctl->snap + static_cast<long long>(ctl->col - 1) * ctl->snap_per +
-             3 * static_cast<size_t>(nm.snap_perm ? __ldg(nm.snap_perm + g) : static_cast<int>(g));
-  o[0] = st.u.x;
-  o[1] = st.u.y;
-  o[2] = st.u.z;
-}
-
-// The adjoint step at a node whose force f = -K lam is complete (NM 2): the receiver
-// residuals of the step at this node added to f in ascending receiver order (G / dt^2), then
-// the leapfrog lam_old <- 2 lam - lam_old + dt^2 M^-1 f (the same float operations as the
-// separate injection and leapfrog passes).
-__device__ __forceinline__ void adjoint_receivers(const SweepNewmark& nm, int2 rr, uint32_t node, float& fx, float& fy,
-                                                  float& fz) {
-  const float* G = nm.idx ? nm.idx->adj_G + static_cast<long long>(nm.idx->adj_j - 1) * nm.idx->adj_gstep : nm.G;
-  if (!G) return;
-  for (int i = rr.x; i < rr.x + rr.y; ++i) {
-    const PatchRecv e = nm.recv[i];
-    if (e.node != static_cast<int>(node)) continue;
-    fx += G[3 * e.r] * nm.inv_dt2;
-    fy += G[3 * e.r + 1] * nm.inv_dt2;
-    fz += G[3 * e.r + 2] * nm.inv_dt2;
-  }
-}
-__device__ __forceinline__ void load_adjoint_state(const SweepNewmark& nm, uint32_t w, NodeState& st) {
-  const size_t g = w & kNodeMask;
-  st.m = __ldg(nm.minv + g);
-  st.u = __ldcg(reinterpret_cast<const float4*>(nm.u) + g);        // lam^m
-  st.v = __ldcg(reinterpret_cast<const float4*>(nm.lam_old) + g);  // lam^{m+1}
-}
-__device__ __forceinline__ void adjoint_node(const SweepNewmark& nm, uint32_t w, const NodeState& st, float fx,
-                                             float fy, float fz) {
-  const size_t g = w & kNodeMask;
-  const float s = nm.dt2 * st.m;
-  const float4 l = st.u, o = st.v;
-  reinterpret_cast<float4*>(nm.lam_old)[g] =
-      make_float4(2.f * l.x - o.x + s * fx, 2.f * l.y - o.y + s * fy, 2.f * l.z - o.z + s * fz, 0.f);
-}
-
-// Phase 4a for the calling thread's team: the forces of its points that are alone at their
-// patch node added to the node (stored at its first touch; with a Newmark mode, used for the
-// node's update at its last touch and not stored).
-template <int N, bool COHERENT, bool MS = false, int NM = 0>
-__device__ __forceinline__ void patch_write_alone(const PatchDesc& d, float4* __restrict__ f, const float* wsb,
-                                                  const SweepNewmark& nm, int S = 1, int shot = 0,
-                                                  int2 rr = make_int2(0, 0)) {
+// Persistent sweeps (forces only), phase 4a for the calling thread's team: the forces of its
+// points that are alone at their patch node added to the node (stored at its first touch).
+template <int N>
+__device__ __forceinline__ void patch_write_alone(const PatchDesc& d, float4* __restrict__ f, const float* wsb) {
   using C = PatchCfg<N>;
-  constexpr int NP = C::NP, E = C::E, TEAM = C::TEAM, ES = C::ES, GB = NM ? 2 : 4;
+  constexpr int NP = C::NP, E = C::E, TEAM = C::TEAM, ES = C::ESW, GB = 4;
   const int team = threadIdx.x / TEAM;
   const int tl = threadIdx.x - team * TEAM;
   const int ne = min(E, d.nelem - team * E);
-  const float* ts = wsb + team * C::TS;
-  constexpr uint32_t last_bit = NM ? kPatchLastBit : 0u;
+  const float* ts = wsb + team * C::TSW;
   for (int base = tl; base < ne * NP; base += GB * TEAM) {
     uint32_t w[GB];
     float4 prev[GB];
-    NodeState st[GB];
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
       const int idx = base + r * TEAM;
@@ -831,14 +759,8 @@ __device__ __forceinline__ void patch_write_alone(const PatchDesc& d, float4* __
       prev[r] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (idx < ne * NP) {
         const int e = idx / NP;
-        w[r] = reinterpret_cast<const uint32_t*>(ts + e * ES + 9 * NP)[idx - e * NP];
-        if ((w[r] & kAloneBit) && !(w[r] & kPatchFirstBit)) prev[r] = load_f<COHERENT>(f + node_slot<MS>(w[r], S, shot));
-        if ((w[r] & kAloneBit) && (w[r] & last_bit)) {
-          if constexpr (NM == 2)
-            load_adjoint_state(nm, w[r], st[r]);
-          else
-            load_node_state<MS, NM == 3>(nm, w[r], S, shot, st[r]);
-        }
+        w[r] = reinterpret_cast<const uint32_t*>(ts + e * ES + C::WORDS)[idx - e * NP];
+        if ((w[r] & kAloneBit) && !(w[r] & kPatchFirstBit)) prev[r] = __ldcg(f + (w[r] & kNodeMask));
       }
     }
 #pragma unroll
@@ -846,44 +768,56 @@ __device__ __forceinline__ void patch_write_alone(const PatchDesc& d, float4* __
       const int idx = base + r * TEAM;
       if (w[r] & kAloneBit) {
         const int e = idx / NP;
-        const float* src = ts + e * ES + 3 * (idx - e * NP);
-        float fx = src[0] + prev[r].x, fy = src[1] + prev[r].y, fz = src[2] + prev[r].z;
-        if (w[r] & last_bit) {
-          if constexpr (NM == 2) {
-            if (rr.y) adjoint_receivers(nm, rr, w[r] & kNodeMask, fx, fy, fz);
-            adjoint_node(nm, w[r], st[r], fx, fy, fz);
-          } else {
-            if constexpr (NM == 3) snapshot_node(nm, w[r], st[r]);
-            if (d.nsrc) add_point_sources(d, nm, w[r] & kNodeMask, shot, fx, fy, fz);
-            newmark_node<MS>(nm, w[r], S, shot, st[r], fx, fy, fz);
-          }
-        } else {
-          f[node_slot<MS>(w[r], S, shot)] = make_float4(fx, fy, fz, 0.f);
-        }
+        const float* src = ts + e * ES + Ws<N>::at(idx - e * NP);
+        f[w[r] & kNodeMask] = make_float4(src[0] + prev[r].x, src[1] + prev[r].y, src[2] + prev[r].z, 0.f);
       }
     }
   }
 }
 
-// Phase 4b over the CTA: per shared patch node, the sum of its local points' forces in table
-// order (its slots, shared-memory offsets of those forces, read as one 16-byte word), then
-// one store (first touch) or one read-modify-write, or at the node's last touch (with a
-// Newmark mode) its update; the previous values of GB nodes are loaded before any is written.
-template <int N, bool COHERENT, bool MS = false, int NM = 0>
+// The forces of the local points that meet at a patch node, in table order: the slot group g4
+// (shared-memory offsets, filled from the first, read as one 16-byte word) and the groups
+// chained to it from the last slot. Most nodes have one, two or four points, so a warp leaves
+// after the half-words that hold any.
+template <class Add>
+__device__ __forceinline__ void sum_slots(uint4 g4, const uint4* __restrict__ slots, Add add) {
+  while (true) {
+    add(g4.x & 0xFFFFu);
+    if ((g4.x >> 16) == kPatchNoSlot) return;
+    add(g4.x >> 16);
+    if (g4.y == 0xFFFFFFFFu) return;
+    add(g4.y & 0xFFFFu);
+    if ((g4.y >> 16) != kPatchNoSlot) add(g4.y >> 16);
+    if (g4.z == 0xFFFFFFFFu) return;
+    add(g4.z & 0xFFFFu);
+    if ((g4.z >> 16) != kPatchNoSlot) add(g4.z >> 16);
+    if (g4.w == 0xFFFFFFFFu) return;
+    add(g4.w & 0xFFFFu);
+    const uint32_t last = g4.w >> 16;
+    if (last == kPatchNoSlot) return;
+    if (!(last & kPatchChain)) {
+      add(last);
+      return;
+    }
+    g4 = __ldg(slots + (last & ~static_cast<uint32_t>(kPatchChain)));
+  }
+}
+
+// Persistent sweeps, phase 4b over the CTA: per shared patch node, the sum of its local points'
+// forces, then one store (first touch) or one read-modify-write; the previous values of GB
+// nodes are loaded before any is written.
+template <int N>
 __device__ __forceinline__ void patch_write_shared(const PatchDesc& d, const uint16_t* __restrict__ slot_tab,
                                                    const uint16_t* __restrict__ word_tab, float4* __restrict__ f,
-                                                   const float* wsb, const SweepNewmark& nm, int S = 1,
-                                                   int shot = 0, int2 rr = make_int2(0, 0)) {
+                                                   const float* wsb) {
   using C = PatchCfg<N>;
-  constexpr int T = C::T, GB = NM ? 2 : 4;
+  constexpr int T = C::T, GB = 4;
   const uint4* __restrict__ slots = reinterpret_cast<const uint4*>(slot_tab + d.slot_off);
   const uint16_t* __restrict__ words = word_tab + d.word_off;
-  constexpr uint32_t last_bit = NM ? kPatchLastBit : 0u;
   for (int base = threadIdx.x; base < d.nshared; base += GB * T) {
     uint4 sl[GB];
     uint32_t w[GB];
     float4 prev[GB];
-    NodeState st[GB];
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
       const int t = base + r * T;
@@ -894,98 +828,156 @@ __device__ __forceinline__ void patch_write_shared(const PatchDesc& d, const uin
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
       prev[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!(w[r] & kPatchFirstBit)) prev[r] = load_f<COHERENT>(f + node_slot<MS>(w[r], S, shot));
-      if (w[r] & last_bit) {
-        if constexpr (NM == 2)
-          load_adjoint_state(nm, w[r], st[r]);
-        else
-          load_node_state<MS, NM == 3>(nm, w[r], S, shot, st[r]);
-      }
+      if (!(w[r] & kPatchFirstBit)) prev[r] = __ldcg(f + (w[r] & kNodeMask));
     }
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
-      const int t = base + r * T;
-      if (t < d.nshared) {
-        float sx = 0.f, sy = 0.f, sz = 0.f;
-        uint4 g4 = sl[r];
-        while (true) {
-          const uint32_t wd[4] = {g4.x, g4.y, g4.z, g4.w};
-          uint32_t chain = 0;
-#pragma unroll
-          for (int k = 0; k < kPatchSlots; ++k) {
-            const uint32_t q = (wd[k >> 1] >> (16 * (k & 1))) & 0xFFFFu;
-            if (q == kPatchNoSlot) continue;
-            if (q & kPatchChain) {
-              chain = q;
-              continue;
-            }
-            const float* F = wsb + q;
-            sx += F[0];
-            sy += F[1];
-            sz += F[2];
-          }
-          if (!chain) break;
-          g4 = __ldg(slots + (chain & ~static_cast<uint32_t>(kPatchChain)));
-        }
-        float fx = prev[r].x + sx, fy = prev[r].y + sy, fz = prev[r].z + sz;
-        if (w[r] & last_bit) {
-          if constexpr (NM == 2) {
-            if (rr.y) adjoint_receivers(nm, rr, w[r] & kNodeMask, fx, fy, fz);
-            adjoint_node(nm, w[r], st[r], fx, fy, fz);
-          } else {
-            if constexpr (NM == 3) snapshot_node(nm, w[r], st[r]);
-            if (d.nsrc) add_point_sources(d, nm, w[r] & kNodeMask, shot, fx, fy, fz);
-            newmark_node<MS>(nm, w[r], S, shot, st[r], fx, fy, fz);
-          }
-        } else {
-          f[node_slot<MS>(w[r], S, shot)] = make_float4(fx, fy, fz, 0.f);
-        }
-      }
+      if (base + r * T >= d.nshared) continue;
+      float sx = 0.f, sy = 0.f, sz = 0.f;
+      sum_slots(sl[r], slots, [&](uint32_t q) {
+        sx += wsb[q];
+        sy += wsb[q + 1];
+        sz += wsb[q + 2];
+      });
+      f[w[r] & kNodeMask] = make_float4(prev[r].x + sx, prev[r].y + sy, prev[r].z + sz, 0.f);
     }
   }
 }
 
-// One launch per patch colour: one CTA per patch of the colour [p0, p0 + gridDim.x).
-// The launches of one sweep are programmatic dependent launches: a colour's CTAs may start
-// while the previous colour drains. The first colour of a sweep (p0 == 0) waits for the
-// previous grid before anything (that grid may have written u). A later colour reads only u
-// (which no colour writes, and which was complete before the first colour began; read from
-// L2) and the records until it writes f, so it gathers and evaluates its elements first and
-// waits for the previous colour only before its writes.
-// With S shots (MS true) the fields are [nglob][S][4] and CTA b takes patch p0 + b / S for
-// shot b % S: consecutive CTAs take the shots of one patch, so its records come from DRAM
-// once (the first shot's prefetch) and from L2 for the others.
+// The receivers of a patch sample u^{n+1} (modes 1 and 2) for shots s0 .. s0 + ns - 1 before any
+// of its nodes is updated (the barrier; nodes of other patches' rims change only in the rim
+// pass). All threads of the CTA.
+__device__ __forceinline__ void record_receivers(const PatchDesc& d, const SweepNewmark& nm, const float4* u, int shots,
+                                                 int s0, int ns) {
+  if (d.nrec == 0) return;
+  const DevCtl* ctl = nm.ctl;
+  float* seis = ctl->seis;
+  const int col = ctl->col + nm.ahead, ncols = ctl->ncols;
+  if (seis != nullptr && col < ncols) {  // seis [shots][nrec][3][ncols]
+    for (int q = threadIdx.x; q < d.nrec * ns; q += blockDim.x) {
+      const int i = q / ns, sh = s0 + q - i * ns;
+      const PatchRecv e = nm.recv[d.rec_off + i];
+      const float4 x = __ldcg(u + field_slot(nm.nglob, shots, e.node, sh));
+      float* o = seis + (static_cast<size_t>(sh) * nm.nrec + e.r) * 3 * ncols + col;
+      o[0] = x.x;
+      o[ncols] = x.y;
+      o[2 * static_cast<size_t>(ncols)] = x.z;
+    }
+  }
+  __syncthreads();
+}
+
+// The state and 1/M of a patch's inner nodes, which are consecutive, to L2 (whole 16-byte
+// blocks around 1/M) for their update at the end of the patch: slots a node, from nm.v on. One
+// thread.
+template <int NM>
+__device__ __forceinline__ void prefetch_inner(const PatchDesc& d, const SweepNewmark& nm, int slots) {
+  const int n = d.nalone + d.nin;
+  if (n == 0) return;
+  const float* v = NM == 2 ? nm.lam_old : nm.v;
+  prefetch_l2(v + 4 * slots * static_cast<size_t>(d.inner0), 16u * slots * n);
+  const int m0 = d.inner0 & ~3;
+  const int nm4 = (d.inner0 + n - m0) & ~3;
+  if (nm4 > 0) prefetch_l2(nm.minv + m0, 4u * nm4);
+}
+
+// Phase 4 over the CTA, once every team's forces are in shared memory. Per rim node the sum of
+// the patch's forces there goes into its partial. Then the inner nodes are completed: their ids
+// are consecutive, so the state streams, and it is loaded (st, the first round) before the
+// barrier that precedes this.
+template <int N, bool MS, int NM>
+struct PatchFinish {
+  using C = PatchCfg<N>;
+  static constexpr int T = C::T;
+  static constexpr bool STATE = NM != 0 && NM != 4;
+  NodeState st;
+  __device__ __forceinline__ void load(const PatchDesc& d, const SweepNewmark& nm, int t) {
+    if constexpr (STATE)
+      if (t < d.nalone + d.nin) load_node_state<MS, NM>(nm, d.inner0 + t, st);
+  }
+  __device__ __forceinline__ void run(const PatchDesc& d, const uint16_t* __restrict__ slot_tab,
+                                      const uint16_t* __restrict__ word_tab, float4* __restrict__ f,
+                                      float4* __restrict__ partials, const float* wsb, const SweepNewmark& nm,
+                                      int shot) {
+    auto sum_at = [&](uint4 g4, const uint4* __restrict__ slots) {
+      float sx = 0.f, sy = 0.f, sz = 0.f;
+      sum_slots(g4, slots, [&](uint32_t q) {
+        sx += wsb[q];
+        sy += wsb[q + 1];
+        sz += wsb[q + 2];
+      });
+      return make_float4(sx, sy, sz, 0.f);
+    };
+    const uint4* __restrict__ groups = reinterpret_cast<const uint4*>(slot_tab);
+    const uint4* __restrict__ rim = groups + d.rim_slots;
+    for (int t = threadIdx.x; t < d.nrim; t += T)
+      partials[(static_cast<size_t>(d.rim0) + t) * (MS ? 2 : 1)] = sum_at(__ldg(rim + t), rim);
+    const uint16_t* __restrict__ alone = word_tab + d.alone_off;
+    const uint4* __restrict__ in = groups + d.in_slots;
+    for (int t = threadIdx.x; t < d.nalone + d.nin; t += T) {
+      if (t >= T) load(d, nm, t);
+      float4 s;
+      if (t < d.nalone) {
+        const float* F = wsb + __ldg(alone + t);
+        s = make_float4(F[0], F[1], F[2], 0.f);
+      } else {
+        s = sum_at(__ldg(in + (t - d.nalone)), in);
+      }
+      complete_node<MS, NM>(nm, f, d.inner0 + t, shot, st, nm.src + d.src_off, d.nsrc, nm.recv + d.rec_off,
+                            d.nrec_in, s.x, s.y, s.z);
+    }
+  }
+};
+
+// The sweep: one launch over every patch, one CTA per patch. A CTA completes its inner nodes
+// and leaves its share of each rim node in the partials buffer; the rim pass adds the shares of
+// a node in sweep order. No patch waits for another, no node is read back, and the order of
+// every sum is fixed (that of a colour-by-colour assembly of the same patches: the results are
+// the same bit for bit).
+// What bounds it (ncu, NGLL 5, 48^3): the L1 data pipe, 81 % busy (576 wavefronts an element:
+// 379 of shared memory, 197 of global loads), DRAM 59 %, issue slots 56 %; 250 us. With one
+// launch per patch colour (eight, each waiting for the one before) a step of that mesh took 329
+// us against 308, of 8^3 elements 50 us against 17, of 25 x 21 x 23 at NGLL 7 128 against 116.
+// With S shots (MS true) CTA b takes patch b / S for shot b % S: consecutive CTAs take the shots of one patch, so its records come from DRAM once
+// (the first shot's prefetch) and from L2 for the others.
 template <int N, bool LO, bool MS, int NM>
 __global__ void __launch_bounds__(PatchCfg<N>::T, PatchCfg<N>::MIN_BLOCKS)
     patch_forces_kernel(const float* __restrict__ rec, const PatchDesc* __restrict__ desc,
                         const uint16_t* __restrict__ slot_tab, const uint16_t* __restrict__ word_tab,
-                        const float4* __restrict__ u, float4* __restrict__ f, int p0, int S_arg,
-                        const SweepNewmark nm) {
+                        const float4* __restrict__ u, float4* __restrict__ f, float4* __restrict__ partials,
+                        int S_arg, const SweepNewmark nm_arg) {
   using C = PatchCfg<N>;
+  SweepNewmark nm = nm_arg;
   extern __shared__ float4 smem4[];
   float* wsb = reinterpret_cast<float*>(smem4);
   const int S = MS ? S_arg : 1;
-  const int P = p0 + (MS ? static_cast<int>(blockIdx.x) / S : static_cast<int>(blockIdx.x));
-  const int shot = MS ? static_cast<int>(blockIdx.x) - (P - p0) * S : 0;
+  const int P = MS ? static_cast<int>(blockIdx.x) / S : static_cast<int>(blockIdx.x);
+  const int shot = MS ? static_cast<int>(blockIdx.x) - P * S : 0;
   const PatchDesc d = desc[P];
-  // 0. records to L2 (by the patch's first shot)
+  // 0. records to L2 (by the patch's first shot) while the previous kernel drains
   if (shot == 0 && threadIdx.x < d.nelem)
     prefetch_l2(rec + static_cast<size_t>(d.slot0 + threadIdx.x) * C::REC, kForceFields * C::NP * sizeof(float));
-  if (p0 == 0) wait_prerequisite_grid();
+  wait_prerequisite_grid();
   allow_dependent_grid();
-  // before the wait, u comes from L2 (the coherence point), never from a line this SM's L1
-  // may hold from before the grid that wrote u
-  patch_gather_compute<N, LO, MS, NM>(d, rec, u, wsb, p0 != 0, S, shot, &nm);
-  if (p0 != 0) wait_prerequisite_grid();  // the previous colour's writes to f
-  const int2 rr = NM == 2 && nm.recv_range ? make_int2(nm.recv_range[2 * P], nm.recv_range[2 * P + 1]) : make_int2(0, 0);
-  patch_write_alone<N, false, MS, NM>(d, f, wsb, nm, S, shot, rr);  // no wait for the other teams
+  if constexpr (NM == 1 || NM == 3) record_receivers(d, nm, u, S, shot, 1);
+  if constexpr (MS) {  // to the shot's slots
+    const size_t slot = field_slot(nm.nglob, 2, 0, shot);
+    move_fields(nm, slot);
+    u += slot;
+    f += slot;
+    partials += field_slot(nm.nsums, 2, 0, shot);
+  }
+  if constexpr (NM != 0 && NM != 4)
+    if (threadIdx.x == 0) prefetch_inner<NM>(d, nm, MS ? 2 : 1);
+  patch_gather_compute<N, LO, MS, false, NM == 4>(d, rec, u, wsb, NM == 4 ? nm.perm : nullptr);
+  PatchFinish<N, MS, NM> fin;
+  fin.load(d, nm, threadIdx.x);
   __syncthreads();
-  patch_write_shared<N, false, MS, NM>(d, slot_tab, word_tab, f, wsb, nm, S, shot, rr);
+  fin.run(d, slot_tab, word_tab, f, partials, wsb, nm, shot);
 }
 
 // ---------------------------------------------------------------------------------------
-// Shot pairs. With several shots of one model (fields [nglob][S][4]), a CTA takes one patch
-// for two shots: every thread carries both shots' values as float32 pairs (shot 2k in .x,
+// Shot pairs. With several shots of one model, a CTA takes one patch for two shots: every thread carries both shots' values as float32 pairs (shot 2k in .x,
 // 2k + 1 in .y), so one packed fma serves both shots, and every geometry and modulus value
 // read from the records serves both. The workspace is the single-shot layout with every
 // float widened to a pair (an element at twice its single-shot offset; u/F, eta and zeta
@@ -1015,16 +1007,17 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
 // Phases 2-3 of one team's elements for a shot pair (ES2 floats per element workspace).
 template <int N, int KIND, int TEAM, int ES2, class RecOf>
 __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int ne, int team, RecOf rec_of) {
-  constexpr int NP = N * N * N, NL = N * N;
+  constexpr int NP = N * N * N, NL = N * N, PV = Ws<N>::PV;
+  using L = Ws<N>;
   const float* __restrict__ W = c_w;
   const int le = tl / NL;
   const int line = tl - le * NL;
   const int a = line % N;
   const int b = line / N;
   const bool active = le < ne;
-  float2* su = reinterpret_cast<float2*>(ts2 + (active ? le : 0) * ES2);  // u, then F: [NP][3]
-  float2* se = su + 3 * NP;                                                 // eta values [NP][3]
-  float2* sz = su + 6 * NP;                                                 // zeta values [NP][3]
+  float2* su = reinterpret_cast<float2*>(ts2 + (active ? le : 0) * ES2);  // u, then F
+  float2* se = su + 3 * PV;                                                 // eta values
+  float2* sz = su + 6 * PV;                                                 // zeta values
   const float* __restrict__ r = rec_of(active ? le : 0);
 
   // 2a. eta derivatives along the eta-line (i, k) = (a, b), zeta derivatives along the
@@ -1035,8 +1028,8 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
       float2 ve[N], vz[N];
 #pragma unroll
       for (int l = 0; l < N; ++l) {
-        ve[l] = su[3 * (a + N * (l + N * b)) + c];
-        vz[l] = su[3 * (a + N * (b + N * l)) + c];
+        ve[l] = su[L::at(a, l, b) + c];
+        vz[l] = su[L::at(a, b, l) + c];
       }
 #pragma unroll
       for (int m = 0; m < N; ++m) {
@@ -1046,8 +1039,8 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
           de = ffma2(c_h2[m * N + l], ve[l], de);
           dz = ffma2(c_h2[m * N + l], vz[l], dz);
         }
-        se[3 * (a + N * (m + N * b)) + c] = de;
-        sz[3 * (a + N * (b + N * m)) + c] = dz;
+        se[L::at(a, m, b) + c] = de;
+        sz[L::at(a, b, m) + c] = dz;
       }
     }
   }
@@ -1061,10 +1054,10 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
     float2 ux[N], uy[N], uz[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const int p = i + N * line;
-      ux[i] = su[3 * p];
-      uy[i] = su[3 * p + 1];
-      uz[i] = su[3 * p + 2];
+      const int p = L::at(i, a, b);
+      ux[i] = su[p];
+      uy[i] = su[p + 1];
+      uz[i] = su[p + 2];
       fx[i] = fy[i] = fz[i] = make_float2(0.f, 0.f);
     }
 #pragma unroll
@@ -1076,15 +1069,15 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
         dxi_y = ffma2(c_h2[i * N + l], uy[l], dxi_y);
         dxi_z = ffma2(c_h2[i * N + l], uz[l], dxi_z);
       }
-      const int p3 = 3 * (i + N * line);
+      const int p3 = L::at(i, a, b);
       const float2 det_x = se[p3], det_y = se[p3 + 1], det_z = se[p3 + 2];
       const float2 dze_x = sz[p3], dze_y = sz[p3 + 1], dze_z = sz[p3 + 2];
       const int q = i * NL + line;
+      const PointRec pr = load_point<NP>(r, q, active);
       float2 G[9];
 #pragma unroll
-      for (int c = 0; c < 9; ++c) G[c] = bcast2(active ? __ldg(r + (kG + c) * NP + q) : 0.f);
-      const float kappa = active ? __ldg(r + kJKappa * NP + q) : 0.f;  // J kappa
-      const float mu = active ? __ldg(r + kJMu * NP + q) : 0.f;        // J mu
+      for (int c = 0; c < 9; ++c) G[c] = bcast2(pr.G[c]);
+      const float kappa = pr.kappa, mu = pr.mu;  // J kappa, J mu
 
       const float2 uxx = ffma2(dze_x, G[6], ffma2(det_x, G[3], fmul2(dxi_x, G[0])));
       const float2 uxy = ffma2(dze_x, G[7], ffma2(det_x, G[4], fmul2(dxi_x, G[1])));
@@ -1135,8 +1128,8 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
       float2 ve[N], vz[N];
 #pragma unroll
       for (int l = 0; l < N; ++l) {
-        ve[l] = se[3 * (a + N * (l + N * b)) + c];
-        vz[l] = sz[3 * (a + N * (b + N * l)) + c];
+        ve[l] = se[L::at(a, l, b) + c];
+        vz[l] = sz[L::at(a, b, l) + c];
       }
 #pragma unroll
       for (int m = 0; m < N; ++m) {
@@ -1146,8 +1139,8 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
           te = ffma2(c_hw2[l * N + m], ve[l], te);
           tz = ffma2(c_hw2[l * N + m], vz[l], tz);
         }
-        se[3 * (a + N * (m + N * b)) + c] = te;
-        sz[3 * (a + N * (b + N * m)) + c] = tz;
+        se[L::at(a, m, b) + c] = te;
+        sz[L::at(a, b, m) + c] = tz;
       }
     }
   }
@@ -1160,7 +1153,7 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
     for (int i = 0; i < N; ++i) {
       const float wi = W[i];
       const float2 cjk = bcast2(-(wj * wk)), cik = bcast2(-(wi * wk)), cij = bcast2(-(wi * wj));
-      const int p = 3 * (i + N * line);
+      const int p = L::at(i, a, b);
       su[p] = ffma2(cij, sz[p], ffma2(cik, se[p], fmul2(cjk, fx[i])));
       su[p + 1] = ffma2(cij, sz[p + 1], ffma2(cik, se[p + 1], fmul2(cjk, fy[i])));
       su[p + 2] = ffma2(cij, sz[p + 2], ffma2(cik, se[p + 2], fmul2(cjk, fz[i])));
@@ -1169,26 +1162,30 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
   team_sync<KIND, TEAM>(team);
 }
 
-// Points a thread gathers per pass in the pair kernel (all their loads in flight together),
-// lone points and shared nodes it writes per pass (GB300, 48^3 at NGLL 5, 32 shots: a
-// gather batch of 2 beats 4; write batches of 2 beat 1 by 7 %).
+// Points a thread gathers per pass in the pair kernel, all their loads in flight together
+// (GB300, 48^3 at NGLL 5, 32 shots: 2 beats 4).
 constexpr int kPairGatherBatch = 2;
-constexpr int kPairWriteBatch = 4;
-constexpr int kPairSharedBatch = 2;
 
-// Phases 1-3 of one patch for a shot pair (s0, s0 + 1; the second absent when has1 is false:
-// its lanes then carry a copy of the first, never written back).
-template <int N, bool NM>
+// Both shots' slots of a node, one 32-byte load (through L2: u may have been written by the
+// previous kernel).
+__device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+               : "l"(p)
+               : "memory");
+}
+
+// Phases 1-3 of one patch for the shot pair whose slots start at u (the slot past an odd last
+// shot holds zeros, so its lanes compute zeros).
+template <int N>
 __device__ __forceinline__ void patch_gather_compute_pair(const PatchDesc& d, const float* __restrict__ rec,
-                                                          const float4* __restrict__ u, float* wsb2, bool u_from_l2,
-                                                          int S, int s0, bool has1, const SweepNewmark& nm) {
+                                                          const float4* u, float* wsb2) {
   using C = PatchCfg<N>;
   constexpr int NP = C::NP, E = C::E, TEAM = C::TEAM, ES2 = 2 * C::ES, REC = C::REC, GB = kPairGatherBatch;
   const int team = threadIdx.x / TEAM;
   const int tl = threadIdx.x - team * TEAM;
   const int ne = min(E, d.nelem - team * E);
   const float* __restrict__ trec = rec + static_cast<size_t>(d.slot0 + team * E) * REC;
-  const int s1 = has1 ? s0 + 1 : s0;
   float* ts2 = wsb2 + team * 2 * C::TS;
   for (int base = tl; base < ne * NP; base += GB * TEAM) {
     uint32_t w[GB];
@@ -1196,32 +1193,18 @@ __device__ __forceinline__ void patch_gather_compute_pair(const PatchDesc& d, co
     for (int r = 0; r < GB; ++r) {
       const int idx = base + r * TEAM;
       const int le = idx / NP;
-      w[r] = idx < ne * NP ? __float_as_uint(__ldg(trec + static_cast<size_t>(le) * REC + (idx - le * NP))) : 0u;
-    }
-    if constexpr (NM) {
-#pragma unroll
-      for (int r = 0; r < GB; ++r)
-        if (w[r] & kPatchLastBit) {
-          prefetch_l2_line(reinterpret_cast<const float4*>(nm.v) + node_slot<true>(w[r], S, s0));
-          prefetch_l2_line(nm.minv + (w[r] & kNodeMask));
-        }
+      w[r] = idx < ne * NP ? __float_as_uint(__ldg(trec + static_cast<size_t>(le) * REC + kIbool * NP + (idx - le * NP)))
+                           : 0u;
     }
     float4 q0[GB], q1[GB];
 #pragma unroll
-    for (int r = 0; r < GB; ++r) {
-      const float4* pu = u + node_slot<true>(w[r], S, s0);
-      q0[r] = u_from_l2 ? __ldcg(pu) : __ldg(pu);
-      q1[r] = u_from_l2 ? __ldcg(pu + (s1 - s0)) : __ldg(pu + (s1 - s0));
-    }
+    for (int r = 0; r < GB; ++r) load_pair(u + node_slot<true>(w[r]), q0[r], q1[r]);
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
       const int idx = base + r * TEAM;
       if (idx < ne * NP) {
         const int le = idx / NP;
-        const int p = idx - le * NP;
-        float* eb2 = ts2 + le * ES2;
-        reinterpret_cast<uint32_t*>(eb2 + 18 * NP)[2 * p] = w[r];
-        float2* pu2 = reinterpret_cast<float2*>(eb2) + 3 * p;
+        float2* pu2 = reinterpret_cast<float2*>(ts2 + le * ES2) + Ws<N>::at(idx - le * NP);
         pu2[0] = make_float2(q0[r].x, q1[r].x);
         pu2[1] = make_float2(q0[r].y, q1[r].y);
         pu2[2] = make_float2(q0[r].z, q1[r].z);
@@ -1235,135 +1218,54 @@ __device__ __forceinline__ void patch_gather_compute_pair(const PatchDesc& d, co
   }
 }
 
-// The write of one node for one shot of the pair: stored (first touch), added (later
-// touches), or (NM, last touch) the sources and the Newmark update.
-template <bool NM>
-__device__ __forceinline__ void write_node_shot(const PatchDesc& d, const SweepNewmark& nm, float4* __restrict__ f,
-                                                uint32_t w, int S, int shot, float4 prev, const NodeState& st,
-                                                float fx, float fy, float fz) {
-  fx += prev.x;
-  fy += prev.y;
-  fz += prev.z;
-  if (NM && (w & kPatchLastBit)) {
-    if (d.nsrc) add_point_sources(d, nm, w & kNodeMask, shot, fx, fy, fz);
-    newmark_node<true>(nm, w, S, shot, st, fx, fy, fz);
-  } else {
-    f[node_slot<true>(w, S, shot)] = make_float4(fx, fy, fz, 0.f);
-  }
-}
-
-// Phase 4a for a shot pair (the points alone at their patch node, team by team; the loads
-// of GB points in flight before any is written).
+// Phase 4 for a shot pair over the CTA: the rim partials, then the inner nodes completed (nm, f
+// and partials moved to the pair's first slots).
 template <int N, bool NM>
-__device__ __forceinline__ void patch_write_alone_pair(const PatchDesc& d, float4* __restrict__ f, const float* wsb2,
-                                                       const SweepNewmark& nm, int S, int s0, bool has1) {
+__device__ __forceinline__ void patch_finish_pair(const PatchDesc& d, const uint16_t* __restrict__ slot_tab,
+                                                  const uint16_t* __restrict__ word_tab, float4* __restrict__ f,
+                                                  float4* __restrict__ partials, const float* wsb2,
+                                                  const SweepNewmark& nm, int s0) {
   using C = PatchCfg<N>;
-  constexpr int NP = C::NP, E = C::E, TEAM = C::TEAM, ES2 = 2 * C::ES, GB = kPairWriteBatch;
-  const int team = threadIdx.x / TEAM;
-  const int tl = threadIdx.x - team * TEAM;
-  const int ne = min(E, d.nelem - team * E);
-  const float* ts2 = wsb2 + team * 2 * C::TS;
-  const int s1 = has1 ? s0 + 1 : s0;
-  for (int base = tl; base < ne * NP; base += GB * TEAM) {
-    uint32_t w[GB];
-    float4 prev0[GB], prev1[GB];
-    NodeState st0[GB], st1[GB];
-#pragma unroll
-    for (int r = 0; r < GB; ++r) {
-      const int idx = base + r * TEAM;
-      w[r] = 0u;
-      prev0[r] = prev1[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (idx < ne * NP) {
-        const int e = idx / NP;
-        w[r] = reinterpret_cast<const uint32_t*>(ts2 + e * ES2 + 18 * NP)[2 * (idx - e * NP)];
-        if ((w[r] & kAloneBit) && !(w[r] & kPatchFirstBit)) {
-          prev0[r] = load_f<false>(f + node_slot<true>(w[r], S, s0));
-          prev1[r] = load_f<false>(f + node_slot<true>(w[r], S, s1));
-        }
-        if (NM && (w[r] & kAloneBit) && (w[r] & kPatchLastBit)) {
-          load_node_state<true>(nm, w[r], S, s0, st0[r]);
-          load_node_state<true>(nm, w[r], S, s1, st1[r]);
-        }
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < GB; ++r) {
-      const int idx = base + r * TEAM;
-      if (w[r] & kAloneBit) {
-        const int e = idx / NP;
-        const float2* F = reinterpret_cast<const float2*>(ts2 + e * ES2) + 3 * (idx - e * NP);
-        const float2 Fx = F[0], Fy = F[1], Fz = F[2];
-        write_node_shot<NM>(d, nm, f, w[r], S, s0, prev0[r], st0[r], Fx.x, Fy.x, Fz.x);
-        if (has1) write_node_shot<NM>(d, nm, f, w[r], S, s1, prev1[r], st1[r], Fx.y, Fy.y, Fz.y);
-      }
-    }
+  constexpr int T = C::T, MODE = NM ? 1 : 0;
+  SweepNewmark nm1 = nm;  // the second shot's
+  move_fields(nm1, 1);
+  float2 sx, sy, sz;
+  auto sum_at = [&](uint4 g4, const uint4* __restrict__ slots) {
+    sx = sy = sz = make_float2(0.f, 0.f);
+    sum_slots(g4, slots, [&](uint32_t q) {
+      const float2* F = reinterpret_cast<const float2*>(wsb2) + q;
+      sx = fadd2(sx, F[0]);
+      sy = fadd2(sy, F[1]);
+      sz = fadd2(sz, F[2]);
+    });
+  };
+  const uint4* __restrict__ groups = reinterpret_cast<const uint4*>(slot_tab);
+  const uint4* __restrict__ rim = groups + d.rim_slots;
+  for (int t = threadIdx.x; t < d.nrim; t += T) {
+    sum_at(__ldg(rim + t), rim);
+    float4* o = partials + 2 * (static_cast<size_t>(d.rim0) + t);
+    o[0] = make_float4(sx.x, sy.x, sz.x, 0.f);
+    o[1] = make_float4(sx.y, sy.y, sz.y, 0.f);
   }
-}
-
-// Phase 4b for a shot pair over the CTA (the shared patch nodes, their slots summed as pairs;
-// the loads of GB nodes in flight before any is written).
-template <int N, bool NM>
-__device__ __forceinline__ void patch_write_shared_pair(const PatchDesc& d, const uint16_t* __restrict__ slot_tab,
-                                                        const uint16_t* __restrict__ word_tab, float4* __restrict__ f,
-                                                        const float* wsb2, const SweepNewmark& nm, int S, int s0,
-                                                        bool has1) {
-  using C = PatchCfg<N>;
-  constexpr int T = C::T, GB = kPairSharedBatch;
-  const uint4* __restrict__ slots = reinterpret_cast<const uint4*>(slot_tab + d.slot_off);
-  const uint16_t* __restrict__ words = word_tab + d.word_off;
-  const int s1 = has1 ? s0 + 1 : s0;
-  for (int base = threadIdx.x; base < d.nshared; base += GB * T) {
-    uint4 sl[GB];
-    uint32_t w[GB];
-    float4 prev0[GB], prev1[GB];
-    NodeState st0[GB], st1[GB];
-#pragma unroll
-    for (int r = 0; r < GB; ++r) {
-      const int t = base + r * T;
-      const int tt = t < d.nshared ? t : 0;
-      sl[r] = __ldg(slots + tt);
-      w[r] = t < d.nshared ? reinterpret_cast<const uint32_t*>(wsb2)[2 * static_cast<uint32_t>(__ldg(words + tt))]
-                           : kPatchFirstBit;
+  const uint16_t* __restrict__ alone = word_tab + d.alone_off;
+  const uint4* __restrict__ in = groups + d.in_slots;
+  for (int t = threadIdx.x; t < d.nalone + d.nin; t += T) {
+    const uint32_t node = d.inner0 + t;
+    NodeState st0, st1;
+    if constexpr (NM) {
+      load_node_state<true, MODE>(nm, node, st0);
+      load_node_state<true, MODE>(nm1, node, st1);
     }
-#pragma unroll
-    for (int r = 0; r < GB; ++r) {
-      prev0[r] = prev1[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!(w[r] & kPatchFirstBit)) {
-        prev0[r] = load_f<false>(f + node_slot<true>(w[r], S, s0));
-        prev1[r] = load_f<false>(f + node_slot<true>(w[r], S, s1));
-      }
-      if (NM && (w[r] & kPatchLastBit)) {
-        load_node_state<true>(nm, w[r], S, s0, st0[r]);
-        load_node_state<true>(nm, w[r], S, s1, st1[r]);
-      }
+    if (t < d.nalone) {
+      const float2* F = reinterpret_cast<const float2*>(wsb2) + __ldg(alone + t);
+      sx = F[0];
+      sy = F[1];
+      sz = F[2];
+    } else {
+      sum_at(__ldg(in + (t - d.nalone)), in);
     }
-#pragma unroll
-    for (int r = 0; r < GB; ++r) {
-      if (base + r * T >= d.nshared) continue;
-      float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx;
-      uint4 g4 = sl[r];
-      while (true) {
-        const uint32_t wd[4] = {g4.x, g4.y, g4.z, g4.w};
-        uint32_t chain = 0;
-#pragma unroll
-        for (int k = 0; k < kPatchSlots; ++k) {
-          const uint32_t q = (wd[k >> 1] >> (16 * (k & 1))) & 0xFFFFu;
-          if (q == kPatchNoSlot) continue;
-          if (q & kPatchChain) {
-            chain = q;
-            continue;
-          }
-          const float2* F = reinterpret_cast<const float2*>(wsb2 + 2 * q);
-          sx = fadd2(sx, F[0]);
-          sy = fadd2(sy, F[1]);
-          sz = fadd2(sz, F[2]);
-        }
-        if (!chain) break;
-        g4 = __ldg(slots + (chain & ~static_cast<uint32_t>(kPatchChain)));
-      }
-      write_node_shot<NM>(d, nm, f, w[r], S, s0, prev0[r], st0[r], sx.x, sy.x, sz.x);
-      if (has1) write_node_shot<NM>(d, nm, f, w[r], S, s1, prev1[r], st1[r], sx.y, sy.y, sz.y);
-    }
+    complete_node<true, MODE>(nm, f, node, s0, st0, nm.src + d.src_off, d.nsrc, nullptr, 0, sx.x, sy.x, sz.x);
+    complete_node<true, MODE>(nm1, f + 1, node, s0 + 1, st1, nm.src + d.src_off, d.nsrc, nullptr, 0, sx.y, sy.y, sz.y);
   }
 }
 
@@ -1379,34 +1281,40 @@ struct PairCfg {
   static_assert(SMEM <= 227 * 1024, "pair workspace exceeds shared memory");
 };
 
-// One launch per patch colour for S shots: CTA b takes patch p0 + b / ceil(S/2) for the shot
-// pair (2k, 2k + 1), k = b % ceil(S/2) (with odd S the last pair has one shot). The pairs of
-// one patch are consecutive CTAs, so its records come from DRAM once (the first pair's
-// prefetch) and from L2 for the others. Launch order and waits as in patch_forces_kernel.
+// The sweep for S shots: CTA b takes patch b / ceil(S/2) for the shot pair (2k, 2k + 1), k = b %
+// ceil(S/2) (with odd S the last pair has one shot). The pairs of one patch are consecutive
+// CTAs, so its records come from DRAM once (the first pair's prefetch) and from L2 for the
+// others. What a CTA writes is as in patch_forces_kernel.
 template <int N, bool NM>
 __global__ void __launch_bounds__(PatchCfg<N>::T, PairCfg<N>::MIN_BLOCKS)
     patch_forces_pair_kernel(const float* __restrict__ rec, const PatchDesc* __restrict__ desc,
                              const uint16_t* __restrict__ slot_tab, const uint16_t* __restrict__ word_tab,
-                             const float4* __restrict__ u, float4* __restrict__ f, int p0, int S,
-                             const SweepNewmark nm) {
+                             const float4* __restrict__ u, float4* __restrict__ f, float4* __restrict__ partials,
+                             int S, const SweepNewmark nm_arg) {
   using C = PatchCfg<N>;
+  SweepNewmark nm = nm_arg;
   extern __shared__ float4 smem4[];
   float* wsb2 = reinterpret_cast<float*>(smem4);
   const int SP = (S + 1) / 2;
-  const int P = p0 + static_cast<int>(blockIdx.x) / SP;
-  const int k = static_cast<int>(blockIdx.x) - (P - p0) * SP;
+  const int P = static_cast<int>(blockIdx.x) / SP;
+  const int k = static_cast<int>(blockIdx.x) - P * SP;
   const int s0 = 2 * k;
-  const bool has1 = s0 + 1 < S;
   const PatchDesc d = desc[P];
   if (k == 0 && threadIdx.x < d.nelem)
     prefetch_l2(rec + static_cast<size_t>(d.slot0 + threadIdx.x) * C::REC, kForceFields * C::NP * sizeof(float));
-  if (p0 == 0) wait_prerequisite_grid();
+  wait_prerequisite_grid();
   allow_dependent_grid();
-  patch_gather_compute_pair<N, NM>(d, rec, u, wsb2, p0 != 0, S, s0, has1, nm);
-  if (p0 != 0) wait_prerequisite_grid();
-  patch_write_alone_pair<N, NM>(d, f, wsb2, nm, S, s0, has1);
+  if constexpr (NM) record_receivers(d, nm, u, S, s0, s0 + 1 < S ? 2 : 1);
+  const size_t slot = field_slot(nm.nglob, 2, 0, s0);  // to the pair's slots
+  move_fields(nm, slot);
+  u += slot;
+  f += slot;
+  partials += field_slot(nm.nsums, 2, 0, s0);
+  if constexpr (NM)
+    if (threadIdx.x == 0) prefetch_inner<1>(d, nm, 2);
+  patch_gather_compute_pair<N>(d, rec, u, wsb2);
   __syncthreads();
-  patch_write_shared_pair<N, NM>(d, slot_tab, word_tab, f, wsb2, nm, S, s0, has1);
+  patch_finish_pair<N, NM>(d, slot_tab, word_tab, f, partials, wsb2, nm, s0);
 }
 
 // Persistent form: one sweep (all patch colours) in one launch. CTAs take patches in sweep
@@ -1466,12 +1374,11 @@ __device__ __noinline__ int sweep_one_patch(int P, const float* __restrict__ rec
   }
   __syncthreads();
   const PatchDesc& d = sh->d;
-  const SweepNewmark none{};  // the persistent sweep assembles forces only
   prefetch_patch_records<N>(rec, desc, sh->next, npatch);
-  patch_gather_compute<N, LO>(d, rec, u, wsb, false);
+  patch_gather_compute<N, LO, false, true>(d, rec, u, wsb);
   const int c = sh->color;
   if (sh->ready) {
-    patch_write_alone<N, true>(d, f, wsb, none);
+    patch_write_alone<N>(d, f, wsb);
     __syncthreads();
   } else {
     __syncthreads();
@@ -1489,9 +1396,9 @@ __device__ __noinline__ int sweep_one_patch(int P, const float* __restrict__ rec
     }
     __syncthreads();  // the wait is over for the CTA
     if (sh->abort) return -1;
-    patch_write_alone<N, true>(d, f, wsb, none);
+    patch_write_alone<N>(d, f, wsb);
   }
-  patch_write_shared<N, true>(d, slot_tab, word_tab, f, wsb, none);
+  patch_write_shared<N>(d, slot_tab, word_tab, f, wsb);
   __syncthreads();  // all of the patch's writes issued before it counts as done
   if (threadIdx.x == 0) {
     __threadfence();
@@ -1592,14 +1499,13 @@ __device__ __noinline__ int group_one_item(int item, const GroupLaunch L, GroupS
   __syncthreads();
   const PatchDesc& d = sh->d;
   const GroupModel& m = sh->m;
-  const SweepNewmark none{};
   group_prefetch_item<N>(L, sh->next);
   float4* f = reinterpret_cast<float4*>(m.f);
-  patch_gather_compute<N, LO>(d, m.rec, reinterpret_cast<const float4*>(m.u), wsb, false);
+  patch_gather_compute<N, LO, false, true>(d, m.rec, reinterpret_cast<const float4*>(m.u), wsb);
   const int c = sh->color;
   unsigned int* done = &L.sync->done[sh->model * kMaxSweepColors];
   if (sh->ready) {
-    patch_write_alone<N, true>(d, f, wsb, none);
+    patch_write_alone<N>(d, f, wsb);
     __syncthreads();
   } else {
     __syncthreads();
@@ -1617,9 +1523,9 @@ __device__ __noinline__ int group_one_item(int item, const GroupLaunch L, GroupS
     }
     __syncthreads();  // the wait is over for the CTA
     if (sh->abort) return -1;
-    patch_write_alone<N, true>(d, f, wsb, none);
+    patch_write_alone<N>(d, f, wsb);
   }
-  patch_write_shared<N, true>(d, m.slots, m.words, f, wsb, none);
+  patch_write_shared<N>(d, m.slots, m.words, f, wsb);
   __syncthreads();  // all of the patch's writes issued before it counts as done
   if (threadIdx.x == 0) {
     __threadfence();
@@ -1709,7 +1615,8 @@ __global__ void __launch_bounds__(ForceCfg<N>::T)
       const int idx = base + r * TEAM;
       const int le = idx / NP;
       g[r] = idx < ne * NP
-                 ? __float_as_uint(__ldg(rec + static_cast<size_t>(ebase + le) * REC + (idx - le * NP))) & kNodeMask
+                 ? __float_as_uint(__ldg(rec + static_cast<size_t>(ebase + le) * REC + kIbool * NP + (idx - le * NP))) &
+                       kNodeMask
                  : 0;
     }
     float4 l4[GB];
@@ -1778,9 +1685,8 @@ __global__ void __launch_bounds__(ForceCfg<N>::T)
       }
     }
     const int q = i * NL + line;
-    float G[9];
-#pragma unroll
-    for (int a = 0; a < 9; ++a) G[a] = __ldg(r + (kG + a) * NP + q);
+    const PointRec pr = load_point<NP>(r, q, true);
+    const float(&G)[9] = pr.G;
     const float jac = __ldg(r + kJac * NP + q);
     float gl[3][3], gu[3][3];  // physical gradients [component][x_d]
 #pragma unroll
@@ -1834,7 +1740,7 @@ int launch_forces_ms(const ForceLaunch& L, cudaStream_t s) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return static_cast<int>(cudaLaunchKernelEx(&cfg, forces_kernel<SEM_NGLL, MS, LO, CALLER, ATOMIC>, L.rec, L.elist, L.perm, L.u, L.f, L.e0, L.e1, S));
+  return static_cast<int>(cudaLaunchKernelEx(&cfg, forces_kernel<SEM_NGLL, MS, LO, CALLER, ATOMIC>, L.rec, L.elist, L.perm, L.u, L.f, L.e0, L.e1, S, L.nglob));
 }
 
 int launch_forces_n(const ForceLaunch& L, cudaStream_t s) {
@@ -1854,92 +1760,90 @@ int launch_forces_n(const ForceLaunch& L, cudaStream_t s) {
   return lo ? launch_forces_ms<false, true, false>(L, s) : launch_forces_ms<false, false, false>(L, s);
 }
 
-template <bool LO, bool PAIRS>
-int launch_patch_lo(const PatchLaunch& L, cudaStream_t s) {
-  using C = PatchCfg<SEM_NGLL>;
-  static std::atomic<unsigned long long> attr_done{0}, attr_done_n{0}, attr_done_s{0}, attr_done_sn{0}, attr_done_a{0}, attr_done_ns{0}, attr_done_p{0};
-  static std::atomic<int> resident[64];  // CTAs of the persistent kernel per SM, per device
+// A launch of the sweep kernel k on grid CTAs, its shared-memory limit raised first.
+template <class K>
+int launch_sweep(std::atomic<unsigned long long>& attr_done, K k, unsigned grid, int smem, int shots,
+                 const PatchLaunch& L, cudaStream_t s) {
+  if (int r = raise_smem_limit(attr_done, k, smem)) return r;
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(C::T);
-  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(PatchCfg<SEM_NGLL>::T);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (L.sync && !PAIRS) {  // one persistent launch for the whole sweep
-    if (int r = raise_smem_limit(attr_done_p, patch_sweep_kernel<SEM_NGLL, LO>, C::SMEM)) return r;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int per_sm = resident[dev & 63].load();
-    if (per_sm <= 0) {
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, patch_sweep_kernel<SEM_NGLL, LO>, C::T,
-                                                                    C::SMEM);
-      if (e != cudaSuccess) return static_cast<int>(e);
-      per_sm = per_sm < 1 ? 1 : per_sm;
-      resident[dev & 63].store(per_sm);
-    }
-    int sms = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return static_cast<int>(cudaLaunchKernelEx(&cfg, k, L.rec, L.desc, L.slots, L.words,
+                                             reinterpret_cast<const float4*>(L.u), reinterpret_cast<float4*>(L.f),
+                                             reinterpret_cast<float4*>(L.partials), shots, L.nm));
+}
+
+template <bool LO, bool MS, int NM>
+int launch_patch_nm(const PatchLaunch& L, cudaStream_t s) {
+  static std::atomic<unsigned long long> attr_done{0};
+  const long long grid = static_cast<long long>(L.npatch) * (MS ? L.shots : 1);
+  if (grid > 0x7FFFFFFFll) return static_cast<int>(cudaErrorInvalidValue);
+  return launch_sweep(attr_done, patch_forces_kernel<SEM_NGLL, LO, MS, NM>, static_cast<unsigned>(grid),
+                      PatchCfg<SEM_NGLL>::SMEM, MS ? L.shots : 1, L, s);
+}
+
+template <bool NM>
+int launch_pair(const PatchLaunch& L, cudaStream_t s) {
+  static std::atomic<unsigned long long> attr_done{0};
+  const long long grid = static_cast<long long>(L.npatch) * ((L.shots + 1) / 2);
+  if (grid > 0x7FFFFFFFll) return static_cast<int>(cudaErrorInvalidValue);
+  return launch_sweep(attr_done, patch_forces_pair_kernel<SEM_NGLL, NM>, static_cast<unsigned>(grid),
+                      PairCfg<SEM_NGLL>::SMEM, L.shots, L, s);
+}
+
+template <bool LO>
+int launch_persistent(const PatchLaunch& L, cudaStream_t s) {
+  using C = PatchCfg<SEM_NGLL>;
+  static std::atomic<unsigned long long> attr_done{0};
+  static std::atomic<int> resident[64];  // CTAs per SM, per device
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(C::T);
+  cfg.dynamicSmemBytes = C::SMEMW;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (int r = raise_smem_limit(attr_done, patch_sweep_kernel<SEM_NGLL, LO>, C::SMEMW)) return r;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int per_sm = resident[dev & 63].load();
+  if (per_sm <= 0) {
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, patch_sweep_kernel<SEM_NGLL, LO>, C::T,
+                                                                  C::SMEMW);
     if (e != cudaSuccess) return static_cast<int>(e);
-    cfg.gridDim = dim3(static_cast<unsigned>(sms * per_sm));
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_sweep_kernel<SEM_NGLL, LO>, L.rec, L.desc, L.slots, L.words,
-                                               reinterpret_cast<const float4*>(L.u), reinterpret_cast<float4*>(L.f),
-                                               L.npatch, L.color_end, L.ncolors, L.stall ? 1u : 0u, L.sync));
+    per_sm = per_sm < 1 ? 1 : per_sm;
+    resident[dev & 63].store(per_sm);
   }
-  if constexpr (PAIRS) {
-    using PC = PairCfg<SEM_NGLL>;
-    cfg.dynamicSmemBytes = PC::SMEM;
-    cfg.gridDim = dim3(static_cast<unsigned>((L.p1 - L.p0) * ((L.shots + 1) / 2)));
-    if (L.nm.mode) {
-      if (int r = raise_smem_limit(attr_done_n, patch_forces_pair_kernel<SEM_NGLL, true>, PC::SMEM)) return r;
-      return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_pair_kernel<SEM_NGLL, true>, L.rec, L.desc,
-                                                 L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                                 reinterpret_cast<float4*>(L.f), L.p0, L.shots, L.nm));
-    }
-    if (int r = raise_smem_limit(attr_done, patch_forces_pair_kernel<SEM_NGLL, false>, PC::SMEM)) return r;
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_pair_kernel<SEM_NGLL, false>, L.rec, L.desc,
-                                               L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                               reinterpret_cast<float4*>(L.f), L.p0, L.shots, L.nm));
-  } else if (L.shots > 1) {  // one CTA per (patch, shot)
-    const int S = L.shots;
-    cfg.gridDim = dim3(static_cast<unsigned>((L.p1 - L.p0) * S));
-    if (L.nm.mode) {
-      if (int r = raise_smem_limit(attr_done_sn, patch_forces_kernel<SEM_NGLL, LO, true, 1>, C::SMEM)) return r;
-      return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_kernel<SEM_NGLL, LO, true, 1>, L.rec, L.desc,
-                                                 L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                                 reinterpret_cast<float4*>(L.f), L.p0, S, L.nm));
-    }
-    if (int r = raise_smem_limit(attr_done_s, patch_forces_kernel<SEM_NGLL, LO, true, 0>, C::SMEM)) return r;
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_kernel<SEM_NGLL, LO, true, 0>, L.rec, L.desc,
-                                               L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                               reinterpret_cast<float4*>(L.f), L.p0, S, L.nm));
-  } else {
-    const int S = 1;
-    cfg.gridDim = dim3(static_cast<unsigned>(L.p1 - L.p0));
-    if (L.nm.mode && L.nm.mode != 3 && L.nm.snap_ctl) {  // a snapshot run's Newmark sweep
-      if (int r = raise_smem_limit(attr_done_ns, patch_forces_kernel<SEM_NGLL, LO, false, 3>, C::SMEM)) return r;
-      return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_kernel<SEM_NGLL, LO, false, 3>, L.rec, L.desc,
-                                                 L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                                 reinterpret_cast<float4*>(L.f), L.p0, S, L.nm));
-    }
-    if (L.nm.mode == 3) {  // the adjoint leapfrog at each node's last touch
-      if (int r = raise_smem_limit(attr_done_a, patch_forces_kernel<SEM_NGLL, LO, false, 2>, C::SMEM)) return r;
-      return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_kernel<SEM_NGLL, LO, false, 2>, L.rec, L.desc,
-                                                 L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                                 reinterpret_cast<float4*>(L.f), L.p0, S, L.nm));
-    }
-    if (L.nm.mode) {
-      if (int r = raise_smem_limit(attr_done_n, patch_forces_kernel<SEM_NGLL, LO, false, 1>, C::SMEM)) return r;
-      return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_kernel<SEM_NGLL, LO, false, 1>, L.rec, L.desc,
-                                                 L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                                 reinterpret_cast<float4*>(L.f), L.p0, S, L.nm));
-    }
-    if (int r = raise_smem_limit(attr_done, patch_forces_kernel<SEM_NGLL, LO, false, 0>, C::SMEM)) return r;
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_forces_kernel<SEM_NGLL, LO, false, 0>, L.rec, L.desc,
-                                               L.slots, L.words, reinterpret_cast<const float4*>(L.u),
-                                               reinterpret_cast<float4*>(L.f), L.p0, S, L.nm));
+  int sms = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return static_cast<int>(e);
+  cfg.gridDim = dim3(static_cast<unsigned>(sms * per_sm));
+  return static_cast<int>(cudaLaunchKernelEx(&cfg, patch_sweep_kernel<SEM_NGLL, LO>, L.rec, L.desc, L.slots, L.words,
+                                             reinterpret_cast<const float4*>(L.u), reinterpret_cast<float4*>(L.f),
+                                             L.npatch, L.color_end, L.ncolors, L.stall ? 1u : 0u, L.sync));
+}
+
+template <bool LO>
+int launch_patch_lo(const PatchLaunch& L, cudaStream_t s) {
+  if (L.sync) return launch_persistent<LO>(L, s);
+  if (L.shots > 1) {  // one CTA per (patch, shot)
+    if (L.nm.mode > 2) return static_cast<int>(cudaErrorInvalidValue);
+    return L.nm.mode ? launch_patch_nm<LO, true, 1>(L, s) : launch_patch_nm<LO, true, 0>(L, s);
+  }
+  switch (L.nm.mode) {
+    case 0: return launch_patch_nm<LO, false, 0>(L, s);
+    case 3: return launch_patch_nm<LO, false, 2>(L, s);
+    case 4: return launch_patch_nm<LO, false, 4>(L, s);
+    default: return L.nm.snap ? launch_patch_nm<LO, false, 3>(L, s) : launch_patch_nm<LO, false, 1>(L, s);
   }
 }
 
@@ -1948,13 +1852,13 @@ int launch_group_lo(const GroupLaunch& L, cudaStream_t s) {
   using C = PatchCfg<SEM_NGLL>;
   static std::atomic<unsigned long long> attr_done{0};
   static std::atomic<int> resident[64];  // CTAs per SM, per device
-  if (int r = raise_smem_limit(attr_done, group_sweep_kernel<SEM_NGLL, LO>, C::SMEM)) return r;
+  if (int r = raise_smem_limit(attr_done, group_sweep_kernel<SEM_NGLL, LO>, C::SMEMW)) return r;
   int dev = 0;
   cudaGetDevice(&dev);
   int per_sm = resident[dev & 63].load();
   if (per_sm <= 0) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, group_sweep_kernel<SEM_NGLL, LO>, C::T,
-                                                                  C::SMEM);
+                                                                  C::SMEMW);
     if (e != cudaSuccess) return static_cast<int>(e);
     per_sm = per_sm < 1 ? 1 : per_sm;
     resident[dev & 63].store(per_sm);
@@ -1968,7 +1872,7 @@ int launch_group_lo(const GroupLaunch& L, cudaStream_t s) {
   const int grid = std::min(sms * per_sm, std::max(1, L.nitems));
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
   cfg.blockDim = dim3(C::T);
-  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.dynamicSmemBytes = C::SMEMW;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1979,11 +1883,14 @@ int launch_group_lo(const GroupLaunch& L, cudaStream_t s) {
 }
 
 int launch_patch_n(const PatchLaunch& L, cudaStream_t s) {
-  if (L.sync ? L.npatch <= 0 : L.p1 <= L.p0) return 0;
+  if (L.npatch <= 0) return 0;
   using C = ForceCfg<SEM_NGLL>;
+  if (L.shots > 1 && L.pairs && !L.sync) {  // shot pairs: line owners
+    if (L.nm.mode > 2) return static_cast<int>(cudaErrorInvalidValue);
+    return L.nm.mode ? launch_pair<true>(L, s) : launch_pair<false>(L, s);
+  }
   const bool lo = L.variant == 0 ? C::LINE_OWNERS : L.variant == 1;
-  if (L.shots > 1 && L.pairs) return launch_patch_lo<true, true>(L, s);  // shot pairs: line owners
-  return lo ? launch_patch_lo<true, false>(L, s) : launch_patch_lo<false, false>(L, s);
+  return lo ? launch_patch_lo<true>(L, s) : launch_patch_lo<false>(L, s);
 }
 
 }  // namespace
@@ -2046,11 +1953,9 @@ int SEM_CAT(launch_group_sweep_, SEM_NGLL)(const GroupLaunch& L, void* stream) {
             : launch_group_lo<false>(L, static_cast<cudaStream_t>(stream));
 }
 
-void SEM_CAT(patch_layout_, SEM_NGLL)(int* es, int* ts, int* e) {
+void SEM_CAT(patch_layout_, SEM_NGLL)(PatchLayout* out) {
   using C = PatchCfg<SEM_NGLL>;
-  *es = C::ES;
-  *ts = C::TS;
-  *e = C::E;
+  *out = PatchLayout{Ws<SEM_NGLL>::SY, Ws<SEM_NGLL>::SZ, C::ES, C::TS, C::ESW, C::TSW, C::WORDS, C::E};
 }
 
 void SEM_CAT(patch_shape_, SEM_NGLL)(PatchShape* out) {

@@ -13,21 +13,44 @@ namespace semgb {
 
 using sem_ctx_fwd = ::sem_ctx;
 
+#ifdef __CUDACC__
+#define SEM_HD __host__ __device__
+#else
+#define SEM_HD
+#endif
+
 constexpr int kMaxNgll = 10;
 constexpr int kMinNgll = 2;
 
-// Words per local point in the element record: ibool, nine inverse-Jacobian terms
-// dxi_r/dx_d (r-major: xix xiy xiz etax etay etaz gammax gammay gammaz), J kappa, J mu, J.
-// The force kernels read the first kForceFields fields only (J sigma from J kappa and J mu
-// needs no separate J); J serves the mass and the material sensitivities.
+// Element record: per local point nine inverse-Jacobian terms dxi_r/dx_d (r-major: xix xiy xiz
+// etax etay etaz gammax gammay gammaz), J kappa, J mu, the ibool word and J. Laid out for wide
+// loads, the points of a field group in rec_pos order: [np][4] G0..G3, [np][4] G4..G7, [np][2]
+// G8 and J kappa, [np] J mu, then [np] ibool words (natural point order) and [np] J, so the
+// eleven values a force kernel needs at a point are two 16-byte, one 8-byte and one 4-byte load
+// (eleven 4-byte loads of 500-byte fields, which straddle 128-byte lines, measured 1.8 L1
+// wavefronts each at NGLL 5). The force kernels read the first kForceFields words per point
+// (J sigma from J kappa and J mu needs no separate J); J serves the mass and the sensitivities.
 constexpr int kRecFields = 13;
 constexpr int kForceFields = 12;
-enum RecField { kIbool = 0, kG = 1, kJKappa = 10, kJMu = 11, kJac = 12 };
+constexpr int kIbool = 11, kJac = 12;  // words per point before the ibool words and before J
+// Word of inverse-Jacobian term c (0 .. 8), J kappa (9) or J mu (10) at point position q.
+SEM_HD constexpr int rec_at(int np, int c, int q) {
+  return c < 4 ? 4 * q + c : c < 8 ? 4 * np + 4 * q + c - 4 : c < 10 ? 8 * np + 2 * q + c - 8 : 10 * np + q;
+}
 
 // The context's own wavefields u, v, a are float32 [nglob][kNodeStride]: x, y, z and a zero
 // pad, so that every node is one aligned 16-byte access in the gather, the scatter and the
 // Newmark passes. Caller-facing arrays stay [nglob][3]; copies at the boundary are strided.
 constexpr int kNodeStride = 4;
+// With several shots a field is [ceil(shots / 2)][nglob][2][kNodeStride]: the shots in pairs, a
+// pair's two slots one 32-byte sector, the nodes of a pair as for a single shot. The gather of
+// a shot pair reads a row of nodes as one run (with the shots of a node together, 512 bytes
+// apart at 32 shots, every node was an L1 wavefront of its own). An odd last shot leaves a slot
+// that stays zero.
+SEM_HD constexpr int padded_shots(int shots) { return shots > 1 ? (shots + 1) / 2 * 2 : 1; }
+SEM_HD inline size_t field_slot(size_t nglob, int shots, size_t node, int shot) {
+  return shots > 1 ? (static_cast<size_t>(shot >> 1) * nglob + node) * 2 + (shot & 1) : node;
+}
 
 // Bit 31 of a record's ibool word marks the first contribution to that node in the
 // colour-by-colour processing order: the force kernel stores instead of adding there,
@@ -37,8 +60,8 @@ constexpr uint32_t kFirstTouchBit = 0x80000000u;
 // word of the first local point (in patch-table order) of each patch node. Bit 29 marks a
 // local point that is the only one of its patch at its node (its element's team writes it
 // alone). Bit 28 marks, on every local point of a patch node, that this patch is the node's
-// last toucher in the sweep (its force is complete there: the Newmark update of the node can
-// run in the same pass). Node ids are below 2^28.
+// last toucher in the sweep. A first local point with bits 30 and 28 is at an inner node (one
+// that only this patch touches). Node ids are below 2^28.
 constexpr uint32_t kPatchFirstBit = 0x40000000u;
 constexpr uint32_t kAloneBit = 0x20000000u;
 constexpr uint32_t kPatchLastBit = 0x10000000u;
@@ -92,6 +115,7 @@ struct PatchPlan {
   std::vector<int> tab_nelem, tab_nnode, tab_nshared, tab_lid_off, tab_csr_off, tab_excl_off, tab_first_off;
   std::vector<uint16_t> lid;      // per table: [nelem][np] patch-local node of each local point
   std::vector<int> node_new;      // [nglob] internal id of every caller node
+  int ninner = 0;                 // internal ids below this: nodes of one patch only
   std::vector<uint16_t> csr;      // per table: per shared patch node (one met by several local
                                   // points) kPatchSlots slots holding those local points
                                   // (le*np + p, ascending)
@@ -134,7 +158,7 @@ struct DevProblem {
   int ngll;
   int nspec;
   int nglob;
-  int shots;  // wavefields are [nglob][shots][kNodeStride]
+  int shots;  // wavefields are (fields, kNodeStride)
   const float* rec;
   float* u;
   float* v;
@@ -165,14 +189,16 @@ struct ForceLaunch {
   int e0, e1;
   int node_stride;  // floats per node in u and f: kNodeStride (internal order), or 3 for caller
                     // arrays in caller order
-  int shots;        // > 1: u and f are [nglob][shots][kNodeStride], items (element, shot)
+  int shots;        // > 1: u and f are fields of several shots, items (element, shot)
+  int nglob;
   int variant;      // contraction form: 0 the order's default, 1 line owners, 2 per point
   int atomic;       // colouring ablation: float atomic adds into a zeroed f, any element order
 };
 int launch_forces(int ngll, const ForceLaunch& launch, void* stream);
 
-// One patch colour [p0, p1) of the patch sweep order on the context's own [nglob][shots][4]
-// fields: f (=|+=) -K u.
+// A patch of the sweep. Its nodes are inner (of this patch only) or rim (shared with other
+// patches); the sweep completes the inner ones and leaves one partial force sum per rim node
+// in the partials buffer, which the rim pass (launch_rim_combine) sums per node.
 struct alignas(16) PatchDesc {
   int slot0;     // record slot of the patch's first element (its elements are consecutive)
   int nelem;
@@ -182,10 +208,22 @@ struct alignas(16) PatchDesc {
   int word_off;  // its table: per shared node, the shared-memory offset of its first local
                  // point's ibool word
   int src_off;   // its point sources (PatchSrc entries [src_off, src_off + nsrc)): the ones at
-  int nsrc;      // nodes it touches last, added there to the complete force
-  int pad;
+  int nsrc;      // its inner nodes, added there to the complete force
+  int inner0;    // its inner nodes: ids inner0 .. + nalone (one local point each, the shared-
+  int nalone;    // memory offsets of their forces at alone_off), then nin met by several
+  int alone_off; // (slot groups from in_slots on)
+  int nin;
+  int in_slots;
+  int nrim;      // rim nodes, ascending internal id
+  int rim_slots; // their slot groups (index of the first)
+  int rim0;      // partial of rim node k: field_slot(partials a shot, shots, rim0 + k, shot)
+  int rec_off;   // its receivers (PatchRecv entries [rec_off, rec_off + nrec)): the ones at its
+  int nrec;      // inner nodes, then at rim nodes it touches last
+  int nrec_in;   // how many of them are at inner nodes
+  int pad[2];
 };
-// A receiver in the adjoint sweep: internal node, receiver index (its residual G[3 r + c]).
+static_assert(sizeof(PatchDesc) == 80, "PatchDesc is five 16-byte words");
+// A receiver in the sweep: internal node, receiver index (residual G[3 r + c]).
 struct PatchRecv {
   int node;
   int r;
@@ -197,35 +235,52 @@ struct PatchSrc {
   int shot;
   double f[3];
 };
-// The explicit Newmark update (Sec. I) run by the patch sweep at each node's last toucher:
+// The point sources and receivers at kRimBlock consecutive rim nodes (by block of rim nodes).
+constexpr int kRimBlock = 256;
+struct alignas(16) RimBlock {
+  int src_off, nsrc;
+  int rec_off, nrec;
+};
+// The partials that meet at a rim node, in sweep order of their patches: up to four indices
+// (-1: none); with more, w = -2 - o names the list over[o] = count, over[o + 1 ..] = indices.
+struct alignas(16) RimNode {
+  int x, y, z, w;
+};
+// The explicit Newmark update (Sec. I) run by the sweep at every node whose force is complete:
 // mode 1 corrector of step n fused with the predictor of step n+1
 //   a = M^-1 f ; v = v_half + dt/2 a ; u <- u + dt v + dt^2/2 a ; v_half <- v + dt/2 a
 // (f is then not stored), mode 2 the corrector alone (v <- v_half + dt/2 a, a stored), mode 0
-// none (f stored). The point sources of the step, at t = ctl->step dt, are added to f first.
+// none (f stored), mode 4 none (f stored into a caller array [nglob][3] through perm). The
+// point sources of the step, at t = (ctl->step + ahead + 1) dt, are added to f first.
 struct SweepNewmark {
   int mode;           // 3: the adjoint leapfrog (u = lam^m; lam_old: lam^{m+1} in, lam^{m-1} out)
-  float* u;           // [nglob][shots][4], written at last touch (mode 1)
-  float* v;           // [nglob][shots][4], half-step velocity in, out as above
-  float* a;           // [nglob][shots][4], acceleration out (mode 2)
+  int nglob, nsums;   // field and partials strides of a shot pair
+  float* u;           // field, written where the force is complete (mode 1)
+  float* v;           // field, half-step velocity in, out as above
+  float* a;           // field, acceleration out (mode 2)
   const float* minv;  // [nglob]
   const PatchSrc* src;
-  const long long* step;  // the step counter (t_{n+1} = step dt)
-  double f0, t0, dtd;     // Ricker centre frequency and delay, step (double)
+  const PatchSrc* rim_src;  // the sources at rim nodes, by rim block
+  const DevCtl* ctl;        // step counter, seismogram and snapshot buffers
+  int ahead;                // steps enqueued since the counter was last set or advanced
+  double f0, t0, dtd;       // Ricker centre frequency and delay, step (double)
   float dt, hdt, hdt2;
-  // adjoint (mode 3): the receivers at the nodes each patch touches last (recv_range[2 P],
-  // recv_range[2 P + 1] = first, count into recv, ascending receiver within a patch), the
-  // residual G [nrec][3]
-  // (or, with idx, the one the device's adjoint counter names), 1/dt^2 and dt^2
-  // snapshot run (modes 1, 2): u^{n+1} also stored at each node's last touch into
-  // ctl->snap + (ctl->col - 1) ctl->snap_per, [nglob][3] in the order snap_perm maps to
-  const DevCtl* snap_ctl;
+  // the receivers by patch: sampled (u^{n+1}, modes 1 and 2) into ctl->seis column ctl->col +
+  // ahead before the patch's nodes are updated; adjoint (mode 3): their residuals G [nrec][3]
+  // (or, with idx, those the device's adjoint counter names) added at inner nodes, and by rim
+  // block at rim nodes, ascending receiver
+  const PatchRecv* recv;
+  const PatchRecv* rim_recv;
+  int nrec;            // receivers of the model
+  // snapshot run (modes 1, 2): u^{n+1} also stored where it is updated into ctl->snap +
+  // (ctl->col + ahead) ctl->snap_per, [nglob][3] in the order snap_perm maps to
+  int snap;
   const int* snap_perm;
   float* lam_old;
-  const int* recv_range;
-  const PatchRecv* recv;
   const float* G;
   const DevCtl* idx;
   float inv_dt2, dt2;
+  const int* perm;  // mode 4: internal -> caller node
 };
 // Counters of a persistent sweep (all patch colours in one launch): patches taken, CTAs
 // that have left, a wait that gave up, patches finished per colour. Zero between sweeps.
@@ -278,47 +333,71 @@ struct GroupLaunch {
 };
 int launch_group_sweep(int ngll, const GroupLaunch& launch, void* stream);
 
+// One patch sweep on (fields, kNodeStride) fields: f = -K u at the inner nodes (or their
+// update, nm.mode), partial sums at the rim.
 struct PatchLaunch {
   const float* rec;
   const PatchDesc* desc;
   const uint16_t* slots;
   const uint16_t* words;
-  SweepSync* sync;        // non-null: one persistent launch over all colours
+  SweepSync* sync;        // non-null: one persistent launch over all colours (assembles all of f)
   const int* color_end;   // per colour, the end of its patch range (persistent launch)
-  int npatch, ncolors;    // (persistent launch)
+  int ncolors;            // (persistent launch)
   int stall;              // (persistent launch) wait for a count that never arrives (tests)
+  int npatch;
   const float* u;
   float* f;
-  int p0, p1;
+  float* partials;  // laid out like a field over the rim partials
   int variant;  // contraction form as in ForceLaunch
-  int shots;    // > 1: fields [nglob][shots][kNodeStride]
+  int shots;    // > 1: fields (fields, kNodeStride)
   int pairs;    // with shots > 1: one CTA per (patch, shot pair) (else one per (patch, shot))
   SweepNewmark nm;  // mode 0: forces only
 };
 int launch_patch_forces(int ngll, const PatchLaunch& launch, void* stream);
-// Shared-memory layout of the patch kernel for this order: workspace floats per element,
-// per team, and elements per team (the slot tables hold offsets into it).
-int patch_layout(int ngll, int* es, int* ts, int* e);
+// Shared-memory layout of the patch kernels for this order: a local point (i, j, k) of an
+// element workspace at float 3 (i + sy j + sz k); floats per element and per team of the sweep
+// (es, ts) and of the persistent sweeps, which also keep the ibool words (from float words on;
+// esw, tsw); elements per team.
+struct PatchLayout {
+  int sy, sz, es, ts, esw, tsw, words, e;
+};
+int patch_layout(int ngll, PatchLayout* out);
 // the brick each order's patch kernel is compiled for
 int patch_shape(int ngll, PatchShape* out);
 int forces_kernel_smem_bytes(int ngll);
 int forces_elements_per_cta(int ngll);
 
+// The rim pass after a sweep: per rim node the sum of its partials in sweep order, then what
+// the sweep did at the inner nodes (nm.mode).
+struct RimLaunch {
+  const RimNode* rim;   // [nrim]
+  const int* over;
+  const RimBlock* blocks;  // [ceil(nrim / kRimBlock)]
+  const float* partials;
+  float* f;
+  int ninner;           // internal id of rim node 0
+  int nrim;
+  int shots;
+  SweepNewmark nm;
+};
+int launch_rim_combine(const RimLaunch& launch, void* stream);
+// step and column of the counter += steps
+int launch_advance_ctl(DevCtl* ctl, int steps, void* stream);
 int launch_set_ctl(DevCtl* ctl, long long step, int ncols, float* seis, void* stream, float* snap = nullptr,
                    long long snap_per = 0);
-// the displacement into snapshot ctl->col - 1 (the column the receivers just sampled)
-int launch_snapshot(const float* u, DevCtl* ctl, const int* perm, int nglob, int shots, void* stream);
+// the displacement into snapshot ctl->col + ahead
+int launch_snapshot(const float* u, const DevCtl* ctl, int ahead, const int* perm, int nglob, int shots, void* stream);
 int launch_predictor(const DevProblem& p, void* stream);
 int launch_fused_newmark(const DevProblem& p, void* stream);
 int launch_corrector(const DevProblem& p, void* stream);
-int launch_sources_record(const DevProblem& p, void* stream);
+int launch_sources_record(const DevProblem& p, int ahead, void* stream);
 // u_lo, u_mid, u_hi: [nglob][3] in caller order (perm: internal -> caller node) or in
 // internal order (perm null); the terms are added to float32 partials g_* [nlocal]
 // (idx non-null: the snapshots are idx->adj_u + (j - 1 .. j + 1) idx->adj_n3, j = idx->adj_j)
 int launch_sensitivity(int ngll, const float* rec, const int* perm, const float* lam, const float* u_lo,
                        const float* u_mid, const float* u_hi, float* g_rho, float* g_kappa, float* g_mu, int nspec,
                        double c_m, double c_k, void* stream, const DevCtl* idx = nullptr);
-// solver layout [nglob][shots][kNodeStride] in internal node order <-> caller layout
+// fields in internal node order <-> caller layout
 // [shots][nglob][3] in caller node order (perm: internal -> caller node)
 int launch_pack(const float* u, float* out, const int* perm, int nglob, int shots, void* stream);
 int launch_unpack(const float* in, float* u, const int* perm, int nglob, int shots, void* stream);

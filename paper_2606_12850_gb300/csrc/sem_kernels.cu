@@ -5,6 +5,7 @@
 #include <cmath>
 
 #include "sem_internal.h"
+#include "sem_newmark.cuh"
 
 namespace semgb {
 
@@ -18,7 +19,7 @@ namespace semgb {
   int launch_patch_forces_##n(const PatchLaunch& L, void* stream);                                        \
   int launch_group_sweep_##n(const GroupLaunch& L, void* stream);                                         \
   void patch_shape_##n(PatchShape* out);                                                                  \
-  void patch_layout_##n(int* es, int* ts, int* e);                                                        \
+  void patch_layout_##n(PatchLayout* out);                                                                \
   int launch_sensitivity_##n(const float* rec, const int* perm, const float* lam, const float* u_lo,       \
                              const float* u_mid, const float* u_hi, float* g_rho, float* g_kappa,       \
                              float* g_mu, int nspec, double c_m, double c_k, void* stream,              \
@@ -92,8 +93,8 @@ int patch_shape(int n, PatchShape* out) {
   return -1;
 }
 
-int patch_layout(int n, int* es, int* ts, int* e) {
-#define SEM_CALL(k) (patch_layout_##k(es, ts, e), 0)
+int patch_layout(int n, PatchLayout* out) {
+#define SEM_CALL(k) (patch_layout_##k(out), 0)
   SEM_ORDER_SWITCH(n, SEM_CALL)
 #undef SEM_CALL
   return -1;
@@ -113,9 +114,12 @@ int forces_elements_per_cta(int n) {
 
 // ---------------------------------------------------------------------------------------
 // Newmark streaming passes (Sec. I / V-C explicit second-order Newmark, diagonal mass).
-// Fields are [nglob][shots][kNodeStride] float32: one thread per (node, shot) reads one
-// float4 of each field (the 4th lane stays zero) and the node's inverse mass.
+// One thread per (node, shot) reads one float4 of each field (the 4th lane stays zero) and the
+// node's inverse mass; with several shots a block works on one shot pair, whose slots are
+// consecutive, two a node (half 1, else 0).
 // ---------------------------------------------------------------------------------------
+__device__ __forceinline__ long long block_pair() { return static_cast<long long>(blockIdx.z) * gridDim.y + blockIdx.y; }
+
 __device__ __forceinline__ float4 axpy3(float4 y, float s, float4 x) {
   return make_float4(y.x + s * x.x, y.y + s * x.y, y.z + s * x.z, 0.f);
 }
@@ -136,10 +140,14 @@ __global__ void predictor_kernel(float4* __restrict__ u, float4* __restrict__ v,
 // a_raw stays in place: the next force sweep overwrites it at each node's first touch.
 __global__ void fused_newmark_kernel(float4* __restrict__ u, float4* __restrict__ v,
                                      const float4* __restrict__ a, const float* __restrict__ minv, long long n,
-                                     int shots, float dt, float hdt, float hdt2) {
+                                     int pairs, int half, float dt, float hdt, float hdt2) {
+  if (block_pair() >= pairs) return;
+  u += block_pair() * n;
+  v += block_pair() * n;
+  a += block_pair() * n;
   for (long long g = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; g < n;
        g += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const float m = minv[g / shots];
+    const float m = minv[g >> half];
     const float4 ar = a[g], vh = v[g], ug = u[g];
     const float4 acc = make_float4(ar.x * m, ar.y * m, ar.z * m, 0.f);
     const float4 vf = axpy3(vh, hdt, acc);
@@ -150,15 +158,26 @@ __global__ void fused_newmark_kernel(float4* __restrict__ u, float4* __restrict_
 
 // Corrector alone (completes the state): a = M^-1 a_raw ; v = v_half + dt/2 a
 __global__ void corrector_kernel(float4* __restrict__ v, float4* __restrict__ a, const float* __restrict__ minv,
-                                 long long n, int shots, float hdt) {
+                                 long long n, int pairs, int half, float hdt) {
+  if (block_pair() >= pairs) return;
+  v += block_pair() * n;
+  a += block_pair() * n;
   for (long long g = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; g < n;
        g += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const float m = minv[g / shots];
+    const float m = minv[g >> half];
     const float4 ar = a[g];
     const float4 acc = make_float4(ar.x * m, ar.y * m, ar.z * m, 0.f);
     a[g] = acc;
     v[g] = axpy3(v[g], hdt, acc);
   }
+}
+
+// Blocks over the slots of a single shot or a shot pair, and the pairs.
+static int stream_grid(long long n);
+static long long pair_slots(int nglob, int shots) { return static_cast<long long>(nglob) * (shots > 1 ? 2 : 1); }
+static dim3 pair_grid(int nglob, int shots) {
+  const unsigned pairs = static_cast<unsigned>((shots + 1) / 2), y = pairs < 32768u ? pairs : 32768u;
+  return dim3(stream_grid(pair_slots(nglob, shots)), y, (pairs + y - 1) / y);
 }
 
 static int stream_grid(long long n) {
@@ -167,7 +186,7 @@ static int stream_grid(long long n) {
 }
 
 int launch_predictor(const DevProblem& p, void* stream) {
-  const long long n = static_cast<long long>(p.nglob) * p.shots;
+  const long long n = static_cast<long long>(p.nglob) * padded_shots(p.shots);
   predictor_kernel<<<stream_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
       reinterpret_cast<float4*>(p.u), reinterpret_cast<float4*>(p.v), reinterpret_cast<const float4*>(p.a), n,
       static_cast<float>(p.dt), static_cast<float>(0.5 * p.dt), static_cast<float>(0.5 * p.dt * p.dt));
@@ -175,19 +194,117 @@ int launch_predictor(const DevProblem& p, void* stream) {
 }
 
 int launch_fused_newmark(const DevProblem& p, void* stream) {
-  const long long n = static_cast<long long>(p.nglob) * p.shots;
-  fused_newmark_kernel<<<stream_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+  fused_newmark_kernel<<<pair_grid(p.nglob, p.shots), 256, 0, static_cast<cudaStream_t>(stream)>>>(
       reinterpret_cast<float4*>(p.u), reinterpret_cast<float4*>(p.v), reinterpret_cast<const float4*>(p.a), p.minv,
-      n, p.shots, static_cast<float>(p.dt), static_cast<float>(0.5 * p.dt), static_cast<float>(0.5 * p.dt * p.dt));
+      pair_slots(p.nglob, p.shots), (p.shots + 1) / 2, p.shots > 1, static_cast<float>(p.dt), static_cast<float>(0.5 * p.dt), static_cast<float>(0.5 * p.dt * p.dt));
   return static_cast<int>(cudaGetLastError());
 }
 
 int launch_corrector(const DevProblem& p, void* stream) {
-  const long long n = static_cast<long long>(p.nglob) * p.shots;
-  corrector_kernel<<<stream_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      reinterpret_cast<float4*>(p.v), reinterpret_cast<float4*>(p.a), p.minv, n, p.shots,
-      static_cast<float>(0.5 * p.dt));
+  corrector_kernel<<<pair_grid(p.nglob, p.shots), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      reinterpret_cast<float4*>(p.v), reinterpret_cast<float4*>(p.a), p.minv, pair_slots(p.nglob, p.shots),
+      (p.shots + 1) / 2, p.shots > 1, static_cast<float>(0.5 * p.dt));
   return static_cast<int>(cudaGetLastError());
+}
+
+// ---------------------------------------------------------------------------------------
+// The rim pass (Sec. IV-C assembly without colours or atomics): one thread per (rim node,
+// shot) adds the partial sums the node's patches left, in sweep order, and does with the
+// force what the sweep did at the inner nodes. The node's entry names up to four partials, so
+// a face or edge node needs one dependent load before its partials; rim nodes are the last
+// internal ids, so the fields stream, and neighbouring nodes of a face have neighbouring
+// partials. The entry and the node's state, which no sweep writes at the rim, are loaded
+// while the sweep drains. Bound by DRAM: 119 bytes a rim node (entry, partials, u, v, 1/M read,
+// u, v written), 56 us for the 2.8 M rim nodes of a 48^3 mesh at NGLL 5, 6.0 TB/s.
+// ---------------------------------------------------------------------------------------
+template <bool MS, int NM>
+__global__ void __launch_bounds__(256) rim_combine_kernel(const RimLaunch R) {
+  const long long idx = blockIdx.x * 256ll + threadIdx.x;
+  const int t = static_cast<int>(MS ? idx >> 1 : idx);
+  const int shot = MS ? 2 * static_cast<int>(block_pair()) + static_cast<int>(idx & 1) : 0;
+  const bool in = t < R.nrim && (!MS || shot < R.shots);
+  SweepNewmark nm = R.nm;
+  float4* f = reinterpret_cast<float4*>(R.f);
+  const float4* __restrict__ part = reinterpret_cast<const float4*>(R.partials);
+  if constexpr (MS) {
+    const size_t slot = field_slot(nm.nglob, 2, 0, shot);
+    move_fields(nm, slot);
+    f += slot;
+    part += field_slot(nm.nsums, 2, 0, shot);
+  }
+  const uint32_t node = static_cast<uint32_t>(R.ninner + (in ? t : 0));
+  int4 q = make_int4(-1, -1, -1, -1);
+  NodeState st;
+  RimBlock blk{0, 0, 0, 0};
+  if (in) {
+    q = __ldg(reinterpret_cast<const int4*>(R.rim) + t);
+    if constexpr (NM == 1 || NM == 2 || NM == 3) {
+      load_node_state<MS, NM>(nm, node, st);
+      blk = R.blocks[t / kRimBlock];
+    }
+  }
+  wait_prerequisite_grid();
+  allow_dependent_grid();
+  if (!in) return;
+  constexpr int S = MS ? 2 : 1;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 p0 = __ldcg(part + static_cast<size_t>(q.x) * S);
+  const float4 p1 = __ldcg(part + static_cast<size_t>(q.y) * S);
+  const float4 p2 = q.z >= 0 ? __ldcg(part + static_cast<size_t>(q.z) * S) : zero;
+  const float4 p3 = q.w >= 0 ? __ldcg(part + static_cast<size_t>(q.w) * S) : zero;
+  float fx = p0.x + p1.x, fy = p0.y + p1.y, fz = p0.z + p1.z;
+  if (q.z >= 0) {
+    fx += p2.x;
+    fy += p2.y;
+    fz += p2.z;
+  }
+  if (q.w >= 0) {
+    fx += p3.x;
+    fy += p3.y;
+    fz += p3.z;
+  } else if (q.w <= -2) {
+    const int* __restrict__ o = R.over + (-2 - q.w);
+    const int n = __ldg(o);
+    for (int k = 1; k <= n; ++k) {
+      const float4 p = __ldcg(part + static_cast<size_t>(__ldg(o + k)) * S);
+      fx += p.x;
+      fy += p.y;
+      fz += p.z;
+    }
+  }
+  complete_node<MS, NM>(nm, f, node, shot, st, nm.rim_src + blk.src_off, blk.nsrc, nm.rim_recv + blk.rec_off, blk.nrec,
+                        fx, fy, fz);
+}
+
+template <bool MS, int NM>
+static int launch_rim(const RimLaunch& R, cudaStream_t s) {
+  const long long n = static_cast<long long>(R.nrim) * (MS ? 2 : 1);
+  cudaLaunchConfig_t cfg = {};
+  const unsigned pairs = MS ? (R.shots + 1) / 2 : 1, y = pairs < 32768u ? pairs : 32768u;
+  cfg.gridDim = dim3(static_cast<unsigned>((n + 255) / 256), y, (pairs + y - 1) / y);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return static_cast<int>(cudaLaunchKernelEx(&cfg, rim_combine_kernel<MS, NM>, R));
+}
+
+int launch_rim_combine(const RimLaunch& R, void* stream) {
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (R.nrim <= 0) return 0;
+  if (R.shots > 1) {
+    if (R.nm.mode > 2) return static_cast<int>(cudaErrorInvalidValue);
+    return R.nm.mode ? launch_rim<true, 1>(R, s) : launch_rim<true, 0>(R, s);
+  }
+  switch (R.nm.mode) {
+    case 0: return launch_rim<false, 0>(R, s);
+    case 3: return launch_rim<false, 2>(R, s);
+    case 4: return launch_rim<false, 4>(R, s);
+    default: return R.nm.snap ? launch_rim<false, 3>(R, s) : launch_rim<false, 1>(R, s);
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -323,8 +440,8 @@ __global__ void material_records_kernel(MaterialLaunch m) {
     float* r = m.rec + s * RW;
     const int qq = i * n * n + j + n * k;
     const double J = r[kJac * np + qq];
-    r[kJKappa * np + qq] = static_cast<float>(J * kappa);
-    r[kJMu * np + qq] = static_cast<float>(J * mu);
+    r[rec_at(np, 9, qq)] = static_cast<float>(J * kappa);
+    r[rec_at(np, 10, qq)] = static_cast<float>(J * mu);
   }
 }
 
@@ -386,16 +503,24 @@ int launch_material_apply(const MaterialLaunch& m, const int* sweep_off, int nra
   return static_cast<int>(cudaGetLastError());
 }
 
-// Layout changes between the solver's fields [nglob][shots][4] (internal node order) and the
-// caller's arrays [shots][nglob][3] (caller node order through perm, or internal order when
+// Layout changes between the solver's fields (internal node order) and the caller's arrays [shots][nglob][3] (caller node order through perm, or internal order when
 // perm is null): state copies, displacement snapshots. One thread per (node, shot).
-__global__ void pack_kernel(const float4* __restrict__ u, float* __restrict__ out, const int* __restrict__ perm,
-                            long long nglob, int shots) {
-  const long long n = nglob * shots;
+// Node and shot of slot t of the calling block's shot (pair); false for the slot past an odd
+// last shot.
+__device__ __forceinline__ bool slot_of(long long t, int shots, long long* node, long long* shot) {
+  *node = shots > 1 ? t >> 1 : t;
+  *shot = shots > 1 ? 2 * block_pair() + (t & 1) : 0;
+  return *shot < shots;
+}
+
+__device__ __forceinline__ void pack_slots(const float4* __restrict__ u, float* __restrict__ out,
+                                           const int* __restrict__ perm, long long nglob, int shots) {
+  const long long n = nglob * (shots > 1 ? 2 : 1);
+  u += block_pair() * n;
   for (long long t = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; t < n;
        t += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long g = shots == 1 ? t : t / shots;
-    const long long sh = t - g * shots;
+    long long g, sh;
+    if (!slot_of(t, shots, &g, &sh)) continue;
     const float4 v = u[t];
     float* o = out + 3 * (sh * nglob + (perm ? perm[g] : g));
     o[0] = v.x;
@@ -404,98 +529,86 @@ __global__ void pack_kernel(const float4* __restrict__ u, float* __restrict__ ou
   }
 }
 
+__global__ void pack_kernel(const float4* __restrict__ u, float* __restrict__ out, const int* __restrict__ perm,
+                            long long nglob, int shots) {
+  pack_slots(u, out, perm, nglob, shots);
+}
+
 __global__ void unpack_kernel(const float* __restrict__ in, float4* __restrict__ u, const int* __restrict__ perm,
                               long long nglob, int shots) {
-  const long long n = nglob * shots;
+  const long long n = nglob * (shots > 1 ? 2 : 1);
+  u += block_pair() * n;
   for (long long t = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; t < n;
        t += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long g = shots == 1 ? t : t / shots;
-    const long long sh = t - g * shots;
+    long long g, sh;
+    if (!slot_of(t, shots, &g, &sh)) continue;
     const float* i = in + 3 * (sh * nglob + (perm ? perm[g] : g));
     u[t] = make_float4(i[0], i[1], i[2], 0.f);
   }
 }
 
 int launch_pack(const float* u, float* out, const int* perm, int nglob, int shots, void* stream) {
-  const long long n = static_cast<long long>(nglob) * shots;
-  if (n == 0) return 0;
-  pack_kernel<<<stream_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(reinterpret_cast<const float4*>(u), out,
-                                                                             perm, nglob, shots);
+  if (nglob <= 0) return 0;
+  pack_kernel<<<pair_grid(nglob, shots), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      reinterpret_cast<const float4*>(u), out, perm, nglob, shots);
   return static_cast<int>(cudaGetLastError());
 }
 
 int launch_unpack(const float* in, float* u, const int* perm, int nglob, int shots, void* stream) {
-  const long long n = static_cast<long long>(nglob) * shots;
-  if (n == 0) return 0;
-  unpack_kernel<<<stream_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(in, reinterpret_cast<float4*>(u),
-                                                                               perm, nglob, shots);
+  if (nglob <= 0) return 0;
+  unpack_kernel<<<pair_grid(nglob, shots), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      in, reinterpret_cast<float4*>(u), perm, nglob, shots);
   return static_cast<int>(cudaGetLastError());
 }
 
 // ---------------------------------------------------------------------------------------
-// Sources and receivers (Sec. V-C): Ricker point forces added to a_raw at t_{n+1}, then the
-// displacement u^{n+1} sampled at the receiver nodes; advances the device step counter.
-// Source nodes are distinct (the host merges duplicates), so the adds do not race.
+// Sources and receivers (Sec. V-C): Ricker point forces added to a_raw at t_{n+1} (the first
+// block), then the displacement u^{n+1} sampled at the receiver nodes, one thread per receiver
+// and shot; n is the device step counter plus the steps enqueued since it was written. Source
+// nodes are distinct (the host merges duplicates), so the adds do not race.
 // ---------------------------------------------------------------------------------------
-__global__ void sources_record_kernel(float* __restrict__ a, const float* __restrict__ u, DevCtl* ctl, int shots,
-                                      int nsrc, const int* __restrict__ src_node, const int* __restrict__ src_shot,
-                                      const double* __restrict__ src_force, double f0, double t0, double dt,
-                                      int nrec, const int* __restrict__ rec_node) {
-  const long long n = ctl->step;
-  const int col = ctl->col;
-  const int ncols = ctl->ncols;
-  float* seis = ctl->seis;
-  __syncthreads();
-  const double tau = static_cast<double>(n + 1) * dt - t0;
-  const double x = M_PI * f0 * tau;
-  const double aa = x * x;
-  const double R = (1.0 - 2.0 * aa) * exp(-aa);
-  for (int s = threadIdx.x; s < nsrc; s += blockDim.x) {
-    const size_t g = kNodeStride * (static_cast<size_t>(src_node[s]) * shots + src_shot[s]);
-    a[g] += static_cast<float>(src_force[3 * s] * R);
-    a[g + 1] += static_cast<float>(src_force[3 * s + 1] * R);
-    a[g + 2] += static_cast<float>(src_force[3 * s + 2] * R);
-  }
-  if (seis != nullptr && col < ncols) {  // seis [shots][nrec][3][ncols]
-    for (int q = threadIdx.x; q < 3 * nrec * shots; q += blockDim.x) {
-      const int sh = q / (3 * nrec);
-      const int rq = q - sh * 3 * nrec;
-      const int r = rq / 3, c = rq - 3 * r;
-      seis[static_cast<size_t>(q) * ncols + col] =
-          u[kNodeStride * (static_cast<size_t>(rec_node[r]) * shots + sh) + c];
+__global__ void sources_record_kernel(float* __restrict__ a, const float4* __restrict__ u,
+                                      const DevCtl* __restrict__ ctl, int ahead, int nglob, int shots, int nsrc,
+                                      const int* __restrict__ src_node, const int* __restrict__ src_shot,
+                                      const double* __restrict__ src_force, double f0, double t0, double dt, int nrec,
+                                      const int* __restrict__ rec_node) {
+  if (blockIdx.x == 0 && nsrc > 0) {
+    const double tau = static_cast<double>(ctl->step + ahead + 1) * dt - t0;
+    const double x = M_PI * f0 * tau;
+    const double aa = x * x;
+    const double R = (1.0 - 2.0 * aa) * exp(-aa);
+    for (int s = threadIdx.x; s < nsrc; s += blockDim.x) {
+      const size_t g = kNodeStride * field_slot(nglob, shots, src_node[s], src_shot[s]);
+      a[g] += static_cast<float>(src_force[3 * s] * R);
+      a[g + 1] += static_cast<float>(src_force[3 * s + 1] * R);
+      a[g + 2] += static_cast<float>(src_force[3 * s + 2] * R);
     }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ctl->step = n + 1;
-    ctl->col = col + 1;
+  const int col = ctl->col + ahead, ncols = ctl->ncols;
+  float* seis = ctl->seis;
+  if (seis == nullptr || col >= ncols) return;  // seis [shots][nrec][3][ncols]
+  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nrec * shots; q += gridDim.x * blockDim.x) {
+    const int r = q / shots, sh = q - r * shots;
+    const float4 x = u[field_slot(nglob, shots, rec_node[r], sh)];
+    float* o = seis + (static_cast<size_t>(sh) * nrec + r) * 3 * ncols + col;
+    o[0] = x.x;
+    o[ncols] = x.y;
+    o[2 * static_cast<size_t>(ncols)] = x.z;
   }
 }
 
 // pack_kernel into the snapshot slot the step counter names (graph-replayable)
-__global__ void snapshot_kernel(const float4* __restrict__ u, const DevCtl* __restrict__ ctl,
+__global__ void snapshot_kernel(const float4* __restrict__ u, const DevCtl* __restrict__ ctl, int ahead,
                                 const int* __restrict__ perm, long long nglob, int shots) {
   float* base = ctl->snap;
   if (!base) return;
-  float* out = base + static_cast<long long>(ctl->col - 1) * ctl->snap_per;
-  const long long n = nglob * shots;
-  for (long long t = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; t < n;
-       t += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const long long g = shots == 1 ? t : t / shots;
-    const long long sh = t - g * shots;
-    const float4 v = u[t];
-    float* o = out + 3 * (sh * nglob + (perm ? perm[g] : g));
-    o[0] = v.x;
-    o[1] = v.y;
-    o[2] = v.z;
-  }
+  pack_slots(u, base + static_cast<long long>(ctl->col + ahead) * ctl->snap_per, perm, nglob, shots);
 }
 
-int launch_snapshot(const float* u, DevCtl* ctl, const int* perm, int nglob, int shots, void* stream) {
-  const long long n = static_cast<long long>(nglob) * shots;
-  if (n == 0) return 0;
-  snapshot_kernel<<<stream_grid(n), 256, 0, static_cast<cudaStream_t>(stream)>>>(reinterpret_cast<const float4*>(u),
-                                                                                 ctl, perm, nglob, shots);
+int launch_snapshot(const float* u, const DevCtl* ctl, int ahead, const int* perm, int nglob, int shots, void* stream) {
+  if (nglob <= 0) return 0;
+  snapshot_kernel<<<pair_grid(nglob, shots), 256, 0, static_cast<cudaStream_t>(stream)>>>(reinterpret_cast<const float4*>(u),
+                                                                                 ctl, ahead, perm, nglob, shots);
   return static_cast<int>(cudaGetLastError());
 }
 
@@ -509,15 +622,28 @@ __global__ void set_ctl_kernel(DevCtl* ctl, long long step, int ncols, float* se
   ctl->snap_per = snap_per;
 }
 
+__global__ void advance_ctl_kernel(DevCtl* ctl, int steps) {
+  ctl->step += steps;
+  ctl->col += steps;
+}
+
+int launch_advance_ctl(DevCtl* ctl, int steps, void* stream) {
+  advance_ctl_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(ctl, steps);
+  return static_cast<int>(cudaGetLastError());
+}
+
 int launch_set_ctl(DevCtl* ctl, long long step, int ncols, float* seis, void* stream, float* snap,
                    long long snap_per) {
   set_ctl_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(ctl, step, ncols, seis, snap, snap_per);
   return static_cast<int>(cudaGetLastError());
 }
 
-int launch_sources_record(const DevProblem& p, void* stream) {
-  sources_record_kernel<<<1, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      p.a, p.u, p.ctl, p.shots, p.nsrc, p.src_node, p.src_shot, p.src_force, p.f0, p.t0, p.dt, p.nrec, p.rec_node);
+int launch_sources_record(const DevProblem& p, int ahead, void* stream) {
+  const long long n = static_cast<long long>(p.nrec) * p.shots;
+  const int grid = static_cast<int>(n < 256 ? 1 : (n + 255) / 256 > 608 ? 608 : (n + 255) / 256);
+  sources_record_kernel<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(
+      p.a, reinterpret_cast<const float4*>(p.u), p.ctl, ahead, p.nglob, p.shots, p.nsrc, p.src_node, p.src_shot, p.src_force,
+      p.f0, p.t0, p.dt, p.nrec, p.rec_node);
   return static_cast<int>(cudaGetLastError());
 }
 
@@ -538,7 +664,7 @@ __global__ void nonfinite_kernel(const float4* __restrict__ u, const float4* __r
 }
 
 int launch_nonfinite_check(const DevProblem& p, int* flag, void* stream) {
-  const int n = p.nglob * p.shots;
+  const int n = p.nglob * padded_shots(p.shots);
   nonfinite_kernel<<<kEnergyBlocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
       reinterpret_cast<const float4*>(p.u), reinterpret_cast<const float4*>(p.v),
       reinterpret_cast<const float4*>(p.a), n, flag);
@@ -553,10 +679,10 @@ __global__ void energy_partials_kernel(const float4* __restrict__ u, const float
                                        int shots, double* __restrict__ partials) {
   __shared__ double sk[256], sp[256];
   double kin = 0.0, pot = 0.0;
-  const long long n = static_cast<long long>(nglob) * shots;
+  const long long n = static_cast<long long>(nglob) * padded_shots(shots);
   for (long long g = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; g < n;
        g += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const float m = minv[g / shots];
+    const float m = minv[shots == 1 ? g : (g >> 1) % nglob];
     const float4 vg = v[g], ug = u[g], fg = f[g];
     const double vx = vg.x, vy = vg.y, vz = vg.z;
     kin += (vx * vx + vy * vy + vz * vz) / static_cast<double>(m);

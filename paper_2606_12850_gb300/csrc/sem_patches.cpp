@@ -19,7 +19,8 @@
 //      order, points in natural order), the patch-local index of every local point and,
 //      per patch node, the list of local points that meet there; patches with the same
 //      local structure share one table (every interior brick of a structured mesh does);
-//   5. an internal numbering of the nodes in which every patch finds its nodes in runs.
+//   5. an internal numbering of the nodes: inner nodes (of one patch) first, then the rim
+//      nodes (shared by patches), so that every patch finds its nodes in runs.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -355,22 +356,36 @@ int build_patches(int nspec, int n, int nglob, const int32_t* ibool, const Patch
     out.table_of.push_back(tid);
   }
 
-  // 5. internal node numbering: the nodes a patch touches first (in sweep order) get the
-  //    next consecutive ids, grouped by the set of patches that share them (the patch's own
-  //    interior, then each shared face, edge and corner group together, so that the
-  //    neighbours that read them find them in runs), in first appearance order inside a
-  //    group
+  // 5. internal node numbering: first the inner nodes (touched by one patch only), patch after
+  //    patch in sweep order and in a patch the ones met by one local point first, then the rim
+  //    nodes (shared by patches): those a patch touches
+  //    first get the next consecutive ids, grouped by the set of patches that share them
+  //    (each face, edge and corner group together, so that the neighbours that read them
+  //    find them in runs). First appearance order inside a patch or group.
   {
     std::vector<int> sweep_pos(npatch);
     for (int s2 = 0; s2 < npatch; ++s2) sweep_pos[porder[s2]] = s2;
     out.node_new.assign(nglob, -1);
     int next = 0;
+    for (int s2 = 0; s2 < npatch; ++s2) {
+      // per patch node, whether several of the patch's local points meet there
+      const int t0 = out.node_off[s2], nn = out.node_off[s2 + 1] - t0, tab = out.table_of[s2];
+      std::vector<int> met(nn, 0);
+      for (int q = 0; q < out.tab_nelem[tab] * np; ++q) ++met[out.lid[static_cast<size_t>(out.tab_lid_off[tab]) + q]];
+      for (int several = 0; several < 2; ++several)
+        for (int t = 0; t < nn; ++t) {
+          const int g = static_cast<int>(out.nodes[t0 + t] & ~kFirstTouchBit);
+          if (pcount[g + 1] - pcount[g] == 1 && (met[t] > 1) == (several == 1)) out.node_new[g] = next++;
+        }
+    }
+    out.ninner = next;
     std::vector<std::pair<std::vector<int>, int>> keyed;  // (sharers in sweep order, appearance)
     for (int s2 = 0; s2 < npatch; ++s2) {
       keyed.clear();
       for (int t = out.node_off[s2]; t < out.node_off[s2 + 1]; ++t) {
         if (!(out.nodes[t] & kFirstTouchBit)) continue;
         const int g = static_cast<int>(out.nodes[t] & ~kFirstTouchBit);
+        if (out.node_new[g] >= 0) continue;
         std::vector<int> sh;
         for (int q = pcount[g]; q < pcount[g + 1]; ++q) sh.push_back(sweep_pos[patches_of[q]]);
         std::sort(sh.begin(), sh.end());
