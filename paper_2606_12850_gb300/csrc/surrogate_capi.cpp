@@ -36,6 +36,14 @@ struct sg_model {
   bf16* d_pack = nullptr;  // the convolutions' weights packed for the tcgen05 kernel
   float* d_red = nullptr;  // per-slice sums of the bias gradients
   sgk::Products prod;    // product kernel (SG_OPT_PRODUCT) and d_err
+  // packed forward (kind 1, sizes that fit it): weights and activations in the tensor cores' layout
+  bool packed = false;
+  int Bp = 0;              // max_batch rounded up to whole tiles
+  bf16* d_wp = nullptr;    // packed weights
+  size_t pW1 = 0, pW2 = 0, pW3 = 0;
+  std::vector<size_t> pC;
+  bf16 *d_h1p = nullptr, *d_h2p = nullptr;
+  std::vector<bf16*> d_zp;  // input of every stage
   long long step = 0;
   size_t dev_bytes = 0;
   std::vector<void*> allocs;
@@ -88,6 +96,51 @@ int check_products(sg_model* m, const char* where) {
   if (h == 0) return SG_OK;
   SG_CUDA(m, cudaMemset(m->d_err, 0, sizeof(int)));
   return sg_fail(m, SEM_ETIMEOUT, std::string(where) + ": a tensor-core product timed out waiting for its MMAs");
+}
+
+// Whether the sizes fit the packed forward kernels (64-feature and 32-channel granules, weights
+// resident in shared memory, a contracted last stage); else the general kernels run.
+bool packed_sizes(const sg_model* m) {
+  if (!sgk::packed_dense_ok(m->in_dim, m->hidden) || !sgk::packed_dense_ok(m->hidden, m->hidden) ||
+      !sgk::packed_dense_ok(m->hidden, m->c0 * m->l0) || m->contract < 1 || m->up.back() != 1 || m->out_c % 32 != 0)
+    return false;
+  for (int st = 0; st < m->nstages; ++st) {
+    const int n = st + 1 < m->nstages ? m->cout[st] : 32 * m->contract;
+    if (!sgk::packed_conv_ok(m->cin[st], n, m->up[st])) return false;
+  }
+  return true;
+}
+
+// The packed copies of the bfloat16 weights, after they changed.
+int pack_weights(sg_model* m) {
+  if (!m->packed) return SG_OK;
+  cudaStream_t s = m->stream;
+  SG_LAUNCH(m, sgk::pack_dense(m->in_dim, m->hidden, 0, m->d_pb + m->oW1, m->d_wp + m->pW1, s));
+  SG_LAUNCH(m, sgk::pack_dense(m->hidden, m->hidden, 0, m->d_pb + m->oW2, m->d_wp + m->pW2, s));
+  SG_LAUNCH(m, sgk::pack_dense(m->hidden, m->c0 * m->l0, m->l0, m->d_pb + m->oW3, m->d_wp + m->pW3, s));
+  for (int st = 0; st < m->nstages; ++st) {
+    const bool last = st + 1 == m->nstages;
+    SG_LAUNCH(m, sgk::pack_conv(m->cin[st], last ? 32 * m->contract : m->cout[st], last ? m->out_c / 32 : 1,
+                                last ? m->out_c : 0, m->d_pb + m->oC[st], m->d_wp + m->pC[st], s));
+  }
+  return SG_OK;
+}
+
+int forward_packed(sg_model* m, int b, const float* x, float* y) {
+  cudaStream_t s = m->stream;
+  SG_LAUNCH(m, sgk::packed_dense(b, m->Bp, m->in_dim, m->hidden, x, nullptr, m->d_wp + m->pW1, m->d_p + m->ob1,
+                                 m->d_h1p, nullptr, 0, m->prod, s));
+  SG_LAUNCH(m, sgk::packed_dense(b, m->Bp, m->hidden, m->hidden, nullptr, m->d_h1p, m->d_wp + m->pW2, m->d_p + m->ob2,
+                                 m->d_h2p, nullptr, 0, m->prod, s));
+  SG_LAUNCH(m, sgk::packed_dense(b, m->Bp, m->hidden, m->c0 * m->l0, nullptr, m->d_h2p, m->d_wp + m->pW3,
+                                 m->d_p + m->ob3, m->d_zp[0], nullptr, m->l0, m->prod, s));
+  const int last = m->nstages - 1;
+  for (int st = 0; st < last; ++st)
+    SG_LAUNCH(m, sgk::packed_conv(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], m->d_zp[st], m->d_wp + m->pC[st],
+                                  m->d_p + m->oc[st], m->d_zp[st + 1], nullptr, m->prod, s));
+  SG_LAUNCH(m, sgk::packed_conv_contract(b, m->cin[last], m->contract, m->out_c, m->lin[last], m->in_dim,
+                                         m->d_zp[last], m->d_wp + m->pC[last], m->d_p + m->oc[last], x, y, m->prod, s));
+  return SG_OK;
 }
 
 int forward_chunk(sg_model* m, int b, const float* x, float* y_last) {
@@ -222,6 +275,33 @@ int sg_create(sg_model** out, int device, void* stream, int in_dim, int hidden, 
     r = sg_alloc(m, &m->d_pre[st], n);
     if (r == SG_OK && st + 1 < nstages) r = sg_alloc(m, &m->d_out[st], n);
   }
+  m->packed = packed_sizes(m);
+  if (r == SG_OK && m->packed) {
+    m->Bp = (max_batch + 127) / 128 * 128;
+    size_t w = 0;
+    m->pW1 = w; w += sgk::packed_dense_elems(in_dim, hidden);
+    m->pW2 = w; w += sgk::packed_dense_elems(hidden, hidden);
+    m->pW3 = w; w += sgk::packed_dense_elems(hidden, c0 * l0);
+    for (int st = 0; st < nstages; ++st) {
+      m->pC.push_back(w);
+      w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
+    }
+    const size_t h = static_cast<size_t>(hidden) * m->Bp;
+    r = sg_alloc(m, &m->d_wp, w);
+    if (r == SG_OK) r = sg_alloc(m, &m->d_h1p, h);
+    if (r == SG_OK) r = sg_alloc(m, &m->d_h2p, h);
+    cudaError_t z = r == SG_OK ? cudaMemsetAsync(m->d_wp, 0, w * sizeof(bf16), m->stream) : cudaSuccess;
+    if (r == SG_OK && z == cudaSuccess) z = cudaMemsetAsync(m->d_h1p, 0, h * sizeof(bf16), m->stream);
+    if (r == SG_OK && z == cudaSuccess) z = cudaMemsetAsync(m->d_h2p, 0, h * sizeof(bf16), m->stream);
+    for (int st = 0; st < nstages && r == SG_OK && z == cudaSuccess; ++st) {  // zero rows pad the time axis
+      bf16* q = nullptr;
+      const size_t n = B * m->cin[st] * sgk::packed_rows(m->lin[st]);
+      r = sg_alloc(m, &q, n);
+      m->d_zp.push_back(q);
+      if (r == SG_OK) z = cudaMemsetAsync(q, 0, n * sizeof(bf16), m->stream);
+    }
+    if (z != cudaSuccess) r = sg_fail(m, SEM_ECUDA, std::string("sg_create: ") + cudaGetErrorString(z));
+  }
   if (r == SG_OK) {
     const size_t bytes = m->P * sizeof(float);
     cudaError_t z = cudaSuccess;
@@ -276,6 +356,7 @@ int sg_set_params(sg_model* m, const float* params) {
   SG_CUDA(m, cudaMemsetAsync(m->d_m, 0, m->P * sizeof(float), m->stream));
   SG_CUDA(m, cudaMemsetAsync(m->d_v, 0, m->P * sizeof(float), m->stream));
   SG_LAUNCH(m, sgk::to_bf16(m->P, m->d_p, m->d_pb, m->stream));
+  if (int r = pack_weights(m)) return r;
   SG_CUDA(m, cudaStreamSynchronize(m->stream));
   m->step = 0;
   return SG_OK;
@@ -304,7 +385,9 @@ int sg_forward(sg_model* m, int batch, const float* x, float* y) {
   const size_t per_out = static_cast<size_t>(m->out_c) * m->out_l;
   for (int b0 = 0; b0 < batch; b0 += m->max_batch) {
     const int b = std::min(m->max_batch, batch - b0);
-    int r = forward_chunk(m, b, x + static_cast<size_t>(b0) * m->in_dim, y + b0 * per_out);
+    const float* xb = x + static_cast<size_t>(b0) * m->in_dim;
+    const int r = m->packed && m->prod.kind == 1 ? forward_packed(m, b, xb, y + b0 * per_out)
+                                                 : forward_chunk(m, b, xb, y + b0 * per_out);
     if (r) return r;
   }
   return SG_OK;
@@ -370,7 +453,7 @@ int sg_adam_step(sg_model* m, float lr, float beta1, float beta2, float eps) {
   const double c2 = 1.0 - std::pow(static_cast<double>(beta2), static_cast<double>(m->step));
   SG_LAUNCH(m, sgk::adam_update(m->P, m->d_p, m->d_g, m->d_m, m->d_v, m->d_pb, lr, beta1, beta2, eps,
                                 static_cast<float>(1.0 / c1), static_cast<float>(1.0 / c2), m->stream));
-  return SG_OK;
+  return pack_weights(m);
 }
 
 int sg_sync(sg_model* m) {

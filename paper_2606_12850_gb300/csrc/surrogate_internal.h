@@ -72,4 +72,25 @@ int contract_forward(int B, int K, int C, int L, int in_dim, const float* x, con
 int contract_backward(int B, int K, int C, int L, int in_dim, const float* x, const float* dy, float* dD,
                       cudaStream_t s);
 
+// ---- packed forward (surrogate_packed.cu): bfloat16 activations in the tensor cores' layout ----
+// rows of a packed time axis of L samples (one zero row before, zeros after)
+int packed_rows(int L);
+bool packed_dense_ok(int K, int N);
+bool packed_conv_ok(int Ci, int N, int up);
+size_t packed_dense_elems(int K, int N);  // packed weights of a dense layer
+// W [N][K] -> packed; l0 > 0: the layer feeds a convolution of N / l0 channels
+int pack_dense(int K, int N, int l0, const bf16* W, bf16* Wp, cudaStream_t s);
+// W [Co][Ci][3] -> packed blocks of N rows; outC > 0: contracted copies of 32 channels a block
+int pack_conv(int Ci, int N, int blocks, int outC, const bf16* W, bf16* Wp, cudaStream_t s);
+// out = gelu(x W^T + b), from x [B][K] (or, x null, packed [K/8][Bp][8]) to packed [N/8][Bp][8]
+// (or, l0 > 0, [B][N/l0/8][packed_rows(l0)][8]); pre (or null) [B][N]
+int packed_dense(int B, int Bp, int K, int N, const float* x, const bf16* in, const bf16* Wp, const float* bias,
+                 bf16* out, float* pre, int l0, const Products& pr, cudaStream_t s);
+// hidden convolution, packed to packed; pre (or null) [B][N][up Lin]
+int packed_conv(int B, int Ci, int N, int Lin, int up, const bf16* in, const bf16* Wp, const float* bias, bf16* out,
+                float* pre, const Products& pr, cudaStream_t s);
+// the last convolution (K outC channels, no upsampling) and its contraction with x: y [B][outC][Lin]
+int packed_conv_contract(int B, int Ci, int K, int outC, int Lin, int in_dim, const bf16* in, const bf16* Wp,
+                         const float* bias, const float* x, float* y, const Products& pr, cudaStream_t s);
+
 }  // namespace sgk

@@ -13,22 +13,12 @@
 #include <cstdint>
 
 #include "surrogate_internal.h"
+#include "surrogate_tc.cuh"
 
 namespace sgk {
 namespace {
 
 constexpr int BN = 64;
-constexpr float kGeluC = 0.7978845608028654f;  // sqrt(2 / pi)
-constexpr float kGeluA = 0.044715f;
-
-__device__ __forceinline__ float gelu(float x) {
-  return 0.5f * x * (1.f + tanhf(kGeluC * (x + kGeluA * x * x * x)));
-}
-__device__ __forceinline__ float gelu_grad(float x) {
-  const float t = tanhf(kGeluC * (x + kGeluA * x * x * x));
-  return 0.5f * (1.f + t) + 0.5f * x * (1.f - t * t) * kGeluC * (1.f + 3.f * kGeluA * x * x);
-}
-
 // C[m][n] = sum_k A(m, k) B(k, n) over k in this CTA's split, on the tensor cores: the
 // loader functors (kAlong: which index is contiguous in memory, so that consecutive threads
 // load consecutive words) read float32 operands, which are rounded to bfloat16 (nearest
@@ -158,7 +148,6 @@ constexpr int TC_EPI_LD = TC_BN + 1;                         // floats per stage
 // operand stages, then (reused) the epilogue's output tile; 3 CTAs a SM (3 x 128 TMEM columns)
 constexpr int TC_DATA = (TC_STAGES * TC_STAGE > TC_BM * TC_EPI_LD * 4 ? TC_STAGES * TC_STAGE : TC_BM * TC_EPI_LD * 4);
 constexpr int TC_SMEM = TC_DATA + 64;                        // + mbarriers and the TMEM address
-constexpr unsigned long long kTcWaitNs = 2000000000ull;      // 2 s
 static_assert(TC_STAGES * TC_STAGE <= TC_DATA && TC_BM * TC_EPI_LD * 4 <= TC_DATA, "shared memory plan");
 static_assert(TC_GROUPS == 2 * (TC_THREADS / 32) && TC_BN / 2 % 32 == 0, "tile plan: two row groups a warp");
 
@@ -167,34 +156,6 @@ static_assert(TC_GROUPS == 2 * (TC_THREADS / 32) && TC_BN / 2 % 32 == 0, "tile p
 // bits 24-28.
 constexpr uint32_t kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(TC_BN >> 3) << 17) |
                               (static_cast<uint32_t>(TC_BM >> 4) << 24);
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Waits for the phase of the given parity to complete; false after limit_ns.
-__device__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns = kTcWaitNs) {
-  if (mbar_test(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  while (!mbar_test(bar, parity))
-    if (global_ns() - t0 > limit_ns) return false;
-  return true;
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: start, leading (K) and stride (8-row) byte offsets, all
 // >> 4; bit 46 = descriptor version 1; no swizzle, base offset 0.
@@ -208,11 +169,6 @@ __device__ __forceinline__ void tc_mma(uint32_t tmem, uint64_t da, uint64_t db, 
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
       "l"(da), "l"(db), "r"(kTcIdesc), "r"(accumulate)
       : "memory");
-}
-// The stage's mbarrier completes its phase when every MMA this thread issued so far is done.
-__device__ __forceinline__ void tc_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
-               : "memory");
 }
 // Initialises the stages' mbarriers and allocates the CTA's 128 TMEM columns; returns their
 // address. All threads.
