@@ -44,6 +44,10 @@ struct sg_model {
   std::vector<size_t> pC;
   bf16 *d_h1p = nullptr, *d_h2p = nullptr;
   std::vector<bf16*> d_zp;  // input of every stage
+  bool packed_train = false;  // and the backward pass
+  std::vector<size_t> pCt;    // transposed weights, in d_wp
+  std::vector<bf16*> d_dzp;   // gradient at every stage's output
+  float* d_sums = nullptr;    // scratch of the bias gradients
   long long step = 0;
   size_t dev_bytes = 0;
   std::vector<void*> allocs;
@@ -122,24 +126,53 @@ int pack_weights(sg_model* m) {
     const bool last = st + 1 == m->nstages;
     SG_LAUNCH(m, sgk::pack_conv(m->cin[st], last ? 32 * m->contract : m->cout[st], last ? m->out_c / 32 : 1,
                                 last ? m->out_c : 0, m->d_pb + m->oC[st], m->d_wp + m->pC[st], s));
+    if (m->packed_train)
+      SG_LAUNCH(m, sgk::pack_conv_t(m->cin[st], m->cout[st], m->d_pb + m->oC[st], m->d_wp + m->pCt[st], s));
   }
   return SG_OK;
 }
 
-int forward_packed(sg_model* m, int b, const float* x, float* y) {
+// The layers up to the last convolution's input; train: also what the backward pass reads.
+int hidden_packed(sg_model* m, int b, const float* x, bool train) {
   cudaStream_t s = m->stream;
   SG_LAUNCH(m, sgk::packed_dense(b, m->Bp, m->in_dim, m->hidden, x, nullptr, m->d_wp + m->pW1, m->d_p + m->ob1,
-                                 m->d_h1p, nullptr, 0, m->prod, s));
+                                 m->d_h1p, train ? m->d_a1 : nullptr, train ? m->d_h1 : nullptr, 0, m->prod, s));
   SG_LAUNCH(m, sgk::packed_dense(b, m->Bp, m->hidden, m->hidden, nullptr, m->d_h1p, m->d_wp + m->pW2, m->d_p + m->ob2,
-                                 m->d_h2p, nullptr, 0, m->prod, s));
+                                 m->d_h2p, train ? m->d_a2 : nullptr, train ? m->d_h2 : nullptr, 0, m->prod, s));
   SG_LAUNCH(m, sgk::packed_dense(b, m->Bp, m->hidden, m->c0 * m->l0, nullptr, m->d_h2p, m->d_wp + m->pW3,
-                                 m->d_p + m->ob3, m->d_zp[0], nullptr, m->l0, m->prod, s));
-  const int last = m->nstages - 1;
-  for (int st = 0; st < last; ++st)
+                                 m->d_p + m->ob3, m->d_zp[0], train ? m->d_a3 : nullptr, nullptr, m->l0, m->prod, s));
+  for (int st = 0; st + 1 < m->nstages; ++st)
     SG_LAUNCH(m, sgk::packed_conv(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], m->d_zp[st], m->d_wp + m->pC[st],
-                                  m->d_p + m->oc[st], m->d_zp[st + 1], nullptr, m->prod, s));
+                                  m->d_p + m->oc[st], m->d_zp[st + 1], train ? m->d_pre[st] : nullptr, m->prod, s));
+  return SG_OK;
+}
+
+int forward_packed(sg_model* m, int b, const float* x, float* y) {
+  if (int r = hidden_packed(m, b, x, false)) return r;
+  const int last = m->nstages - 1;
   SG_LAUNCH(m, sgk::packed_conv_contract(b, m->cin[last], m->contract, m->out_c, m->lin[last], m->in_dim,
-                                         m->d_zp[last], m->d_wp + m->pC[last], m->d_p + m->oc[last], x, y, m->prod, s));
+                                         m->d_zp[last], m->d_wp + m->pC[last], m->d_p + m->oc[last], x, y, m->prod,
+                                         m->stream));
+  return SG_OK;
+}
+
+// Forward and the convolutions' backward pass; leaves the gradient at the dense layers' output
+// in dz3 [b][c0 * l0].
+int backward_packed(sg_model* m, int b, const float* x, const float* target, float* dz3) {
+  if (int r = hidden_packed(m, b, x, true)) return r;
+  cudaStream_t s = m->stream;
+  const int last = m->nstages - 1;
+  SG_LAUNCH(m, sgk::packed_loss(b, m->cin[last], m->contract, m->out_c, m->lin[last], m->in_dim, m->d_zp[last],
+                                m->d_wp + m->pC[last], m->d_p + m->oc[last], x, target, m->d_dzp[last], m->d_sums,
+                                m->d_g + m->oc[last], m->d_partials, m->prod, s));
+  for (int st = last; st >= 0; --st) {
+    SG_LAUNCH(m, sgk::packed_conv_wgrad(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], m->d_dzp[st], m->d_zp[st],
+                                        m->d_g + m->oC[st], m->d_ws, m->prod, s));
+    SG_LAUNCH(m, sgk::packed_conv_dgrad(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], m->d_dzp[st],
+                                        m->d_wp + m->pCt[st], st ? m->d_pre[st - 1] : m->d_a3,
+                                        st ? m->d_dzp[st - 1] : nullptr, st ? m->up[st - 1] : 1, st ? nullptr : dz3,
+                                        st ? m->d_sums : nullptr, st ? m->d_g + m->oc[st - 1] : nullptr, m->prod, s));
+  }
   return SG_OK;
 }
 
@@ -286,6 +319,18 @@ int sg_create(sg_model** out, int device, void* stream, int in_dim, int hidden, 
       m->pC.push_back(w);
       w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
     }
+    m->packed_train = true;
+    size_t sums = 0;
+    for (int st = 0; st < nstages; ++st) {
+      m->packed_train = m->packed_train && sgk::packed_backward_ok(m->cin[st], m->cout[st], m->up[st]);
+      sums = std::max(sums, static_cast<size_t>(152) * m->cin[st]);
+    }
+    sums = std::max(sums, B * 4 * ((l + 127) / 128) * m->out_c);
+    if (m->packed_train)
+      for (int st = 0; st < nstages; ++st) {
+        m->pCt.push_back(w);
+        w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
+      }
     const size_t h = static_cast<size_t>(hidden) * m->Bp;
     r = sg_alloc(m, &m->d_wp, w);
     if (r == SG_OK) r = sg_alloc(m, &m->d_h1p, h);
@@ -298,6 +343,14 @@ int sg_create(sg_model** out, int device, void* stream, int in_dim, int hidden, 
       const size_t n = B * m->cin[st] * sgk::packed_rows(m->lin[st]);
       r = sg_alloc(m, &q, n);
       m->d_zp.push_back(q);
+      if (r == SG_OK) z = cudaMemsetAsync(q, 0, n * sizeof(bf16), m->stream);
+    }
+    if (m->packed_train && r == SG_OK) r = sg_alloc(m, &m->d_sums, sums);
+    for (int st = 0; m->packed_train && st < nstages && r == SG_OK && z == cudaSuccess; ++st) {
+      bf16* q = nullptr;
+      const size_t n = B * sgk::packed_grad_elems(m->cout[st], m->lin[st], m->up[st]);
+      r = sg_alloc(m, &q, n);
+      m->d_dzp.push_back(q);
       if (r == SG_OK) z = cudaMemsetAsync(q, 0, n * sizeof(bf16), m->stream);
     }
     if (z != cudaSuccess) r = sg_fail(m, SEM_ECUDA, std::string("sg_create: ") + cudaGetErrorString(z));
@@ -398,29 +451,35 @@ int sg_loss_grad(sg_model* m, int b, const float* x, const float* target, double
   if (b < 1 || b > m->max_batch || !x || !target || !loss) return sg_fail(m, SEM_EINVAL, "sg_loss_grad: bad arguments");
   SG_CUDA(m, cudaSetDevice(m->device));
   cudaStream_t s = m->stream;
-  int r = forward_chunk(m, b, x, nullptr);
-  if (r) return r;
+  const bool packed = m->packed_train && m->prod.kind == 1;
   const int last = m->nstages - 1;
   const size_t n = static_cast<size_t>(b) * m->out_c * m->out_l;
   float* cur = m->d_dA;
   float* other = m->d_dB;
-  SG_LAUNCH(m, sgk::mse_grad(n, m->contract ? m->d_y : m->d_pre[last], target, cur, m->d_partials, s));
-  if (m->contract) {
-    SG_LAUNCH(m, sgk::contract_backward(b, m->contract, m->out_c, m->out_l, m->in_dim, x, cur, other, s));
-    std::swap(cur, other);
-  }
-  for (int st = last; st >= 0; --st) {
-    if (st != last)
-      SG_LAUNCH(m, sgk::gelu_backward(static_cast<size_t>(b) * m->cout[st] * m->lout[st], m->d_pre[st], cur, s));
-    const float* input = st == 0 ? m->d_z0 : m->d_out[st - 1];
-    SG_LAUNCH(m, sgk::conv_backward_weight(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], cur, input,
-                                           m->d_g + m->oC[st], m->d_g + m->oc[st], m->d_ws, m->prod, s));
-    SG_LAUNCH(m, sgk::conv_backward_data(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], cur, m->d_pb + m->oC[st],
-                                         other, m->prod, s));
-    std::swap(cur, other);
-  }
   const int n3 = m->c0 * m->l0;
-  SG_LAUNCH(m, sgk::gelu_backward(static_cast<size_t>(b) * n3, m->d_a3, cur, s));
+  int loss_parts = sgk::kLossBlocks;
+  if (packed) {
+    if (int r = backward_packed(m, b, x, target, cur)) return r;
+    loss_parts = sgk::packed_loss_blocks(b, m->out_c, m->out_l);
+  } else {
+    if (int r = forward_chunk(m, b, x, nullptr)) return r;
+    SG_LAUNCH(m, sgk::mse_grad(n, m->contract ? m->d_y : m->d_pre[last], target, cur, m->d_partials, s));
+    if (m->contract) {
+      SG_LAUNCH(m, sgk::contract_backward(b, m->contract, m->out_c, m->out_l, m->in_dim, x, cur, other, s));
+      std::swap(cur, other);
+    }
+    for (int st = last; st >= 0; --st) {
+      if (st != last)
+        SG_LAUNCH(m, sgk::gelu_backward(static_cast<size_t>(b) * m->cout[st] * m->lout[st], m->d_pre[st], cur, s));
+      const float* input = st == 0 ? m->d_z0 : m->d_out[st - 1];
+      SG_LAUNCH(m, sgk::conv_backward_weight(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], cur, input,
+                                             m->d_g + m->oC[st], m->d_g + m->oc[st], m->d_ws, m->prod, s));
+      SG_LAUNCH(m, sgk::conv_backward_data(b, m->cin[st], m->cout[st], m->lin[st], m->up[st], cur, m->d_pb + m->oC[st],
+                                           other, m->prod, s));
+      std::swap(cur, other);
+    }
+    SG_LAUNCH(m, sgk::gelu_backward(static_cast<size_t>(b) * n3, m->d_a3, cur, s));
+  }
   SG_LAUNCH(m, sgk::linear_backward_weight(b, m->hidden, n3, cur, m->d_h2, m->d_g + m->oW3, m->d_g + m->ob3, m->d_ws,
                                            m->prod, s));
   SG_LAUNCH(m, sgk::linear_backward_data(b, m->hidden, n3, cur, m->d_pb + m->oW3, other, m->d_ws, m->prod, s));
@@ -433,7 +492,7 @@ int sg_loss_grad(sg_model* m, int b, const float* x, const float* target, double
   SG_LAUNCH(m, sgk::gelu_backward(static_cast<size_t>(b) * m->hidden, m->d_a1, cur, s));
   SG_LAUNCH(m, sgk::linear_backward_weight(b, m->in_dim, m->hidden, cur, x, m->d_g + m->oW1, m->d_g + m->ob1, m->d_ws,
                                            m->prod, s));
-  std::vector<double> part(sgk::kLossBlocks);
+  std::vector<double> part(loss_parts);
   SG_CUDA(m, cudaMemcpyAsync(part.data(), m->d_partials, part.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   SG_CUDA(m, cudaStreamSynchronize(s));
   if (int e = check_products(m, "sg_loss_grad")) return e;

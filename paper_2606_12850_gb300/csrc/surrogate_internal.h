@@ -72,7 +72,7 @@ int contract_forward(int B, int K, int C, int L, int in_dim, const float* x, con
 int contract_backward(int B, int K, int C, int L, int in_dim, const float* x, const float* dy, float* dD,
                       cudaStream_t s);
 
-// ---- packed forward (surrogate_packed.cu): bfloat16 activations in the tensor cores' layout ----
+// ---- packed passes (surrogate_packed.cu): bfloat16 activations in the tensor cores' layout ----
 // rows of a packed time axis of L samples (one zero row before, zeros after)
 int packed_rows(int L);
 bool packed_dense_ok(int K, int N);
@@ -83,14 +83,33 @@ int pack_dense(int K, int N, int l0, const bf16* W, bf16* Wp, cudaStream_t s);
 // W [Co][Ci][3] -> packed blocks of N rows; outC > 0: contracted copies of 32 channels a block
 int pack_conv(int Ci, int N, int blocks, int outC, const bf16* W, bf16* Wp, cudaStream_t s);
 // out = gelu(x W^T + b), from x [B][K] (or, x null, packed [K/8][Bp][8]) to packed [N/8][Bp][8]
-// (or, l0 > 0, [B][N/l0/8][packed_rows(l0)][8]); pre (or null) [B][N]
+// (or, l0 > 0, [B][N/l0/8][packed_rows(l0)][8]); pre and act (or null) [B][N]
 int packed_dense(int B, int Bp, int K, int N, const float* x, const bf16* in, const bf16* Wp, const float* bias,
-                 bf16* out, float* pre, int l0, const Products& pr, cudaStream_t s);
+                 bf16* out, float* pre, float* act, int l0, const Products& pr, cudaStream_t s);
 // hidden convolution, packed to packed; pre (or null) [B][N][up Lin]
 int packed_conv(int B, int Ci, int N, int Lin, int up, const bf16* in, const bf16* Wp, const float* bias, bf16* out,
                 float* pre, const Products& pr, cudaStream_t s);
 // the last convolution (K outC channels, no upsampling) and its contraction with x: y [B][outC][Lin]
 int packed_conv_contract(int B, int Ci, int K, int outC, int Lin, int in_dim, const bf16* in, const bf16* Wp,
                          const float* bias, const float* x, float* y, const Products& pr, cudaStream_t s);
+// The same in training: the sum of squared errors against target [B][outC][Lin] (loss, a value
+// per block of packed_loss_blocks), the packed gradient dD of the K outC channels and their bias
+// gradients db; row_sums: scratch of B * 4 ceil(Lin / 128) * outC floats
+int packed_loss(int B, int Ci, int K, int outC, int Lin, int in_dim, const bf16* in, const bf16* Wp, const float* bias,
+                const float* x, const float* target, bf16* dD, float* row_sums, float* db, double* loss,
+                const Products& pr, cudaStream_t s);
+int packed_loss_blocks(int B, int outC, int Lin);
+bool packed_backward_ok(int Ci, int Co, int up);
+size_t packed_grad_elems(int Co, int Lin, int up);  // packed gradient of one sample, [Co/8][up][rows][8]
+int pack_conv_t(int Ci, int Co, const bf16* W, bf16* Wt, cudaStream_t s);
+// dW [Co][Ci][3] from the packed gradient dZ of the output and the packed input X
+int packed_conv_wgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, const bf16* X, float* dW, float* ws,
+                      const Products& pr, cudaStream_t s);
+// The gradient at the layer below: dz = dX gelu'(pre), packed (out, of a layer that upsamples by
+// out_up) or float32 [B][Ci][Lin] (out_f32), and its bias gradients db [Ci] (sums: scratch of 152
+// Ci floats; both null to leave them out)
+int packed_conv_dgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, const bf16* Wt, const float* pre,
+                      bf16* out, int out_up, float* out_f32, float* sums, float* db, const Products& pr,
+                      cudaStream_t s);
 
 }  // namespace sgk
