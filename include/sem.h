@@ -410,6 +410,9 @@ int sem_adjoint_begin(sem_ctx* ctx);
 int sem_adjoint_step(sem_ctx* ctx, const float* G_dev);
 int sem_adjoint_accumulate(sem_ctx* ctx, const float* u_lo_dev, const float* u_mid_dev, const float* u_hi_dev);
 int sem_adjoint_gradients(sem_ctx* ctx, double* g_rho, double* g_kappa, double* g_mu);
+/* The same into device arrays, each value rounded to float32; asynchronous on the context's
+ * stream. NULL arrays are skipped. */
+int sem_adjoint_gradients_dev(sem_ctx* ctx, float* g_rho, float* g_kappa, float* g_mu);
 /* One segment of the backward sweep in a single call: with the adjoint at lam^{n0+count+1}
  * (and lam^{n0+count+2}), runs j = count down to 1: sem_adjoint_step(G_dev[j-1]) then
  * sem_adjoint_accumulate(u_dev[j-1], u_dev[j], u_dev[j+1]). G_dev: float32

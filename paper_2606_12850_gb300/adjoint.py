@@ -111,8 +111,9 @@ class Simulation:
         sem.sem_run_snapshots(self.ctx, n1 - n0, out[1:])
         return out
 
-    def gradient(self, G: torch.Tensor):
-        """dL/d(rho, kappa, mu) for dL/ds = G [nrec][3][nsteps]; float64 numpy [nspec][ngll^3]."""
+    def gradient(self, G: torch.Tensor, on_device: bool = False):
+        """dL/d(rho, kappa, mu) for dL/ds = G [nrec][3][nsteps]; float64 numpy [nspec][ngll^3],
+        or with ``on_device`` their float32 values as device tensors (no copy to the host)."""
         N = self.nsteps
         # Gt[m - 1] = G^m as a contiguous [nrec][3] block
         Gt = G.detach().to(self.device, torch.float32).permute(2, 0, 1).contiguous()
@@ -122,7 +123,7 @@ class Simulation:
             if N > 1:
                 sem.sem_adjoint_segment(self.ctx, N - 1, Gt[1:N], self.snapshots)
             sem.sem_sync(self.ctx)
-            return sem.sem_adjoint_gradients(self.ctx)
+            return self._gradients_dev() if on_device else sem.sem_adjoint_gradients(self.ctx)
         for n0 in reversed([c[0] for c in self.checkpoints]):
             # the terms n = n0 + 1 .. n0 + count, which read u^{n0} .. u^{n0 + count + 1}
             count = min(self.every, N - 1 - n0)
@@ -131,7 +132,14 @@ class Simulation:
             U = self._segment_displacements(n0, n0 + count + 1)
             sem.sem_adjoint_segment(self.ctx, count, Gt[n0 + 1:n0 + count + 1], U)
             sem.sem_sync(self.ctx)  # U is released (or reused) after this
-        return sem.sem_adjoint_gradients(self.ctx)
+        return self._gradients_dev() if on_device else sem.sem_adjoint_gradients(self.ctx)
+
+    def _gradients_dev(self):
+        out = [torch.empty((self.ctx.nspec, self.ctx.ngll ** 3), device=self.device) for _ in range(3)]
+        torch.cuda.synchronize(self.device)  # no earlier work of the process still uses their memory
+        sem.sem_adjoint_gradients_dev(self.ctx, *out)
+        sem.sem_sync(self.ctx)
+        return tuple(out)
 
 
 class Seismograms(torch.autograd.Function):
@@ -146,6 +154,8 @@ class Seismograms(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, grad_seis):
+        if ctx.device.type == "cuda":
+            return (*(g.to(ctx.device) for g in ctx.sim.gradient(grad_seis, on_device=True)), None)
         g_rho, g_kappa, g_mu = ctx.sim.gradient(grad_seis)
         as_t = lambda g: torch.from_numpy(g.astype(np.float32)).to(ctx.device)  # noqa: E731
         return as_t(g_rho), as_t(g_kappa), as_t(g_mu), None

@@ -2103,7 +2103,7 @@ bool fused_adjoint(const sem_ctx* c) { return c->fuse_newmark != 0 && c->assembl
 // and the leapfrog (or, unfused, the sweep, then the injection and leapfrog passes). G_dev is
 // the residual [nrec][3]; with idx it is taken from the device's adjoint counter (G_dev then
 // only says whether there is one).
-static int adjoint_sweep_step(sem_ctx* c, const float* G_dev, const DevCtl* idx) {
+static int adjoint_sweep_step(sem_ctx* c, const float* G_dev, const DevCtl* idx, int back = 0) {
   if (fused_adjoint(c)) {
     SweepNewmark nm{};
     nm.mode = 3;
@@ -2115,13 +2115,14 @@ static int adjoint_sweep_step(sem_ctx* c, const float* G_dev, const DevCtl* idx)
     nm.nrec = c->nrec;
     nm.G = idx ? nullptr : G_dev;
     nm.idx = G_dev ? idx : nullptr;
+    nm.back = back;
     nm.inv_dt2 = static_cast<float>(1.0 / (c->dt * c->dt));
     nm.dt2 = static_cast<float>(c->dt * c->dt);
     if (int r = forces_all_colors(c, c->d_lam, c->d_lamF, kNodeStride, 1, &nm)) return r;
   } else {
     if (int r = forces_all_colors(c, c->d_lam, c->d_lamF, kNodeStride, 1)) return r;
     SEM_LAUNCH(c, launch_adjoint_update(c->d_lamF, G_dev, c->d_rnode, c->d_roff, c->d_rlist, c->nrnodes, c->d_lam,
-                                        c->d_lam_old, c->d_minv, c->nglob, c->dt, c->stream, idx));
+                                        c->d_lam_old, c->d_minv, c->nglob, c->dt, c->stream, idx, back));
   }
   std::swap(c->d_lam, c->d_lam_old);  // lam <- lam^{m-1}, lam_old <- lam^m
   return SEM_OK;
@@ -2150,23 +2151,20 @@ int sem_adjoint_accumulate(sem_ctx* c, const float* u_lo, const float* u_mid, co
 }
 
 // One adjoint step (sweep of lam, residual injection and leapfrog, sensitivity terms) with
-// its residual and snapshots named by the device's adjoint counter, which it then lowers.
-// Step k of a run of indexed adjoint steps: the sweep of lam on the context's stream, the
+// its residual and snapshots named by the device's adjoint counter less k. Step k of a run of indexed adjoint steps: the sweep of lam on the context's stream, the
 // sensitivity terms on the auxiliary stream as soon as the sweep is done, so that they overlap
 // the next step's sweep. That sweep only writes the buffer of lam^{m+1}, which these terms do
 // not read; the sweep after it overwrites lam^{m-1}, so it waits for them (ev_sens ring).
 static int adjoint_indexed_step(sem_ctx* c, bool hasG, int k) {
   if (k >= 2) SEM_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_sens[k & 1], 0));
   // (with the counter the residual comes from it; the pointer only marks that there is one)
-  if (int r = adjoint_sweep_step(c, hasG ? c->d_lamF : nullptr, c->d_ctl)) return r;
-  SEM_LAUNCH(c, launch_adjoint_next(c->d_ctl, c->stream));
+  if (int r = adjoint_sweep_step(c, hasG ? c->d_lamF : nullptr, c->d_ctl, k)) return r;
   SEM_CUDA(c, cudaEventRecord(c->ev_sweep[k & 1], c->stream));
   SEM_CUDA(c, cudaStreamWaitEvent(c->aux, c->ev_sweep[k & 1], 0));
   const size_t nloc = static_cast<size_t>(c->nspec) * c->ngll * c->ngll * c->ngll;
   SEM_LAUNCH(c, launch_sensitivity(c->ngll, c->d_rec, c->node_order == 1 ? nullptr : c->d_perm, c->d_lam, nullptr,
                                     nullptr, nullptr, c->d_grad32, c->d_grad32 + nloc, c->d_grad32 + 2 * nloc,
-                                    c->nspec, -1.0, -c->dt * c->dt, c->aux, c->d_ctl));
-  SEM_LAUNCH(c, launch_adjoint_next(c->d_ctl, c->aux, true));
+                                    c->nspec, -1.0, -c->dt * c->dt, c->aux, c->d_ctl, k));
   SEM_CUDA(c, cudaEventRecord(c->ev_sens[k & 1], c->aux));
   return SEM_OK;
 }
@@ -2212,6 +2210,8 @@ static int adjoint_segment_steps(sem_ctx* c, int count, const float* G_dev, cons
       // join the auxiliary branch (its last terms) before the graph ends
       if (rc == SEM_OK && cudaStreamWaitEvent(c->stream, c->ev_sens[(kStepsPerGraph - 1) & 1], 0) != cudaSuccess)
         rc = fail(c, SEM_ECUDA, "adjoint graph join");
+      if (rc == SEM_OK && launch_adjoint_next(c->d_ctl, kStepsPerGraph, c->stream))
+        rc = fail(c, SEM_ECUDA, "adjoint counter");
       cudaError_t e = cudaStreamEndCapture(c->stream, &g);
       if (rc == SEM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_adj, g, 0);
       if (g) cudaGraphDestroy(g);
@@ -2244,23 +2244,33 @@ int sem_adjoint_gradients(sem_ctx* c, double* g_rho, double* g_kappa, double* g_
   if (!c->adjoint) return fail(c, SEM_ESTATE, "sem_adjoint_begin has not been called");
   int r = set_device(c);
   if (r || (r = flush_gradients(c))) return r;
-  const int n = c->ngll, np = n * n * n, nl = n * n;
-  const size_t nloc = static_cast<size_t>(c->nspec) * np;
-  std::vector<double> h(3 * nloc);
-  SEM_CUDA(c, cudaMemcpyAsync(h.data(), c->d_grad, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  SEM_CUDA(c, cudaStreamSynchronize(c->stream));
+  const size_t nloc = static_cast<size_t>(c->nspec) * c->ngll * c->ngll * c->ngll;
+  double* stage = nullptr;
+  SEM_CUDA(c, cudaMallocAsync(reinterpret_cast<void**>(&stage), nloc * sizeof(double), c->stream));
   double* outs[3] = {g_rho, g_kappa, g_mu};
-  for (int f = 0; f < 3; ++f) {
+  cudaError_t e = cudaSuccess;
+  for (int f = 0; f < 3 && e == cudaSuccess; ++f) {
     if (!outs[f]) continue;
-    for (int s = 0; s < c->nspec; ++s) {
-      const size_t caller = static_cast<size_t>(c->order[s]) * np;
-      const double* src = h.data() + f * nloc + static_cast<size_t>(s) * np;
-      for (int q = 0; q < np; ++q) {
-        const int i = q / nl, line = q - i * nl;
-        outs[f][caller + i + n * line] = src[q];
-      }
-    }
+    e = static_cast<cudaError_t>(launch_gradient_order(c->d_grad + f * nloc, c->d_order, stage, c->ngll, c->nspec, c->stream));
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(outs[f], stage, nloc * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   }
+  cudaFreeAsync(stage, c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "gradient copy");
+  SEM_CUDA(c, cudaStreamSynchronize(c->stream));
+  return SEM_OK;
+}
+
+int sem_adjoint_gradients_dev(sem_ctx* c, float* g_rho, float* g_kappa, float* g_mu) {
+  if (!c) return fail(nullptr, SEM_EINVAL, "null context");
+  if (!c->adjoint) return fail(c, SEM_ESTATE, "sem_adjoint_begin has not been called");
+  int r = set_device(c);
+  if (r || (r = flush_gradients(c))) return r;
+  const size_t nloc = static_cast<size_t>(c->nspec) * c->ngll * c->ngll * c->ngll;
+  float* outs[3] = {g_rho, g_kappa, g_mu};
+  for (int f = 0; f < 3; ++f)
+    if (outs[f])
+      SEM_LAUNCH(c, launch_gradient_order(c->d_grad + f * nloc, c->d_order, outs[f], c->ngll, c->nspec, c->stream));
   return SEM_OK;
 }
 

@@ -1587,10 +1587,10 @@ __global__ void __launch_bounds__(ForceCfg<N>::T)
                        const float* __restrict__ u_lo,
                        const float* __restrict__ u_mid, const float* __restrict__ u_hi, float* __restrict__ g_rho,
                        float* __restrict__ g_kappa, float* __restrict__ g_mu, int nspec, double c_m, double c_k,
-                       const DevCtl* __restrict__ idx) {
+                       const DevCtl* __restrict__ idx, int back) {
   using C = ForceCfg<N>;
   if (idx) {  // the snapshots of the step the device's adjoint counter names
-    const float* base = idx->adj_u + static_cast<long long>(idx->adj_js - 1) * idx->adj_n3;
+    const float* base = idx->adj_u + static_cast<long long>(idx->adj_j - back - 1) * idx->adj_n3;
     u_lo = base;
     u_mid = base + idx->adj_n3;
     u_hi = base + 2 * idx->adj_n3;
@@ -1928,14 +1928,14 @@ int SEM_CAT(launch_forces_, SEM_NGLL)(const ForceLaunch& L, void* stream) {
 int SEM_CAT(launch_sensitivity_, SEM_NGLL)(const float* rec, const int* perm, const float* lam, const float* u_lo,
                                           const float* u_mid, const float* u_hi, float* g_rho, float* g_kappa,
                                           float* g_mu, int nspec, double c_m, double c_k, void* stream,
-                                          const DevCtl* idx) {
+                                          const DevCtl* idx, int back) {
   using C = ForceCfg<SEM_NGLL>;
   static std::atomic<unsigned long long> attr_done{0};
   const int smem = C::SMEM_FLOATS * static_cast<int>(sizeof(float));
   if (int r = raise_smem_limit(attr_done, sensitivity_kernel<SEM_NGLL>, smem)) return r;
   const int grid = (nspec + C::EPC - 1) / C::EPC;
   sensitivity_kernel<SEM_NGLL><<<grid, C::T, smem, static_cast<cudaStream_t>(stream)>>>(
-      rec, perm, lam, u_lo, u_mid, u_hi, g_rho, g_kappa, g_mu, nspec, c_m, c_k, idx);
+      rec, perm, lam, u_lo, u_mid, u_hi, g_rho, g_kappa, g_mu, nspec, c_m, c_k, idx, back);
   return static_cast<int>(cudaGetLastError());
 }
 

@@ -149,9 +149,7 @@ struct DevCtl {
   const float* adj_u;
   long long adj_n3;
   int adj_gstep;
-  int adj_j;   // the step the sweep of lam is at (residual injection)
-  int adj_js;  // the step the sensitivity terms are at (they may run one step behind)
-  int pad3;
+  int adj_j;   // the step the captured steps begin at (they count back from it)
 };
 
 struct DevProblem {
@@ -279,6 +277,7 @@ struct SweepNewmark {
   float* lam_old;
   const float* G;
   const DevCtl* idx;
+  int back;   // steps since idx->adj_j was written
   float inv_dt2, dt2;
   const int* perm;  // mode 4: internal -> caller node
 };
@@ -393,22 +392,25 @@ int launch_corrector(const DevProblem& p, void* stream);
 int launch_sources_record(const DevProblem& p, int ahead, void* stream);
 // u_lo, u_mid, u_hi: [nglob][3] in caller order (perm: internal -> caller node) or in
 // internal order (perm null); the terms are added to float32 partials g_* [nlocal]
-// (idx non-null: the snapshots are idx->adj_u + (j - 1 .. j + 1) idx->adj_n3, j = idx->adj_j)
+// (idx non-null: the snapshots are idx->adj_u + (j - 1 .. j + 1) idx->adj_n3, j = idx->adj_j - back)
 int launch_sensitivity(int ngll, const float* rec, const int* perm, const float* lam, const float* u_lo,
                        const float* u_mid, const float* u_hi, float* g_rho, float* g_kappa, float* g_mu, int nspec,
-                       double c_m, double c_k, void* stream, const DevCtl* idx = nullptr);
+                       double c_m, double c_k, void* stream, const DevCtl* idx = nullptr, int back = 0);
 // fields in internal node order <-> caller layout
 // [shots][nglob][3] in caller node order (perm: internal -> caller node)
 int launch_pack(const float* u, float* out, const int* perm, int nglob, int shots, void* stream);
 int launch_unpack(const float* in, float* u, const int* perm, int nglob, int shots, void* stream);
 // rnode[nnodes]: distinct receiver nodes; rlist[roff[t] .. roff[t+1]): their receivers
-// (idx non-null: G_dev is taken from idx->adj_G at step idx->adj_j; G_dev then only says
+// (idx non-null: G_dev is taken from idx->adj_G at step idx->adj_j - back; G_dev then only says
 // whether there is one)
 int launch_adjoint_update(float* F, const float* G_dev, const int* rnode, const int* roff, const int* rlist,
                           int nnodes, const float* lam, float* lam_old, const float* minv, int nglob, double dt,
-                          void* stream, const DevCtl* idx = nullptr);
+                          void* stream, const DevCtl* idx = nullptr, int back = 0);
 int launch_adjoint_index(DevCtl* ctl, const float* G, const float* u, long long n3, int gstep, int j, void* stream);
-int launch_adjoint_next(DevCtl* ctl, void* stream, bool sensitivity = false);  // adj_j (or adj_js) -= 1
+int launch_adjoint_next(DevCtl* ctl, int steps, void* stream);  // adj_j -= steps
+// the accumulators (record order) in caller order [nspec][ngll^3], rounded to T
+template <class T>
+int launch_gradient_order(const double* acc, const int* order, T* out, int ngll, int nspec, void* stream);
 // acc[t] += part[t] (float64), part[t] = 0, for t < n
 int launch_flush_partials(float* part, double* acc, long long n, void* stream);
 // Material on the device (Sec. II-B moduli, Sec. I diagonal mass). rho, p1, p2: per local

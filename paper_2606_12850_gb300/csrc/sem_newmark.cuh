@@ -97,7 +97,7 @@ __device__ __forceinline__ void snapshot_node(const SweepNewmark& nm, uint32_t w
 // f = -K lam in ascending receiver order (G / dt^2).
 __device__ __forceinline__ void adjoint_receivers(const SweepNewmark& nm, const PatchRecv* __restrict__ recv, int nrec,
                                                   uint32_t node, float& fx, float& fy, float& fz) {
-  const float* G = nm.idx ? nm.idx->adj_G + static_cast<long long>(nm.idx->adj_j - 1) * nm.idx->adj_gstep : nm.G;
+  const float* G = nm.idx ? nm.idx->adj_G + static_cast<long long>(nm.idx->adj_j - nm.back - 1) * nm.idx->adj_gstep : nm.G;
   if (!G) return;
   for (int i = 0; i < nrec; ++i) {
     const PatchRecv e = recv[i];

@@ -73,6 +73,7 @@ SIGNATURES = {
     "sem_adjoint_step": (_I, [_P, _P]),
     "sem_adjoint_accumulate": (_I, [_P, _P, _P, _P]),
     "sem_adjoint_gradients": (_I, [_P, _P, _P, _P]),
+    "sem_adjoint_gradients_dev": (_I, [_P, _P, _P, _P]),
     "sem_adjoint_segment": (_I, [_P, _I, _P, _P]),
     "sem_energy_noalloc": (_I, [_P, _I, _P, _P, _P, _P]),
     "sem_sync": (_I, [_P]),
@@ -555,6 +556,12 @@ def sem_adjoint_gradients(ctx: Ctx):
     _check(lib().sem_adjoint_gradients(ctx.handle, *[o.ctypes.data_as(_P) for o in outs]), "sem_adjoint_gradients",
            ctx)
     return tuple(outs)
+
+
+def sem_adjoint_gradients_dev(ctx: Ctx, g_rho, g_kappa, g_mu):
+    n = ctx.nspec * ctx.ngll ** 3
+    _check(lib().sem_adjoint_gradients_dev(ctx.handle, *(_dev(g, n, ctx) for g in (g_rho, g_kappa, g_mu))),
+           "sem_adjoint_gradients_dev", ctx)
 
 
 def sem_adjoint_segment(ctx: Ctx, count: int, G_dev, u_dev):
