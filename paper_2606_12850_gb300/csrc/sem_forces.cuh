@@ -672,7 +672,10 @@ struct PatchCfg {
   static constexpr int SMEMW = TEAMS * TSW * 4;
   static constexpr int REC = ForceCfg<N>::REC;
   static constexpr int SMEM = TEAMS * TS * 4;
-  static constexpr int MIN_BLOCKS = N == 3 ? 3 : N <= 5 ? 4 : N <= 7 ? 3 : 2;
+  // resident CTAs the registers must allow (GB300, 24 steps: NGLL 3, 45 x 41 x 50, 4 CTAs 1.21 ms
+  // against 1.37 at 3 and 1.45 at 5; NGLL 5, 48^3, 7.40 at 4, 7.92 at 3, 9.15 at 5; NGLL 7, 25 x 21
+  // x 23, 2.79 at 3, 3.09 at 2, 3.36 at 4; NGLL 9, 16 x 15 x 17, 2.25 at 2, 3.22 at 1)
+  static constexpr int MIN_BLOCKS = N <= 5 ? 4 : N <= 7 ? 3 : 2;
   static_assert(E >= 1 && TEAM >= E * NL, "team size");
 };
 
