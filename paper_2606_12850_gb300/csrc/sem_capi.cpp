@@ -600,7 +600,7 @@ int sem_patch_plan(int ngll, int nspec, int nglob, const int32_t* ibool, int32_t
   PatchShape shape;
   PatchPlan plan;
   std::string err;
-  if (patch_shape(ngll, &shape) || build_patches(nspec, ngll, nglob, ibool, shape, &plan, &err))
+  if (patch_shape(ngll, nspec, &shape) || build_patches(nspec, ngll, nglob, ibool, shape, &plan, &err))
     return fail(nullptr, SEM_EINVAL, "sem_patch_plan: " + err);
   for (int c = 0; c < plan.ncolors; ++c)
     for (int P = plan.color_off[c]; P < plan.color_off[c + 1]; ++P) {
@@ -785,7 +785,7 @@ int sem_set_option(sem_ctx* c, int option, long long value) {
       return SEM_OK;
     case SEM_OPT_PATCH_SHAPE: {
       PatchShape def;
-      if (patch_shape(c->ngll, &def)) return fail(c, SEM_EINVAL, "no patch kernel for this order");
+      if (patch_shape(c->ngll, 0, &def)) return fail(c, SEM_EINVAL, "no patch kernel for this order");
       if (value == 0) {
         c->shape_opt = PatchShape{0, 0, 0};
         return SEM_OK;
@@ -901,7 +901,7 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
   // patches (bricks of the lattice coordinates, coloured) give the record order
   PatchShape shape;
   PatchPlan plan;
-  if (patch_shape(n, &shape)) return fail(c, SEM_EINVAL, "no patch kernel for this order");
+  if (patch_shape(n, nspec, &shape)) return fail(c, SEM_EINVAL, "no patch kernel for this order");
   if (c->shape_opt.bx > 0) shape = c->shape_opt;
   if (build_patches(nspec, n, nglob, ibool, shape, &plan, &err)) return fail(c, SEM_EINVAL, "patches: " + err);
   c->shape = shape;
@@ -2281,7 +2281,7 @@ int sem_tune_patch_shape(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
   if (reps < 1 || !ibool || (!xyz) == (!ctrl) || !rho || !vp || !vs)
     return fail(c, SEM_EINVAL, "sem_tune_patch_shape: bad arguments");
   PatchShape def;
-  if (patch_shape(c->ngll, &def)) return fail(c, SEM_EINVAL, "no patch kernel for this order");
+  if (patch_shape(c->ngll, 0, &def)) return fail(c, SEM_EINVAL, "no patch kernel for this order");
   const int pe = def.bx * def.by * def.bz;  // elements a patch CTA holds at this order
   std::vector<PatchShape> cand;
   for (int bz = 1; bz <= pe; ++bz)

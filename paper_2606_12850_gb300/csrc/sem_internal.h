@@ -362,7 +362,8 @@ struct PatchLayout {
 };
 int patch_layout(int ngll, PatchLayout* out);
 // the brick each order's patch kernel is compiled for
-int patch_shape(int ngll, PatchShape* out);
+// (nspec: the elements of the mesh it is for)
+int patch_shape(int ngll, int nspec, PatchShape* out);
 int forces_kernel_smem_bytes(int ngll);
 int forces_elements_per_cta(int ngll);
 
