@@ -146,7 +146,7 @@ int sem_destroy(sem_ctx* ctx);
 #define SEM_OPT_CONTRACTION 2
 /*   SEM_OPT_ASSEMBLY (takes effect at once): how the force sweep assembles element forces
  *   on the context's own fields. Patches are bricks of neighbouring elements
- *   (1 x 4 x 2 at NGLL 5, 2 x 2 x 2 from 20000 elements on; SEM_OPT_PATCH_SHAPE sets another,
+ *   (1 x 4 x 2 at NGLL 5, 2 x 2 x 2 from 4000 elements on; SEM_OPT_PATCH_SHAPE sets another,
  *   sem_patch_info gives the shape in use) evaluated by one CTA each, which
  *   sums the forces meeting at each of the brick's nodes in a fixed order; the bricks are
  *   coloured so that no two of a colour share a node (Sec. IV-C's colouring applied to groups of
@@ -516,15 +516,16 @@ int sem_sync(sem_ctx* ctx);
 
 /* Sizes of the set-up problem: out[0] nspec, out[1] nglob, out[2] ngll, out[3] ncolors,
  * out[4] steps taken since sem_set_state, out[5] bytes of device memory held,
- * out[6] shots, out[7] slabs of the sweep order, out[8] force-kernel launches per sweep.
+ * out[6] shots, out[7] slabs of the sweep order, out[8] launches per sweep of the
+ * element kernel (SEM_OPT_ASSEMBLY 1: one per element colour and slab).
  * out has room for 9 values; an entry not yet defined is 0. */
 int sem_info(sem_ctx* ctx, int64_t* out);
 
 /* Element count of each colour, counts[ncolors] (see sem_info for ncolors). */
 int sem_color_counts(sem_ctx* ctx, int32_t* counts);
 
-/* The patches of the force sweep (SEM_OPT_ASSEMBLY): out[0] patches, out[1] patch colours
- * (launches per sweep), out[2] largest patch node count, out[3] distinct patch tables (one
+/* The patches of the force sweep (SEM_OPT_ASSEMBLY): out[0] patches, out[1] patch colours,
+ * out[2] largest patch node count, out[3] distinct patch tables (one
  * for every patch of the same local structure), out[4..6] the brick in elements along the
  * mesh's lattice x, y, z, out[7] the assembly option in force. out has room for 8 values.
  * SEM_ESTATE before sem_set_mesh. */

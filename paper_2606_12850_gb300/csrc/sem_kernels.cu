@@ -93,13 +93,14 @@ static int order_shape(int n, PatchShape* out) {
   return -1;
 }
 
-// The order's brick. At NGLL 5, meshes whose records (6.5 KB an element) no longer fit the 129 MB
-// L2 take the cube of eight instead, which has 386 rim nodes of 729 rather than 450 of 765: there
-// the rim's traffic counts (GB300, us a step, 2 x 2 x 2 against 1 x 4 x 2: 40 x 36 x 44 170.1 /
-// 174.2, 28^3 66.0 / 66.6, 20^3 25.5 / 25.4, 12^3 12.0 / 12.3, 8^3 9.15 / 8.69).
+// The order's brick. At NGLL 5, meshes of some thousand elements and more take the cube of eight
+// instead, which has 386 rim nodes of 729 rather than 450 of 765: there the rim's traffic counts,
+// most with several shots and where the records no longer fit the 129 MB L2 (GB300, us a step,
+// 2 x 2 x 2 against 1 x 4 x 2: 40 x 36 x 44 170.1 / 174.2, 28^3 66.0 / 66.6, 20^3 25.5 / 25.4, with
+// 32 shots 593 / 604; 12^3 12.0 / 12.3, 8^3 9.15 / 8.69).
 int patch_shape(int n, int nspec, PatchShape* out) {
   const int r = order_shape(n, out);
-  if (r == 0 && n == 5 && nspec >= 20000) *out = PatchShape{2, 2, 2};
+  if (r == 0 && n == 5 && nspec >= 4000) *out = PatchShape{2, 2, 2};
   return r;
 }
 
