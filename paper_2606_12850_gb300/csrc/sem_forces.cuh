@@ -940,7 +940,8 @@ struct PatchFinish {
 // What bounds it (ncu, NGLL 5, 48^3): the L1 data pipe, 81 % busy (576 wavefronts an element:
 // 379 of shared memory, 197 of global loads), DRAM 59 %, issue slots 56 %; 250 us. With one
 // launch per patch colour (eight, each waiting for the one before) a step of that mesh took 329
-// us against 308, of 8^3 elements 50 us against 17, of 25 x 21 x 23 at NGLL 7 128 against 116.
+// us against 308 (298 with bricks of 2 x 2 x 2), of 8^3 elements 50 us against 17, of 25 x 21 x
+// 23 at NGLL 7 128 against 116.
 // With S shots (MS true) CTA b takes patch b / S for shot b % S: consecutive CTAs take the shots of one patch, so its records come from DRAM once
 // (the first shot's prefetch) and from L2 for the others.
 template <int N, bool LO, bool MS, int NM>
@@ -1583,6 +1584,10 @@ __global__ void __launch_bounds__(PatchCfg<N>::T, PatchCfg<N>::MIN_BLOCKS) group
 // added to float32 partial sums per local point in record order (element, q = i N^2 +
 // line), which the host flushes into float64 accumulators every few dozen steps. No two
 // threads write the same point, so there are no colours here.
+// Bound by latency (20^3, NGLL 5, ncu: 38 us, long scoreboard 8.4 cycles per issue, occupancy
+// 26 %, L1 pipe 48 %), so it runs on a second stream beside the next step's sweep: a gradient of
+// 64 steps takes 7.03 ms, on one stream (as a programmatic dependent of the rim pass) 7.35.
+// At 80 or 64 registers it spills (7.32, 8.47 ms).
 // ---------------------------------------------------------------------------------------
 template <int N>
 __global__ void __launch_bounds__(ForceCfg<N>::T)
