@@ -293,7 +293,8 @@ int sg_create(sg_model** out, int device, void* stream, int in_dim, int hidden, 
       (r = sg_alloc(m, &m->d_a2, B * hidden)) || (r = sg_alloc(m, &m->d_h2, B * hidden)) ||
       (r = sg_alloc(m, &m->d_a3, B * c0 * l0)) || (r = sg_alloc(m, &m->d_z0, B * c0 * l0)) ||
       (r = sg_alloc(m, &m->d_dA, B * act)) || (r = sg_alloc(m, &m->d_dB, B * act)) ||
-      (r = sg_alloc(m, &m->d_ws, ws)) || (r = sg_alloc(m, &m->d_partials, sgk::kLossBlocks)) ||
+      (r = sg_alloc(m, &m->d_ws, ws)) ||
+      (r = sg_alloc(m, &m->d_partials, sgk::loss_values(max_batch, m->out_c, m->out_l))) ||
       (r = sg_alloc(m, &m->d_err, 1)) || (r = sg_alloc(m, &m->d_pack, pack / sizeof(bf16))) ||
       (r = sg_alloc(m, &m->d_red, kRedFloats)) ||
       (r = sg_alloc(m, &m->d_y, contract ? B * m->out_c * m->out_l : 0))) {

@@ -99,6 +99,10 @@ int packed_loss(int B, int Ci, int K, int outC, int Lin, int in_dim, const bf16*
                 const float* x, const float* target, bf16* dD, float* row_sums, float* db, double* loss,
                 const Products& pr, cudaStream_t s);
 int packed_loss_blocks(int B, int outC, int Lin);
+// values the loss buffer holds: what mse_grad and packed_loss leave there for any batch up to B
+// (past 152 column blocks packed_loss has a CTA per 32 channels, more than kLossBlocks of them
+// from 19488 channels on)
+int loss_values(int B, int outC, int Lin);
 bool packed_backward_ok(int Ci, int Co, int up);
 size_t packed_grad_elems(int Co, int Lin, int up);  // packed gradient of one sample, [Co/8][up][rows][8]
 int pack_conv_t(int Ci, int Co, const bf16* W, bf16* Wt, cudaStream_t s);

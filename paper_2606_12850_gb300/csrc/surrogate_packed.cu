@@ -1153,6 +1153,10 @@ int packed_loss_blocks(int B, int outC, int Lin) {
   return conv_grid(B, outC / 32, Lin);
 }
 
+int loss_values(int B, int outC, int Lin) {
+  return outC < 32 ? kLossBlocks : std::max(kLossBlocks, packed_loss_blocks(B, outC, Lin));
+}
+
 bool packed_backward_ok(int Ci, int Co, int up) {
   return Ci % 16 == 0 && Ci <= 128 && Co % 32 == 0 && (up == 1 || up == 2);
 }
