@@ -262,8 +262,7 @@ __global__ void __launch_bounds__(256) dense_kernel(const DenseArgs a) {
 // back). The default network's forward pass of 4096 samples in chunks of 256, GB300: 16.6 ms
 // with the general kernels (tc_conv_kernel 12.2, contraction 4.4, dense 2.0), 3.6 ms now, 880
 // TFLOP/s of products; one sample 69 against 27 us, bound by the latency of seven launches.
-// Training: the epilogue goes on to the error against the target, its square (summed in a
-// float32 pair, 2^-46 relative, then float64), dy = 2 (y - t) / n, and the packed bfloat16
+// Training: the epilogue goes on to the error against the target, its square (squares16), dy = 2 (y - t) / n, and the packed bfloat16
 // gradient x_k dy of every contracted copy; y and dy themselves are not stored (258 us for 256
 // samples, where the convolution, contraction, loss and expansion kernels took 1.7 ms).
 struct ConvArgs {
@@ -303,6 +302,25 @@ __device__ __forceinline__ float warp_sums16(float (&v)[16], int lane) {
 // index i whose sum warp_sums16 leaves in this lane: its bits, most significant first, are the
 // lane's bits 4 .. 1
 __device__ __forceinline__ int warp_sums16_index(int lane) { return lane >> 1; }
+
+// Sum of the squares of 16 errors. A float32 pair takes them (each square exact as a pair, the
+// sum to about 2^-46) where its range holds them: from 2^-78, below which the low halves of the
+// squares that count would underflow, to float32's largest. Other groups (also all zeros, and
+// NaN) are summed in float64, whose units are too few to take every group.
+__device__ __forceinline__ double squares16(const float (&e)[16]) {
+  float hi = 0.f, lo = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float sq = e[i] * e[i], sq_lo = fmaf(e[i], e[i], -sq);
+    const float s = hi + sq, z = s - hi;  // two-sum
+    lo += ((hi - (s - z)) + (sq - z)) + sq_lo;
+    hi = s;
+  }
+  if (hi >= 0x1p-78f && hi <= 0x1.fffffep127f) return static_cast<double>(hi) + static_cast<double>(lo);
+  double d = 0.0;
+  for (int i = 0; i < 16; ++i) d += static_cast<double>(e[i]) * e[i];
+  return d;
+}
 
 enum { kHidden = 0, kAnswer = 1, kTrain = 2 };
 
@@ -414,7 +432,7 @@ __global__ void __launch_bounds__(320, 1) packed_conv_kernel(const ConvArgs a) {
   } else {
     const int q = warp & 3, h = (warp - 2) >> 2;
     const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
-    float loss_hi = 0.f, loss_lo = 0.f;
+    double loss = 0.0;
     for (int tile = first; tile < ntiles; tile += step, ++issued) {
       const int buf = issued & 1;
       const int b = tile / ntt, s = (tile - b * ntt) * kRows + q * 32 + lane;
@@ -454,14 +472,10 @@ __global__ void __launch_bounds__(320, 1) packed_conv_kernel(const ConvArgs a) {
         } else {
           if (s < a.Lin) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float e = sum[i] - t[i];
-              const float sq = e * e, sq_lo = fmaf(e, e, -sq);
-              const float hi = loss_hi + sq, z = hi - loss_hi;  // two-sum
-              loss_lo += ((loss_hi - (hi - z)) + (sq - z)) + sq_lo;
-              loss_hi = hi;
-              sum[i] = a.scale * e;
-            }
+            for (int i = 0; i < 16; ++i) sum[i] -= t[i];
+            loss += squares16(sum);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum[i] *= a.scale;
             const int row = 1 + s, g0 = (32 * nb + 16 * h) / 8, gs = a.outC / 8;
             for (int k = 0; k < a.K; ++k) {
               const float xk = __ldg(xb + k);
@@ -517,10 +531,9 @@ __global__ void __launch_bounds__(320, 1) packed_conv_kernel(const ConvArgs a) {
       }
     }
     if constexpr (KIND == kTrain) {
-      double sum = static_cast<double>(loss_hi) + static_cast<double>(loss_lo);
 #pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
-      if (lane == 0) reinterpret_cast<volatile double*>(sloss)[warp - 2] = sum;
+      for (int off = 16; off >= 1; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
+      if (lane == 0) reinterpret_cast<volatile double*>(sloss)[warp - 2] = loss;
     }
   }
   __syncwarp();

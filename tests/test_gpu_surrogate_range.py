@@ -49,3 +49,25 @@ def test_outputs_wider_than_the_general_loss_kernel_s_blocks():
     assert abs(loss - ref_loss) <= 1e-3 * ref_loss
     for name in ref_g:
         assert rel_l2(grads[name], ref_g[name]) <= 2e-3, name
+
+
+@pytest.mark.parametrize("scale", [1e21, 1e-22])
+def test_loss_of_errors_whose_squares_leave_float32(scale):
+    """Targets and last layer of this scale: the squared errors, 1e42 or 1e-44, are outside
+    float32's normal range, their mean is an ordinary float64 number (the gradients of the layers
+    below the last are outside float32 at the small scale in any case)."""
+    from paper_2606_12850_gb300 import surrogate
+    spec = surrogate.Spec(in_dim=9, hidden=64, c0=16, l0=20, stage_cout=(32, 3 * 32), stage_up=(2, 1), contract=3)
+    m = surrogate.Model(spec, max_batch=3)
+    flat = spec.init_params(5)
+    last = spec.split(flat)["C1"].size + spec.split(flat)["c1"].size
+    flat[-last:] = inputs.uniform(6, (last,), -0.1, 0.1) * min(scale, 1.0)
+    m.set_params(flat)
+    x = inputs.uniform(7, (3, 9), -1, 1).astype(np.float32)
+    t = (inputs.uniform(8, (3, spec.out_c, spec.out_l), -1, 1) * scale).astype(np.float32)
+    loss = m.loss_grad(torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda())
+    grads = spec.split(m.get_grads())
+    ref_loss, ref_g = oracle_net(spec, flat).backward(x.astype(np.float64), t.astype(np.float64))
+    assert ref_loss > 0 and abs(loss - ref_loss) <= 1e-3 * ref_loss
+    for name in ("C1", "c1"):
+        assert rel_l2(grads[name], ref_g[name]) <= 2e-3, name
