@@ -1027,9 +1027,11 @@ int conv_grid(int B, int blocks, int Lin) {
 }
 int grid1(size_t n) { return static_cast<int>(std::min<size_t>((n + 255) / 256, 65535)); }
 
+// The attribute is the process's, not the launch's: every model sets the same value, so that a
+// model in another thread, of other sizes, cannot lower it between this call and the launch.
 template <class K>
-cudaError_t set_smem(K kernel, int bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+cudaError_t raise_smem(K kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
 }
 
 }  // namespace
@@ -1055,7 +1057,7 @@ int pack_conv(int Ci, int N, int blocks, int outC, const bf16* W, bf16* Wp, cuda
 template <bool FROM_X, bool TO_Z>
 static int launch_dense(const DenseArgs& a, cudaStream_t s) {
   const int smem = dense_smem(a.Kp);
-  const cudaError_t e = set_smem(dense_kernel<FROM_X, TO_Z>, smem);
+  const cudaError_t e = raise_smem(dense_kernel<FROM_X, TO_Z>);
   if (e != cudaSuccess) return static_cast<int>(e);
   dense_kernel<FROM_X, TO_Z><<<dim3(a.N / 64, (a.B + kRows - 1) / kRows), 256, smem, s>>>(a);
   return static_cast<int>(cudaGetLastError());
@@ -1087,7 +1089,7 @@ int packed_dense(int B, int Bp, int K, int N, const float* x, const bf16* in, co
 template <int UP, int KIND>
 static int launch_conv(const ConvArgs& a, cudaStream_t s) {
   const int smem = conv_smem(a.Ci, a.N, a.stages);
-  const cudaError_t e = set_smem(packed_conv_kernel<UP, KIND>, smem);
+  const cudaError_t e = raise_smem(packed_conv_kernel<UP, KIND>);
   if (e != cudaSuccess) return static_cast<int>(e);
   packed_conv_kernel<UP, KIND><<<conv_grid(a.B, a.blocks, a.Lin), 320, smem, s>>>(a);
   return static_cast<int>(cudaGetLastError());
@@ -1199,7 +1201,7 @@ int packed_conv_wgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, co
   a.dst = a.splits > 1 ? ws : dW;
   const int smem = wgrad_smem(Ci, up, wgrad_stages(Ci, up));
   a.stages = wgrad_stages(Ci, up);
-  cudaError_t e = up == 2 ? set_smem(packed_wgrad_kernel<2>, smem) : set_smem(packed_wgrad_kernel<1>, smem);
+  cudaError_t e = up == 2 ? raise_smem(packed_wgrad_kernel<2>) : raise_smem(packed_wgrad_kernel<1>);
   if (e != cudaSuccess) return static_cast<int>(e);
   if (up == 2)
     packed_wgrad_kernel<2><<<ot * a.splits, 256, smem, s>>>(a);
@@ -1232,7 +1234,7 @@ int packed_conv_dgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, co
   a.stages = dgrad_stages(Ci, up);
   const int smem = dgrad_smem(Ci, up, a.stages);
   const int items = B * ((Lin + 2 * kRows - 1) / (2 * kRows)), grid = std::min(152, items);
-  const cudaError_t e = up == 2 ? set_smem(packed_dgrad_kernel<2>, smem) : set_smem(packed_dgrad_kernel<1>, smem);
+  const cudaError_t e = up == 2 ? raise_smem(packed_dgrad_kernel<2>) : raise_smem(packed_dgrad_kernel<1>);
   if (e != cudaSuccess) return static_cast<int>(e);
   if (up == 2)
     packed_dgrad_kernel<2><<<grid, 320, smem, s>>>(a);
