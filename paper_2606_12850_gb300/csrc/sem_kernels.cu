@@ -685,9 +685,10 @@ int launch_sources_record(const DevProblem& p, int ahead, void* stream) {
 // Threads that find one write 1 into the flag word; the host clears it first.
 // ---------------------------------------------------------------------------------------
 __global__ void nonfinite_kernel(const float4* __restrict__ u, const float4* __restrict__ v,
-                                 const float4* __restrict__ a, int nglob, int* flag) {
+                                 const float4* __restrict__ a, long long n, int* flag) {
   bool bad = false;
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nglob; t += gridDim.x * blockDim.x) {
+  for (long long t = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; t < n;
+       t += static_cast<long long>(gridDim.x) * blockDim.x) {
     const float4 x = u[t], y = v[t], z = a[t];
     bad |= !(isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(x.w));
     bad |= !(isfinite(y.x) && isfinite(y.y) && isfinite(y.z) && isfinite(y.w));
@@ -697,7 +698,7 @@ __global__ void nonfinite_kernel(const float4* __restrict__ u, const float4* __r
 }
 
 int launch_nonfinite_check(const DevProblem& p, int* flag, void* stream) {
-  const int n = p.nglob * padded_shots(p.shots);
+  const long long n = static_cast<long long>(p.nglob) * padded_shots(p.shots);
   nonfinite_kernel<<<kEnergyBlocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(
       reinterpret_cast<const float4*>(p.u), reinterpret_cast<const float4*>(p.v),
       reinterpret_cast<const float4*>(p.a), n, flag);
