@@ -2245,8 +2245,9 @@ int sem_adjoint_gradients(sem_ctx* c, double* g_rho, double* g_kappa, double* g_
   int r = set_device(c);
   if (r || (r = flush_gradients(c))) return r;
   const size_t nloc = static_cast<size_t>(c->nspec) * c->ngll * c->ngll * c->ngll;
-  double* stage = nullptr;
-  SEM_CUDA(c, cudaMallocAsync(reinterpret_cast<void**>(&stage), nloc * sizeof(double), c->stream));
+  // the reordered values pass through the flushed partial sums (12 bytes a point, zero at this
+  // point and again afterwards), so the call needs no device memory of its own
+  double* stage = reinterpret_cast<double*>(c->d_grad32);
   double* outs[3] = {g_rho, g_kappa, g_mu};
   cudaError_t e = cudaSuccess;
   for (int f = 0; f < 3 && e == cudaSuccess; ++f) {
@@ -2255,7 +2256,8 @@ int sem_adjoint_gradients(sem_ctx* c, double* g_rho, double* g_kappa, double* g_
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(outs[f], stage, nloc * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   }
-  cudaFreeAsync(stage, c->stream);
+  const cudaError_t z = cudaMemsetAsync(stage, 0, nloc * sizeof(double), c->stream);
+  if (e == cudaSuccess) e = z;
   if (e != cudaSuccess) return cuda_fail(c, e, "gradient copy");
   SEM_CUDA(c, cudaStreamSynchronize(c->stream));
   return SEM_OK;
