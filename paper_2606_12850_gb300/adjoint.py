@@ -154,7 +154,9 @@ class Seismograms(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, grad_seis):
-        if ctx.device.type == "cuda":
+        # (gradient(G) may be redefined, by a subclass or on the object: it then returns host arrays)
+        own = getattr(ctx.sim.gradient, "__func__", None) is Simulation.gradient
+        if own and ctx.device.type == "cuda":
             return (*(g.to(ctx.device) for g in ctx.sim.gradient(grad_seis, on_device=True)), None)
         g_rho, g_kappa, g_mu = ctx.sim.gradient(grad_seis)
         as_t = lambda g: torch.from_numpy(g.astype(np.float32)).to(ctx.device)  # noqa: E731
