@@ -520,23 +520,15 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
       w[r] = idx < ne * NP ? __float_as_uint(__ldg(rec + static_cast<size_t>(elem_of(le)) * REC + kIbool * NP + (idx - le * NP)))
                            : 0u;
     }
-    float q[GB][3];
+    float4 q[GB];
 #pragma unroll
     for (int r = 0; r < GB; ++r) {
       const size_t g = w[r] & kNodeMask;
       if (base + r * TEAM < ne * NP) {
-        if constexpr (CALLER) {
-          const size_t gc = static_cast<size_t>(__ldg(perm + g));
-          q[r][0] = __ldg(u + 3 * gc);
-          q[r][1] = __ldg(u + 3 * gc + 1);
-          q[r][2] = __ldg(u + 3 * gc + 2);
-        } else {
-          const int le = (base + r * TEAM) / NP;
-          const float4 v = __ldg(reinterpret_cast<const float4*>(u) + field_slot(nglob, S, g, shot_of(le)));
-          q[r][0] = v.x;
-          q[r][1] = v.y;
-          q[r][2] = v.z;
-        }
+        if constexpr (CALLER)
+          q[r] = load_node3(u + 3 * static_cast<size_t>(__ldg(perm + g)));
+        else
+          q[r] = __ldcg(reinterpret_cast<const float4*>(u) + field_slot(nglob, S, g, shot_of((base + r * TEAM) / NP)));
       }
     }
 #pragma unroll
@@ -548,9 +540,9 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
         float* eb = ts + le * ES;
         reinterpret_cast<uint32_t*>(eb + C::WORDS)[p] = w[r];
         float* pu = eb + Ws<N>::at(p);
-        pu[0] = q[r][0];
-        pu[1] = q[r][1];
-        pu[2] = q[r][2];
+        pu[0] = q[r].x;
+        pu[1] = q[r].y;
+        pu[2] = q[r].z;
       }
     }
   }
@@ -712,10 +704,8 @@ __device__ __forceinline__ void patch_gather_compute(const PatchDesc& d, const f
 #pragma unroll
       for (int r = 0; r < GB; ++r) w[r] = __ldg(perm + (w[r] & kNodeMask));
 #pragma unroll
-      for (int r = 0; r < GB; ++r) {
-        const float* pu = reinterpret_cast<const float*>(u) + 3 * static_cast<size_t>(w[r]);
-        q[r] = make_float4(__ldg(pu), __ldg(pu + 1), __ldg(pu + 2), 0.f);
-      }
+      for (int r = 0; r < GB; ++r)
+        q[r] = load_node3(reinterpret_cast<const float*>(u) + 3 * static_cast<size_t>(w[r]));
     } else {
 #pragma unroll
       for (int r = 0; r < GB; ++r) q[r] = __ldcg(u + node_slot<MS>(w[r]));
@@ -1170,8 +1160,8 @@ __device__ __forceinline__ void team_element_forces_pair(float* ts2, int tl, int
 // (GB300, 48^3 at NGLL 5, 32 shots: 2 beats 4).
 constexpr int kPairGatherBatch = 2;
 
-// Both shots' slots of a node, one 32-byte load (through L2: u may have been written by the
-// previous kernel).
+// Both shots' slots of a node, one 32-byte load (plain and volatile, behind the wait for the
+// previous kernel, which may have written u; not through the read-only path).
 __device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b) {
   asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)

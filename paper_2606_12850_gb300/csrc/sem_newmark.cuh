@@ -17,6 +17,19 @@ namespace {
 __device__ __forceinline__ void wait_prerequisite_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_dependent_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A wavefield the previous launch may have written is read only after that wait and never through
+// the read-only path (__ldg), which is for data no one writes while the kernel runs, its start
+// before the wait included: float4 nodes by __ldcg, the nodes of caller arrays [nglob][3] by
+// plain loads (volatile, so that they stay behind the wait), whose three words share L1 lines
+// (f = -K u on 44 x 36 x 40 elements at NGLL 5: 167 us, with __ldcg 180).
+__device__ __forceinline__ float4 load_node3(const float* p) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v.x) : "l"(p) : "memory");
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v.y) : "l"(p + 1) : "memory");
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v.z) : "l"(p + 2) : "memory");
+  return v;
+}
+
 // Index of a node's 16-byte slot in its shot's part of a field (see field_slot).
 template <bool MS>
 __device__ __forceinline__ size_t node_slot(uint32_t w) {
