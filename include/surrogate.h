@@ -87,8 +87,9 @@ int sg_sync(sg_model* model);
  * three taps; activations and their gradients pass between layers as the bfloat16 values the
  * products read where the sizes allow: hidden and c0*l0 multiples of 64 with hidden <= 576,
  * channels multiples of 32 and at most 128, c0 of 16, a contracted last stage without
- * upsampling); 0 = warp-level mma.sync, 128/256 x 64 tiles. Both round the
- * operands to bfloat16 and accumulate in float32, so they agree to float32 rounding order.
+ * upsampling, and sg_create finds device memory for them); 0 = warp-level mma.sync, 128/256 x
+ * 64 tiles. Both round the operands to bfloat16 and accumulate in float32, so they agree to
+ * float32 rounding order.
  * Setting an option waits for the model's stream. A tcgen05 product that waits more than 2 s
  * for its MMAs gives up: sg_loss_grad and sg_sync then return SEM_ETIMEOUT. */
 #define SG_OPT_PRODUCT 1

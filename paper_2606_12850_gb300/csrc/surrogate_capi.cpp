@@ -115,6 +115,48 @@ bool packed_sizes(const sg_model* m) {
   return true;
 }
 
+// The packed path's weights and activations, zeroed (zero rows pad the time axis), and whether it
+// also takes the backward pass.
+int alloc_packed(sg_model* m) {
+  const size_t B = m->max_batch;
+  const int n3 = m->c0 * m->l0;
+  m->Bp = (m->max_batch + 127) / 128 * 128;
+  size_t w = 0;
+  m->pW1 = w; w += sgk::packed_dense_elems(m->in_dim, m->hidden);
+  m->pW2 = w; w += sgk::packed_dense_elems(m->hidden, m->hidden);
+  m->pW3 = w; w += sgk::packed_dense_elems(m->hidden, n3);
+  m->packed_train = true;
+  size_t sums = 0;
+  for (int st = 0; st < m->nstages; ++st) {
+    m->pC.push_back(w);
+    w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
+    m->packed_train = m->packed_train && sgk::packed_backward_ok(m->cin[st], m->cout[st], m->up[st]);
+    sums = std::max(sums, static_cast<size_t>(152) * m->cin[st]);
+  }
+  sums = std::max(sums, B * 4 * ((m->out_l + 127) / 128) * m->out_c);
+  for (int st = 0; m->packed_train && st < m->nstages; ++st) {
+    m->pCt.push_back(w);
+    w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
+  }
+  auto zeroed = [&](bf16** p, size_t n) -> int {
+    if (int r = sg_alloc(m, p, n)) return r;
+    SG_CUDA(m, cudaMemsetAsync(*p, 0, n * sizeof(bf16), m->stream));
+    return SG_OK;
+  };
+  int r = SG_OK;
+  const size_t h = static_cast<size_t>(m->hidden) * m->Bp;
+  if ((r = zeroed(&m->d_wp, w)) || (r = zeroed(&m->d_h1p, h)) || (r = zeroed(&m->d_h2p, h))) return r;
+  m->d_zp.assign(m->nstages, nullptr);
+  for (int st = 0; st < m->nstages; ++st)
+    if ((r = zeroed(&m->d_zp[st], B * m->cin[st] * sgk::packed_rows(m->lin[st])))) return r;
+  if (!m->packed_train) return SG_OK;
+  if ((r = sg_alloc(m, &m->d_sums, sums))) return r;
+  m->d_dzp.assign(m->nstages, nullptr);
+  for (int st = 0; st < m->nstages; ++st)
+    if ((r = zeroed(&m->d_dzp[st], B * sgk::packed_grad_elems(m->cout[st], m->lin[st], m->up[st])))) return r;
+  return SG_OK;
+}
+
 // The packed copies of the bfloat16 weights, after they changed.
 int pack_weights(sg_model* m) {
   if (!m->packed) return SG_OK;
@@ -311,50 +353,18 @@ int sg_create(sg_model** out, int device, void* stream, int in_dim, int hidden, 
   }
   m->packed = packed_sizes(m);
   if (r == SG_OK && m->packed) {
-    m->Bp = (max_batch + 127) / 128 * 128;
-    size_t w = 0;
-    m->pW1 = w; w += sgk::packed_dense_elems(in_dim, hidden);
-    m->pW2 = w; w += sgk::packed_dense_elems(hidden, hidden);
-    m->pW3 = w; w += sgk::packed_dense_elems(hidden, c0 * l0);
-    for (int st = 0; st < nstages; ++st) {
-      m->pC.push_back(w);
-      w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
+    const size_t have = m->allocs.size(), bytes = m->dev_bytes;
+    r = alloc_packed(m);
+    if (r == SEM_ENOMEM) {  // no room for it: the general kernels, whose buffers are there, take every call
+      cudaGetLastError();
+      cudaStreamSynchronize(m->stream);
+      for (size_t i = have; i < m->allocs.size(); ++i) cudaFree(m->allocs[i]);
+      m->allocs.resize(have);
+      m->dev_bytes = bytes;
+      m->packed = m->packed_train = false;
+      m->err.clear();
+      r = SG_OK;
     }
-    m->packed_train = true;
-    size_t sums = 0;
-    for (int st = 0; st < nstages; ++st) {
-      m->packed_train = m->packed_train && sgk::packed_backward_ok(m->cin[st], m->cout[st], m->up[st]);
-      sums = std::max(sums, static_cast<size_t>(152) * m->cin[st]);
-    }
-    sums = std::max(sums, B * 4 * ((l + 127) / 128) * m->out_c);
-    if (m->packed_train)
-      for (int st = 0; st < nstages; ++st) {
-        m->pCt.push_back(w);
-        w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
-      }
-    const size_t h = static_cast<size_t>(hidden) * m->Bp;
-    r = sg_alloc(m, &m->d_wp, w);
-    if (r == SG_OK) r = sg_alloc(m, &m->d_h1p, h);
-    if (r == SG_OK) r = sg_alloc(m, &m->d_h2p, h);
-    cudaError_t z = r == SG_OK ? cudaMemsetAsync(m->d_wp, 0, w * sizeof(bf16), m->stream) : cudaSuccess;
-    if (r == SG_OK && z == cudaSuccess) z = cudaMemsetAsync(m->d_h1p, 0, h * sizeof(bf16), m->stream);
-    if (r == SG_OK && z == cudaSuccess) z = cudaMemsetAsync(m->d_h2p, 0, h * sizeof(bf16), m->stream);
-    for (int st = 0; st < nstages && r == SG_OK && z == cudaSuccess; ++st) {  // zero rows pad the time axis
-      bf16* q = nullptr;
-      const size_t n = B * m->cin[st] * sgk::packed_rows(m->lin[st]);
-      r = sg_alloc(m, &q, n);
-      m->d_zp.push_back(q);
-      if (r == SG_OK) z = cudaMemsetAsync(q, 0, n * sizeof(bf16), m->stream);
-    }
-    if (m->packed_train && r == SG_OK) r = sg_alloc(m, &m->d_sums, sums);
-    for (int st = 0; m->packed_train && st < nstages && r == SG_OK && z == cudaSuccess; ++st) {
-      bf16* q = nullptr;
-      const size_t n = B * sgk::packed_grad_elems(m->cout[st], m->lin[st], m->up[st]);
-      r = sg_alloc(m, &q, n);
-      m->d_dzp.push_back(q);
-      if (r == SG_OK) z = cudaMemsetAsync(q, 0, n * sizeof(bf16), m->stream);
-    }
-    if (z != cudaSuccess) r = sg_fail(m, SEM_ECUDA, std::string("sg_create: ") + cudaGetErrorString(z));
   }
   if (r == SG_OK) {
     const size_t bytes = m->P * sizeof(float);

@@ -64,3 +64,40 @@ def test_gradients_to_the_host():
     sem.sem_adjoint_segment(s.ctx, 3, G, u)
     for a, b in zip(sem.sem_adjoint_gradients(s.ctx), both):
         assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(a)
+
+
+def test_surrogate_without_room_for_the_packed_activations():
+    """A max_batch whose general buffers fit and whose packed ones (210 MB beside 1.1 GB here) do not:
+    the model is created and the general kernels take its calls."""
+    from paper_2606_12850_gb300 import surrogate
+    spec = surrogate.Spec()
+    flat = spec.init_params(9)
+    x = torch.from_numpy(inputs.uniform(10, (3, 9), -1, 1).astype(np.float32)).cuda()
+    t = torch.from_numpy(inputs.uniform(11, (3, spec.out_c, spec.out_l), -1, 1).astype(np.float32)).cuda()
+    small = surrogate.Spec(in_dim=9, hidden=24, c0=6, l0=7, stage_cout=(10, 8, 12), stage_up=(2, 2, 1), contract=6)
+    warm = surrogate.Model(small, max_batch=4)  # loads the general kernels
+    warm.set_params(small.init_params(1))
+    warm.loss_grad(x, torch.zeros((3, small.out_c, small.out_l), device="cuda"))
+
+    def use(m):
+        m.set_params(flat)
+        y = torch.zeros((3, spec.out_c, spec.out_l), device="cuda")
+        torch.cuda.synchronize()
+        m.forward(x, y)
+        return m.info()["device_bytes"], m.loss_grad(x, t), y.cpu().numpy().astype(np.float64), m.get_grads()
+
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    m = surrogate.Model(spec, max_batch=64)
+    need = before - torch.cuda.mem_get_info()[0]
+    ref = use(m)
+    del m
+    keep = torch.zeros((3, spec.out_c, spec.out_l), device="cuda")  # cached for use()
+    del keep
+    with full_device(leave=need - (120 << 20)):
+        got = use(surrogate.Model(spec, max_batch=64))
+    assert ref[0] - got[0] > 120 << 20
+    assert abs(got[1] - ref[1]) <= 1e-4 * ref[1]
+    for a, b in zip(ref[2:], got[2:]):
+        assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(a)
