@@ -154,7 +154,9 @@ int sem_destroy(sem_ctx* ctx);
  *     0 (default) = patches, one launch over all of them: the nodes of one brick are completed
  *       by it, and at the nodes bricks share every brick leaves its sum, which a second launch
  *       adds up in the order of the colours (with several shots one CTA per patch and shot or
- *       shot pair). Also used for caller-layout arrays;
+ *       shot pair). Also used for caller-layout arrays. Where those sums (16 bytes per shared
+ *       node of a brick and shot) do not fit on the device, form 2 or, for several shots and
+ *       caller-layout arrays, 1 runs instead;
  *     1 = element by element, one launch per element colour (2 and 3 use this form for
  *       caller-layout arrays);
  *     2 = patches, all colours in one persistent launch (single shot; several shots use 0):

@@ -170,6 +170,17 @@ int dev_alloc(sem_ctx* c, T** p, size_t count) {
   return SEM_OK;
 }
 
+// The partials buffer of the one-launch sweep, taken after everything else a mesh or its shots
+// need. Without room for it the forms that write nodes in place run instead (has_partials).
+int alloc_partials(sem_ctx* c) {
+  const int r = dev_alloc(c, &c->d_rimsums, kNodeStride * c->nrimsums * padded_shots(c->shots));
+  if (r != SEM_ENOMEM) return r;
+  cudaGetLastError();
+  c->err.clear();
+  return SEM_OK;
+}
+bool has_partials(const sem_ctx* c) { return c->nrimsums == 0 || c->d_rimsums; }
+
 void free_device(sem_ctx* c) {
   void* ptrs[] = {c->d_rec, c->d_order, c->d_elist, c->d_perm, c->d_node_new, c->d_pdesc, c->d_pslots, c->d_pwords, c->d_pcolor_end, c->d_sync, c->d_psrc, c->d_rsrc, c->d_rim, c->d_rimover,
                   c->d_rblocks, c->d_rimsums, c->d_u, c->d_v,
@@ -267,12 +278,16 @@ bool pair_rule(const sem_ctx* c, int shots) {
 // Caller arrays [nglob][3] go through the same sweep, read and written through the node
 // permutation (mode 4). With SEM_OPT_ASSEMBLY 1 the element kernel
 // walks the element list slab by slab and, inside a slab, colour by colour: a launch holds
-// elements of one colour only.
+// elements of one colour only. Without room for the partials the persistent launch (one shot) or
+// the element kernel takes the place of SEM_OPT_ASSEMBLY 0.
 // With nm (mode 1, 2 or 3; see fused_sweep) both passes also run the update of every node.
 int forces_all_colors(sem_ctx* c, const float* u, float* f, int node_stride, int shots,
                       const SweepNewmark* nm = nullptr) {
   const bool caller = node_stride == 3;
-  if (c->npatch > 0 && (c->assembly == 0 || (c->assembly == 2 && !caller))) {
+  const int npc = static_cast<int>(c->pcolor_off.size()) - 1;
+  const bool patches = c->npatch > 0 && (c->assembly == 0 || (c->assembly == 2 && !caller));
+  const bool persistent = (c->assembly == 2 || !has_partials(c)) && !caller && !nm && shots == 1 && npc <= kMaxSweepColors;
+  if (patches && (persistent || has_partials(c))) {
     PatchLaunch P{};
     if (nm) P.nm = *nm;
     P.nm.nglob = c->nglob;
@@ -292,8 +307,7 @@ int forces_all_colors(sem_ctx* c, const float* u, float* f, int node_stride, int
       P.nm.mode = 4;
       P.nm.perm = c->d_perm;
     }
-    const int npc = static_cast<int>(c->pcolor_off.size()) - 1;
-    if (c->assembly == 2 && shots == 1 && npc <= kMaxSweepColors && P.nm.mode == 0) {
+    if (persistent) {
       P.sync = c->d_sync;
       P.color_end = c->d_pcolor_end;
       P.ncolors = npc;
@@ -351,7 +365,9 @@ int forces_all_colors(sem_ctx* c, const float* u, float* f, int node_stride, int
 // SEM_OPT_FUSED_NEWMARK not 0. With several shots too: GB300, 20^3 at NGLL 5, 24 steps, 32
 // shots 14.8 ms against 17.1 ms with a separate pass, 4 shots 2.09 against 2.47 ms (before the
 // shots were kept in pairs the separate pass, which streams, was the faster one).
-bool fused_sweep(const sem_ctx* c) { return c->fuse_newmark != 0 && c->assembly == 0 && c->npatch > 0; }
+bool fused_sweep(const sem_ctx* c) {
+  return c->fuse_newmark != 0 && c->assembly == 0 && c->npatch > 0 && has_partials(c);
+}
 
 SweepNewmark sweep_newmark(const sem_ctx* c, int mode) {
   SweepNewmark nm{};
@@ -1225,10 +1241,9 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
       (r = dev_alloc(c, &c->d_pcolor_end, static_cast<size_t>(plan.ncolors))) || (r = dev_alloc(c, &c->d_sync, 1)) ||
       (r = dev_alloc(c, &c->d_rim, rim.size())) || (r = dev_alloc(c, &c->d_rimover, rimover.size())) ||
       (r = dev_alloc(c, &c->d_rblocks, c->rblocks.size())) ||
-      (r = dev_alloc(c, &c->d_rimsums, kNodeStride * nrimsums * padded_shots(c->shots))) ||
       (r = dev_alloc(c, &c->d_u, nf)) ||
       (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf)) ||
-      (r = dev_alloc(c, &c->d_minv, static_cast<size_t>(nglob))))
+      (r = dev_alloc(c, &c->d_minv, static_cast<size_t>(nglob))) || (r = alloc_partials(c)))
     return r;
   // geometry and ibool travel once; the material fields are written on the device
   SEM_CUDA(c, cudaMemcpyAsync(c->d_rec, c->rec.data(), c->rec.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
@@ -1638,8 +1653,12 @@ int sem_set_shots(sem_ctx* c, int nshots) {
   if (r) return r;
   cudaStreamSynchronize(c->stream);
   const size_t old = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots) * sizeof(float);
-  const size_t old_sums = kNodeStride * c->nrimsums * padded_shots(c->shots) * sizeof(float);
   c->dev_bytes -= 3 * old;
+  if (c->d_rimsums) {
+    c->dev_bytes -= kNodeStride * c->nrimsums * padded_shots(c->shots) * sizeof(float);
+    cudaFree(c->d_rimsums);
+    c->d_rimsums = nullptr;
+  }
   if (c->d_f) {
     c->dev_bytes -= old;
     cudaFree(c->d_f);
@@ -1647,9 +1666,8 @@ int sem_set_shots(sem_ctx* c, int nshots) {
   }
   c->shots = nshots;
   const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(nshots);
-  c->dev_bytes -= old_sums;
   if ((r = dev_alloc(c, &c->d_u, nf)) || (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf)) ||
-      (r = dev_alloc(c, &c->d_rimsums, kNodeStride * c->nrimsums * padded_shots(nshots))))
+      (r = alloc_partials(c)))
     return r;
   SEM_CUDA(c, cudaMemsetAsync(c->d_u, 0, nf * sizeof(float), c->stream));
   SEM_CUDA(c, cudaMemsetAsync(c->d_v, 0, nf * sizeof(float), c->stream));
@@ -2097,7 +2115,7 @@ int sem_adjoint_begin(sem_ctx* c) {
 
 // Whether adjoint steps run the leapfrog inside the sweep of lam (the patch sweep with
 // SEM_OPT_FUSED_NEWMARK not 0).
-bool fused_adjoint(const sem_ctx* c) { return c->fuse_newmark != 0 && c->assembly == 0 && c->npatch > 0; }
+bool fused_adjoint(const sem_ctx* c) { return fused_sweep(c); }
 
 // One adjoint step: the sweep of lam with, at each node's last touch, the residual injection
 // and the leapfrog (or, unfused, the sweep, then the injection and leapfrog passes). G_dev is

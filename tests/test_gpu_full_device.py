@@ -22,20 +22,19 @@ def library():
 
 @contextlib.contextmanager
 def full_device(leave=0):
-    """Within it, other arrays hold the free device memory but for ``leave`` bytes, to within 4 MB."""
+    """Within it, other arrays hold the free device memory but for ``leave`` bytes and less than 12 MB
+    more (smaller arrays would come from segments of 20 MB)."""
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     held = []
-    step = 1 << 38
-    while step >= 2 << 20:
-        free = torch.cuda.mem_get_info()[0] - leave
-        if free < step:
-            step >>= 1
-            continue
+    while (free := (torch.cuda.mem_get_info()[0] - leave) // (2 << 20) * (2 << 20)) >= 12 << 20:
         try:
-            held.append(torch.empty(step, dtype=torch.uint8, device="cuda"))
+            held.append(torch.empty(free, dtype=torch.uint8, device="cuda"))
         except torch.OutOfMemoryError:
-            step >>= 1
+            try:
+                held.append(torch.empty(free // 2 // (2 << 20) * (2 << 20), dtype=torch.uint8, device="cuda"))
+            except torch.OutOfMemoryError:
+                break
     try:
         yield
     finally:
@@ -44,7 +43,7 @@ def full_device(leave=0):
 
 
 def test_gradients_to_the_host():
-    w = inputs.layered_cube(5, n=16, side=2000.0, nrec_side=2)  # 4 MB of float64 a gradient
+    w = inputs.layered_cube(5, n=24, side=2000.0, nrec_side=2)  # 14 MB of float64 a gradient
     s = sem.setup_workload(w)
     u = torch.from_numpy(inputs.uniform(5, (5, w.mesh.nglob, 3), -1, 1).astype(np.float32)).cuda()
     G = torch.from_numpy(inputs.uniform(6, (3, len(s.rec_nodes), 3), -1, 1).astype(np.float32)).cuda()
@@ -101,3 +100,75 @@ def test_surrogate_without_room_for_the_packed_activations():
     assert abs(got[1] - ref[1]) <= 1e-4 * ref[1]
     for a, b in zip(ref[2:], got[2:]):
         assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(a)
+
+
+def rel_l2(a, b):
+    return float(np.linalg.norm(a.astype(np.float64) - b) / np.linalg.norm(b))
+
+
+def test_shots_without_room_for_the_sweep_s_partials():
+    """32 shots whose fields fit (422 MB) and whose partial sums (91 MB) do not."""
+    w = inputs.layered_cube(5, n=16, side=2000.0, nrec_side=2)
+    shots, out = 32, []
+    pos = inputs.uniform(3, (shots, 3), 500.0, 1500.0)
+    for tight in (False, True):
+        s = sem.setup_workload(w)
+        nodes = sem.sem_locate_nodes(s.ctx, pos)
+        sem.sem_run(s.ctx, 2)  # loads the kernels of the shots' set-up
+        if tight:
+            with full_device(leave=48 * (shots - 1) * w.mesh.nglob + (32 << 20)):
+                sem.sem_set_shots(s.ctx, shots)
+        else:
+            sem.sem_set_shots(s.ctx, shots)
+        sem.sem_set_shot_sources(s.ctx, np.arange(shots), nodes, np.tile([0.0, 1e10, 1e10], (shots, 1)), w.f0, 0.0)
+        sem.sem_set_state(s.ctx)
+        seis = sem.sem_run(s.ctx, 13)
+        u = sem.sem_get_state(s.ctx, want=(True, False, False))[0]
+        out.append((sem.sem_info(s.ctx)["device_bytes"], seis, u))
+    assert out[0][0] - out[1][0] > 80 << 20
+    assert rel_l2(out[1][1], out[0][1]) <= 2e-5 and rel_l2(out[1][2], out[0][2]) <= 2e-5
+
+
+def test_mesh_without_room_for_the_sweep_s_partials():
+    """A mesh of which only the partial sums (25 MB) do not fit: steps by the persistent sweep, which
+    adds in the same order, f = -K u on caller arrays by the element kernel, the adjoint."""
+    w = inputs.layered_cube(5, n=32, side=4000.0, nrec_side=2)
+    sem.setup_workload(inputs.layered_cube(5, n=2, side=400.0, nrec_side=2))  # loads the kernels
+    out, need = [], None
+    for tight in (False, True):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        before = torch.cuda.mem_get_info()[0]
+        ctx = sem.sem_create(5, 0)
+        if tight:
+            with full_device(leave=need - (18 << 20)):
+                sem.sem_set_mesh_corners(ctx, w.mesh.ibool, w.mesh.ctrl, w.mesh.nglob)
+        else:
+            sem.sem_set_mesh_corners(ctx, w.mesh.ibool, w.mesh.ctrl, w.mesh.nglob)
+            need = before - torch.cuda.mem_get_info()[0]
+        held = sem.sem_info(ctx)["device_bytes"]
+        sem.sem_set_material(ctx, w.rho, w.vp, w.vs)
+        sem.sem_set_dt(ctx, sem.sem_suggest_dt(ctx, 0.3))
+        node = sem.sem_locate_nodes(ctx, w.source_xyz)
+        sem.sem_set_source_nodes(ctx, node, w.source_force, w.f0, 0.0)
+        sem.sem_set_receiver_nodes(ctx, node)
+        sem.sem_set_state(ctx)
+        seis = sem.sem_run(ctx, 13)
+        u = sem.sem_get_state(ctx, want=(True, False, False))[0]
+        field = torch.from_numpy(inputs.random_field(w.mesh.nglob, 6)).cuda()
+        f = torch.empty_like(field)
+        snaps = field[None].repeat(4, 1, 1) * torch.arange(4, device="cuda")[:, None, None]
+        G = torch.ones((2, len(node), 3), device="cuda")
+        torch.cuda.synchronize()
+        sem.sem_apply_stiffness(ctx, field, f)
+        sem.sem_sync(ctx)
+        sem.sem_adjoint_begin(ctx)
+        sem.sem_adjoint_segment(ctx, 2, G, snaps)
+        out.append((held, seis, u, f.cpu().numpy(), sem.sem_adjoint_gradients(ctx)))
+        del ctx, field, f, snaps
+    a, b = out
+    assert a[0] - b[0] > 20 << 20
+    assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2]) and np.any(a[1] != 0)
+    assert rel_l2(b[3], a[3]) <= 1e-6
+    for x, y in zip(a[4], b[4]):
+        assert rel_l2(y, x) <= 1e-5
