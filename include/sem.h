@@ -197,7 +197,7 @@ int sem_destroy(sem_ctx* ctx);
 /*   SEM_OPT_SHOT_PAIRS (takes effect at once; several shots, SEM_OPT_ASSEMBLY 0): 1 = each CTA
  *   of the patch sweep takes one patch for two shots, every thread carrying both shots as
  *   float32 pairs (one packed fma for both; each geometry and modulus value read
- *   once for both); 0 = one CTA per patch and shot; until it is set, pairs up to NGLL 6 (not at
+ *   once for both); 0 = one CTA per patch and shot; 2 (default) = pairs up to NGLL 6 (not at
  *   3) for even shot counts and odd ones from 13 on, where they measure faster. The same
  *   arithmetic per shot; results differ only by the rounding order of a few sums. */
 #define SEM_OPT_SHOT_PAIRS 7

@@ -262,10 +262,12 @@ int set_device(sem_ctx* c) {
 }
 
 // Whether several shots are swept in pairs. GB300, 24 steps of about 3.4e5 points: 16 shots in
-// pairs against one CTA a shot 2.78 / 2.99 ms at NGLL 5, 2.59 / 2.89 at 4, 3.57 / 4.15 at 6, but
-// 3.65 / 3.51 at 7, 4.53 / 3.95 at 8, 4.62 / 4.49 at 9 (one resident CTA, or spills, for the two
-// shots' registers); an odd count leaves half of the last pair idle (3 shots at NGLL 5: 0.77 /
-// 0.69 ms), which a tenth gained on the others pays back from 13 shots on.
+// pairs against one CTA a shot 2.78 / 2.99 ms at NGLL 5, 2.59 / 2.89 at 4, 3.57 / 4.15 at 6 and
+// (6.8e5 points) 4.21 / 4.68 at 2, but 3.65 / 3.51 at 7, 4.53 / 3.95 at 8, 4.62 / 4.49 at 9 (one
+// resident CTA, or spills, for the two shots' registers); an odd count leaves half of the last pair
+// idle (3 shots: 0.77 / 0.69 ms at NGLL 5, 1.21 / 1.06 at 2), which a tenth gained on the others
+// pays back from about 13 shots on (13 shots: 2.54 / 2.60 ms at NGLL 5, 3.72 / 3.89 at 2; 11 shots
+// at NGLL 5 2.23 / 2.26).
 bool pair_rule(const sem_ctx* c, int shots) {
   if (c->shot_pairs != 2) return c->shot_pairs == 1;
   return c->ngll <= 6 && c->ngll != 3 && (shots % 2 == 0 || shots >= 13);
@@ -795,7 +797,7 @@ int sem_set_option(sem_ctx* c, int option, long long value) {
       c->stall_test = static_cast<int>(value);
       return SEM_OK;
     case SEM_OPT_SHOT_PAIRS:
-      if (value < 0 || value > 1) return fail(c, SEM_EINVAL, "shot pairs must be 0 or 1");
+      if (value < 0 || value > 2) return fail(c, SEM_EINVAL, "shot pairs must be 0, 1 or 2");
       c->shot_pairs = static_cast<int>(value);
       drop_graph(c);
       return SEM_OK;
