@@ -1136,8 +1136,7 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
     wd |= bit;
     std::memcpy(&r[kIbool * np + pp], &wd, sizeof(uint32_t));
   };
-  // the patch that touches each node last in the sweep (patches are in sweep order); its
-  // local points at the node carry kPatchLastBit
+  // the patch that touches each node last in the sweep (patches are in sweep order): its receivers
   std::vector<int> last_patch(nglob, -1);
   for (int P = 0; P < plan.npatch; ++P)
     for (int k = plan.node_off[P]; k < plan.node_off[P + 1]; ++k) last_patch[plan.nodes[k] & ~kFirstTouchBit] = P;
@@ -1163,10 +1162,6 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
     d.rim0 = static_cast<int>(nrimsums);
     nrimsums += l.rim.size();
     if (nrimsums > 0x7FFFFFFFull) return fail(c, SEM_EINVAL, "mesh too large for int32 indexing");
-    const uint16_t* lid = plan.lid.data() + plan.tab_lid_off[t];
-    for (int q = 0; q < d.nelem * np; ++q)
-      if (last_patch[plan.nodes[plan.node_off[P] + lid[q]] & ~kFirstTouchBit] == P)
-        flag_word(d.slot0 + q / np, q % np, kPatchLastBit);
     const int nnode = plan.node_off[P + 1] - plan.node_off[P];
     for (int k = 0; k < nnode; ++k) {
       if (!(plan.nodes[plan.node_off[P] + k] & kFirstTouchBit)) continue;

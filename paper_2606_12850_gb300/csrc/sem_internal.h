@@ -59,12 +59,10 @@ constexpr uint32_t kFirstTouchBit = 0x80000000u;
 // Bit 30 marks the same for the patch kernel's order (patch colour by patch colour), on the
 // word of the first local point (in patch-table order) of each patch node. Bit 29 marks a
 // local point that is the only one of its patch at its node (its element's team writes it
-// alone). Bit 28 marks, on every local point of a patch node, that this patch is the node's
-// last toucher in the sweep. A first local point with bits 30 and 28 is at an inner node (one
-// that only this patch touches). Node ids are below 2^28.
+// alone). All three serve the forms that write nodes in place (element kernel, persistent
+// sweeps). Node ids are below 2^28.
 constexpr uint32_t kPatchFirstBit = 0x40000000u;
 constexpr uint32_t kAloneBit = 0x20000000u;
-constexpr uint32_t kPatchLastBit = 0x10000000u;
 constexpr uint32_t kNodeMask = 0x0FFFFFFFu;
 constexpr int kMaxNodes = 1 << 28;
 
