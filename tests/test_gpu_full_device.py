@@ -67,7 +67,9 @@ def test_gradients_to_the_host():
 
 def test_surrogate_without_room_for_the_packed_activations():
     """A max_batch whose general buffers fit and whose packed ones (210 MB beside 1.1 GB here) do not:
-    the model is created and the general kernels take its calls."""
+    the model is created and the general tcgen05 kernels take its calls. Their outputs are the packed
+    kernels' bit for bit (the same operands, K order and roundings); gradients differ in the order of
+    float32 sums."""
     from paper_2606_12850_gb300 import surrogate
     spec = surrogate.Spec()
     flat = spec.init_params(9)
@@ -98,8 +100,10 @@ def test_surrogate_without_room_for_the_packed_activations():
         got = use(surrogate.Model(spec, max_batch=64))
     assert ref[0] - got[0] > 120 << 20
     assert abs(got[1] - ref[1]) <= 1e-4 * ref[1]
-    for a, b in zip(ref[2:], got[2:]):
-        assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(a)
+    assert np.array_equal(ref[2], got[2])
+    for name, a in spec.split(ref[3]).items():
+        b = spec.split(got[3])[name]
+        assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(a), name
 
 
 def rel_l2(a, b):
