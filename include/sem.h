@@ -281,7 +281,8 @@ int sem_set_source_nodes(sem_ctx* ctx, int nsrc, const int32_t* node, const doub
  * sources and wavefield): the shots advance together and every element's geometry and
  * moduli are read once per step for all of them. Reallocates the wavefields, zeroes the
  * state and the step counter and clears the sources (set them again). nshots >= 1; the
- * wavefields take 3 * 16 * nglob * nshots bytes. Requires sem_set_mesh. */
+ * wavefields take 3 * 16 * nglob * nshots bytes (an odd nshots > 1 the room of one more). With
+ * SEM_ENOMEM the context keeps the shots it had, from rest. Requires sem_set_mesh. */
 int sem_set_shots(sem_ctx* ctx, int nshots);
 
 /* Point forces per shot: source s acts only in shot shot[s] (0 <= shot[s] < nshots), with

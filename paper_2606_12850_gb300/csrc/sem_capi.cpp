@@ -139,7 +139,9 @@ int fail(sem_ctx* c, int code, const std::string& msg) {
   return code;
 }
 
+// (the runtime's last error is taken with it, or the next launch would report it once more)
 int cuda_fail(sem_ctx* c, cudaError_t e, const char* what) {
+  cudaGetLastError();
   return fail(c, SEM_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -164,7 +166,10 @@ int dev_alloc(sem_ctx* c, T** p, size_t count) {
   if (count == 0) return SEM_OK;
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, count * sizeof(T));
-  if (e != cudaSuccess) return fail(c, SEM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(c, SEM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   *p = static_cast<T*>(q);
   c->dev_bytes += count * sizeof(T);
   return SEM_OK;
@@ -175,7 +180,6 @@ int dev_alloc(sem_ctx* c, T** p, size_t count) {
 int alloc_partials(sem_ctx* c) {
   const int r = dev_alloc(c, &c->d_rimsums, kNodeStride * c->nrimsums * padded_shots(c->shots));
   if (r != SEM_ENOMEM) return r;
-  cudaGetLastError();
   c->err.clear();
   return SEM_OK;
 }
@@ -1240,8 +1244,10 @@ static int set_mesh_impl(sem_ctx* c, int nspec, int nglob, const int32_t* ibool,
       (r = dev_alloc(c, &c->d_rblocks, c->rblocks.size())) ||
       (r = dev_alloc(c, &c->d_u, nf)) ||
       (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf)) ||
-      (r = dev_alloc(c, &c->d_minv, static_cast<size_t>(nglob))) || (r = alloc_partials(c)))
+      (r = dev_alloc(c, &c->d_minv, static_cast<size_t>(nglob))) || (r = alloc_partials(c))) {
+    c->have_mesh = false;  // what is missing must not be launched on
     return r;
+  }
   // geometry and ibool travel once; the material fields are written on the device
   SEM_CUDA(c, cudaMemcpyAsync(c->d_rec, c->rec.data(), c->rec.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   SEM_CUDA(c, cudaMemcpyAsync(c->d_order, c->order.data(), c->order.size() * sizeof(int), cudaMemcpyHostToDevice,
@@ -1438,8 +1444,6 @@ int sem_locate_nodes(sem_ctx* c, int npts, const double* xyz, const double* surf
   return SEM_OK;
 }
 
-// The point sources of the fused sweep: entry s (internal node, shot, force) goes to the patch
-// that touches its node last; the descriptors name each patch's range.
 // The patch descriptors and rim blocks, after their sources or receivers changed.
 static int upload_places(sem_ctx* c) {
   SEM_CUDA(c, cudaMemcpy(c->d_pdesc, c->pdesc.data(), c->pdesc.size() * sizeof(PatchDesc), cudaMemcpyHostToDevice));
@@ -1448,6 +1452,8 @@ static int upload_places(sem_ctx* c) {
   return SEM_OK;
 }
 
+// The point sources of the fused sweep: entry s (internal node, shot, force) goes to the patch of
+// its inner node, or to the block of its rim node; the descriptors name the ranges.
 static int set_patch_sources(sem_ctx* c, const std::vector<int>& nodes, const std::vector<int>& shots,
                              const std::vector<double>& forces) {
   if (c->npatch <= 0) return SEM_OK;
@@ -1460,8 +1466,10 @@ static int set_patch_sources(sem_ctx* c, const std::vector<int>& nodes, const st
   std::stable_sort(by_place.begin(), by_place.end(),
                    [](const std::pair<int, int>& x, const std::pair<int, int>& y) { return x.first < y.first; });
   std::vector<PatchSrc> list, rim;
-  for (PatchDesc& d : c->pdesc) d.src_off = d.nsrc = 0;
-  for (RimBlock& b : c->rblocks) b.src_off = b.nsrc = 0;
+  int r = SEM_OK;
+  size_t ninner = 0;
+  for (const std::pair<int, int>& x : by_place) ninner += x.first < c->npatch;
+  if ((r = dev_alloc(c, &c->d_psrc, ninner)) || (r = dev_alloc(c, &c->d_rsrc, nodes.size() - ninner))) return r;
   for (const std::pair<int, int>& x : by_place) {
     PatchSrc e{};
     e.node = nodes[x.second];
@@ -1474,13 +1482,35 @@ static int set_patch_sources(sem_ctx* c, const std::vector<int>& nodes, const st
     if (n++ == 0) off = static_cast<int>(to.size());
     to.push_back(e);
   }
-  int r = dev_alloc(c, &c->d_psrc, list.size());
-  if (r || (r = dev_alloc(c, &c->d_rsrc, rim.size()))) return r;
   if (!list.empty())
     SEM_CUDA(c, cudaMemcpy(c->d_psrc, list.data(), list.size() * sizeof(PatchSrc), cudaMemcpyHostToDevice));
   if (!rim.empty())
     SEM_CUDA(c, cudaMemcpy(c->d_rsrc, rim.data(), rim.size() * sizeof(PatchSrc), cudaMemcpyHostToDevice));
   return upload_places(c);
+}
+
+// No point sources (no receivers) until their new lists are on the device: a call that runs out of
+// memory half-way leaves a context without them, not descriptors that name freed lists.
+static int drop_sources(sem_ctx* c) {
+  drop_graph(c);
+  c->dev_bytes -= c->nsrc * (2 * sizeof(int) + 3 * sizeof(double) + sizeof(PatchSrc));
+  c->nsrc = 0;
+  bool any = false;
+  for (PatchDesc& d : c->pdesc) any |= d.nsrc > 0, d.src_off = d.nsrc = 0;
+  for (RimBlock& b : c->rblocks) any |= b.nsrc > 0, b.src_off = b.nsrc = 0;
+  return any ? upload_places(c) : SEM_OK;
+}
+static int drop_receivers(sem_ctx* c) {
+  drop_graph(c);
+  size_t nrim = 0;
+  for (const RimBlock& b : c->rblocks) nrim += b.nrec;
+  if (c->nrec)
+    c->dev_bytes -= (2 * c->nrec + 2 * c->nrnodes + 1) * sizeof(int) + (c->nrec + nrim) * sizeof(PatchRecv);
+  c->nrec = c->nrnodes = 0;
+  bool any = false;
+  for (PatchDesc& d : c->pdesc) any |= d.nrec > 0, d.rec_off = d.nrec = d.nrec_in = 0;
+  for (RimBlock& b : c->rblocks) any |= b.nrec > 0, b.rec_off = b.nrec = 0;
+  return any ? upload_places(c) : SEM_OK;
 }
 
 static int set_sources_impl(sem_ctx* c, int nsrc, const int32_t* shot, const int32_t* node, const double* force,
@@ -1518,8 +1548,7 @@ static int set_sources_impl(sem_ctx* c, int nsrc, const int32_t* shot, const int
   int r = set_device(c);
   if (r) return r;
   cudaStreamSynchronize(c->stream);
-  c->dev_bytes -= c->nsrc * (2 * sizeof(int) + 3 * sizeof(double));
-  c->nsrc = static_cast<int>(nodes.size());
+  if ((r = drop_sources(c))) return r;
   if ((r = dev_alloc(c, &c->d_src_node, nodes.size())) || (r = dev_alloc(c, &c->d_src_shot, shots.size())) ||
       (r = dev_alloc(c, &c->d_src_force, forces.size())))
     return r;
@@ -1529,9 +1558,9 @@ static int set_sources_impl(sem_ctx* c, int nsrc, const int32_t* shot, const int
     SEM_CUDA(c, cudaMemcpy(c->d_src_force, forces.data(), forces.size() * sizeof(double), cudaMemcpyHostToDevice));
   }
   if ((r = set_patch_sources(c, nodes, shots, forces))) return r;
+  c->nsrc = static_cast<int>(nodes.size());
   c->f0 = f0;
   c->t0 = t0;
-  drop_graph(c);
   return SEM_OK;
 }
 
@@ -1649,34 +1678,49 @@ int sem_set_shots(sem_ctx* c, int nshots) {
   int r = set_device(c);
   if (r) return r;
   cudaStreamSynchronize(c->stream);
-  const size_t old = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots) * sizeof(float);
-  c->dev_bytes -= 3 * old;
+  if ((r = drop_sources(c))) return r;  // sources name shots: set them again
+  const size_t slots = kNodeStride * padded_shots(c->shots) * sizeof(float), field = slots * static_cast<size_t>(c->nglob);
+  c->dev_bytes -= 3 * field;
   if (c->d_rimsums) {
-    c->dev_bytes -= kNodeStride * c->nrimsums * padded_shots(c->shots) * sizeof(float);
+    c->dev_bytes -= slots * c->nrimsums;
     cudaFree(c->d_rimsums);
     c->d_rimsums = nullptr;
   }
   if (c->d_f) {
-    c->dev_bytes -= old;
+    c->dev_bytes -= field;
     cudaFree(c->d_f);
     c->d_f = nullptr;
   }
-  c->shots = nshots;
-  const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(nshots);
-  if ((r = dev_alloc(c, &c->d_u, nf)) || (r = dev_alloc(c, &c->d_v, nf)) || (r = dev_alloc(c, &c->d_a, nf)) ||
-      (r = alloc_partials(c)))
-    return r;
+  const size_t rest = c->dev_bytes;
+  size_t nf = 0;
+  auto allocate = [&](int shots) -> int {
+    c->shots = shots;
+    c->dev_bytes = rest;
+    nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(shots);
+    int q = SEM_OK;
+    if ((q = dev_alloc(c, &c->d_u, nf)) || (q = dev_alloc(c, &c->d_v, nf)) || (q = dev_alloc(c, &c->d_a, nf))) return q;
+    return alloc_partials(c);
+  };
+  const int shots = c->shots;
+  std::string why;
+  if ((r = allocate(nshots))) {  // back to the shots there were, from rest
+    why = c->err;
+    for (float** p : {&c->d_u, &c->d_v, &c->d_a}) {
+      if (*p) cudaFree(*p);
+      *p = nullptr;
+    }
+    if (allocate(shots)) {
+      c->have_mesh = false;
+      return r;
+    }
+  }
   SEM_CUDA(c, cudaMemsetAsync(c->d_u, 0, nf * sizeof(float), c->stream));
   SEM_CUDA(c, cudaMemsetAsync(c->d_v, 0, nf * sizeof(float), c->stream));
   SEM_CUDA(c, cudaMemsetAsync(c->d_a, 0, nf * sizeof(float), c->stream));
   SEM_CUDA(c, cudaStreamSynchronize(c->stream));
   c->pending = false;
   c->steps = 0;
-  c->nsrc = 0;  // sources name shots: set them again
-  int rs = set_patch_sources(c, {}, {}, {});
-  if (rs) return rs;
-  drop_graph(c);
-  return SEM_OK;
+  return r ? fail(c, r, why) : SEM_OK;
 }
 
 int sem_set_receivers(sem_ctx* c, int nrec, const double* xyz, int32_t* node_out) {
@@ -1701,8 +1745,7 @@ int sem_set_receiver_nodes(sem_ctx* c, int nrec, const int32_t* node) {
   int r = set_device(c);
   if (r) return r;
   cudaStreamSynchronize(c->stream);
-  c->dev_bytes -= c->nrec * sizeof(int) + (2 * c->nrnodes + 1 + c->nrec) * sizeof(int);
-  c->nrec = nrec;
+  if ((r = drop_receivers(c))) return r;
   std::vector<int> internal(nrec);
   for (int k = 0; k < nrec; ++k) internal[k] = c->node_new[node[k]];
   // distinct receiver nodes and their receivers in ascending order (adjoint injection)
@@ -1717,7 +1760,6 @@ int sem_set_receiver_nodes(sem_ctx* c, int nrec, const int32_t* node) {
     }
   }
   if (nrec > 0) roff.push_back(nrec);
-  c->nrnodes = static_cast<int>(rnode.size());
   if ((r = dev_alloc(c, &c->d_rec_node, static_cast<size_t>(nrec))) ||
       (r = dev_alloc(c, &c->d_rnode, rnode.size())) || (r = dev_alloc(c, &c->d_roff, rnode.empty() ? 0 : roff.size())) ||
       (r = dev_alloc(c, &c->d_rlist, byn.size())))
@@ -1739,8 +1781,9 @@ int sem_set_receiver_nodes(sem_ctx* c, int nrec, const int32_t* node) {
     std::sort(at.begin(), at.end(), [](const Place& x, const Place& y) {
       return x.patch != y.patch ? x.patch < y.patch : x.rim != y.rim ? x.rim < y.rim : x.r < y.r;
     });
-    for (PatchDesc& d : c->pdesc) d.rec_off = d.nrec = d.nrec_in = 0;
-    for (RimBlock& b : c->rblocks) b.rec_off = b.nrec = 0;
+    size_t nrim = 0;
+    for (const Place& x : at) nrim += x.rim;
+    if ((r = dev_alloc(c, &c->d_precv, at.size())) || (r = dev_alloc(c, &c->d_rrecv, nrim))) return r;
     std::vector<PatchRecv> list(at.size()), rim;
     std::vector<std::pair<int, int>> by_block;  // (rim block, receiver)
     for (size_t k = 0; k < at.size(); ++k) {
@@ -1756,14 +1799,14 @@ int sem_set_receiver_nodes(sem_ctx* c, int nrec, const int32_t* node) {
       if (b.nrec++ == 0) b.rec_off = static_cast<int>(rim.size());
       rim.push_back(PatchRecv{internal[x.second], x.second});
     }
-    if ((r = dev_alloc(c, &c->d_precv, list.size())) || (r = dev_alloc(c, &c->d_rrecv, rim.size()))) return r;
     if (!list.empty())
       SEM_CUDA(c, cudaMemcpy(c->d_precv, list.data(), list.size() * sizeof(PatchRecv), cudaMemcpyHostToDevice));
     if (!rim.empty())
       SEM_CUDA(c, cudaMemcpy(c->d_rrecv, rim.data(), rim.size() * sizeof(PatchRecv), cudaMemcpyHostToDevice));
     if ((r = upload_places(c))) return r;
   }
-  drop_graph(c);
+  c->nrec = nrec;
+  c->nrnodes = static_cast<int>(rnode.size());
   return SEM_OK;
 }
 
@@ -2021,7 +2064,7 @@ int sem_energy(sem_ctx* c, double* out) {
   int r = set_device(c);
   if (r || (r = finish_state(c))) return r;
   const size_t nf = kNodeStride * static_cast<size_t>(c->nglob) * padded_shots(c->shots);
-  if (!c->d_f) {
+  if (!c->d_f || !c->d_partials) {
     if ((r = dev_alloc(c, &c->d_f, nf)) || (r = dev_alloc(c, &c->d_partials, 2 * static_cast<size_t>(kEnergyBlocks))))
       return r;
     SEM_CUDA(c, cudaMemsetAsync(c->d_f, 0, nf * sizeof(float), c->stream));

@@ -85,7 +85,10 @@ template <typename T>
 int sg_alloc(sg_model* m, T** p, size_t count) {
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-  if (e != cudaSuccess) return sg_fail(m, SEM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // or the next launch would report it once more
+    return sg_fail(m, SEM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   m->allocs.push_back(q);
   m->dev_bytes += count * sizeof(T);
   *p = static_cast<T*>(q);
@@ -356,7 +359,6 @@ int sg_create(sg_model** out, int device, void* stream, int in_dim, int hidden, 
     const size_t have = m->allocs.size(), bytes = m->dev_bytes;
     r = alloc_packed(m);
     if (r == SEM_ENOMEM) {  // no room for it: the general kernels, whose buffers are there, take every call
-      cudaGetLastError();
       cudaStreamSynchronize(m->stream);
       for (size_t i = have; i < m->allocs.size(); ++i) cudaFree(m->allocs[i]);
       m->allocs.resize(have);

@@ -410,20 +410,25 @@ def sem_set_shot_sources_at(ctx: Ctx, shot, xyz, force=None, moment=None, f0: fl
                                          mo[1] if mo else None, float(f0), float(t0)), "sem_set_shot_sources_at", ctx)
 
 
+def _receivers_set(ctx: Ctx, code: int, n: int, where: str):
+    if code in (-2, -3):  # the old receivers are gone, the new ones did not arrive
+        ctx.nrec = 0
+    _check(code, where, ctx)
+    ctx.nrec = n
+
+
 def sem_set_receivers(ctx: Ctx, xyz) -> np.ndarray:
     """Receivers at positions xyz [nrec][3], snapped to the nearest nodes; returns the nodes."""
     pts, pp = _host(np.atleast_2d(xyz), np.float64)
     n = pts.size // 3
     out = np.empty(n, dtype=np.int32)
-    _check(lib().sem_set_receivers(ctx.handle, n, pp, out.ctypes.data_as(_P)), "sem_set_receivers", ctx)
-    ctx.nrec = n
+    _receivers_set(ctx, lib().sem_set_receivers(ctx.handle, n, pp, out.ctypes.data_as(_P)), n, "sem_set_receivers")
     return out
 
 
 def sem_set_receiver_nodes(ctx: Ctx, node):
     nd, pn = _host(np.atleast_1d(node), np.int32)
-    _check(lib().sem_set_receiver_nodes(ctx.handle, nd.size, pn), "sem_set_receiver_nodes", ctx)
-    ctx.nrec = nd.size
+    _receivers_set(ctx, lib().sem_set_receiver_nodes(ctx.handle, nd.size, pn), nd.size, "sem_set_receiver_nodes")
 
 
 def _state_ptrs(ctx, arrays):

@@ -27,14 +27,12 @@ def full_device(leave=0):
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     held = []
-    while (free := (torch.cuda.mem_get_info()[0] - leave) // (2 << 20) * (2 << 20)) >= 12 << 20:
+    part = 1
+    while (free := (torch.cuda.mem_get_info()[0] - leave) // part // (2 << 20) * (2 << 20)) >= 12 << 20:
         try:
             held.append(torch.empty(free, dtype=torch.uint8, device="cuda"))
         except torch.OutOfMemoryError:
-            try:
-                held.append(torch.empty(free // 2 // (2 << 20) * (2 << 20), dtype=torch.uint8, device="cuda"))
-            except torch.OutOfMemoryError:
-                break
+            part *= 2
     try:
         yield
     finally:
@@ -176,3 +174,54 @@ def test_mesh_without_room_for_the_sweep_s_partials():
     assert rel_l2(b[3], a[3]) <= 1e-6
     for x, y in zip(a[4], b[4]):
         assert rel_l2(y, x) <= 1e-5
+
+
+@pytest.mark.parametrize("what", ["receivers", "sources", "shots", "mesh"])
+def test_set_up_call_that_runs_out_of_memory_leaves_a_usable_context(what):
+    """Receivers, sources, shots or a mesh that do not fit: the call reports it, and the context
+    steps without what it could not take (one shot again; no receivers or sources; no mesh)."""
+    w = inputs.layered_cube(5, n=32, side=2000.0, nrec_side=2)
+    nglob, every = w.mesh.nglob, np.arange(w.mesh.nglob, dtype=np.int32)
+    u = inputs.random_field(nglob, 6, scale=1e-3)
+    big = inputs.layered_cube(5, n=48, side=2000.0, nrec_side=2).mesh if what == "mesh" else None
+    s = sem.setup_workload(w)
+
+    def steps():
+        sem.sem_set_state(s.ctx, u)
+        return sem.sem_run(s.ctx, 13), sem.sem_get_state(s.ctx, want=(True, False, False))[0]
+
+    def again():
+        sem.sem_set_source_nodes(s.ctx, s.src_nodes, w.source_force, w.f0, w.t0)
+        sem.sem_set_receiver_nodes(s.ctx, s.rec_nodes)
+
+    both = steps()
+    sem.sem_set_source_nodes(s.ctx, [], np.zeros((0, 3)), w.f0, 0.0)
+    sourceless = steps()
+    again()
+    steps()  # graphs that hold the present lists
+    with full_device():
+        with pytest.raises(sem.SemError) as info:
+            if what == "receivers":
+                sem.sem_set_receiver_nodes(s.ctx, np.tile(every, 8))
+            elif what == "sources":
+                sem.sem_set_source_nodes(s.ctx, every, np.ones((nglob, 3)), w.f0, 0.0)
+            elif what == "shots":
+                sem.sem_set_shots(s.ctx, 8)
+            else:
+                sem.sem_set_mesh_corners(s.ctx, big.ibool, big.ctrl, big.nglob)
+    assert info.value.code == -2
+    if what == "mesh":
+        with pytest.raises(sem.SemError) as info:
+            sem.sem_step(s.ctx, 1)
+        assert info.value.code == -4
+        return
+    assert s.ctx.shots == 1
+    seis, end = steps()
+    if what == "receivers":
+        assert seis is None and np.array_equal(end, both[1])
+    else:  # none of the old sources either
+        assert np.array_equal(seis, sourceless[0]) and np.array_equal(end, sourceless[1])
+    assert not np.array_equal(both[1], sourceless[1])
+    again()  # and the context takes them again
+    for a, b in zip(steps(), both):
+        assert np.array_equal(a, b)
