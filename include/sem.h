@@ -377,7 +377,8 @@ int sem_check_finite(sem_ctx* ctx);
 /* One matrix-free stiffness application on the device: f_dev = -K u_dev, both
  * [nglob][3] float32 in the caller's node order (Sec. II-B), assembled as SEM_OPT_ASSEMBLY
  * says. Every node of f_dev is written. u_dev and f_dev must not overlap. Allocates
- * nothing. Asynchronous on the context's stream. Does not touch the solver state. */
+ * nothing. Asynchronous on the context's stream. Does not touch the solver state, but shares the
+ * context's scratch: in a graph of the caller's, replay it in order with the context's work. */
 int sem_apply_stiffness(sem_ctx* ctx, const float* u_dev, float* f_dev);
 
 /* Same with node_stride floats per node, 3 or 4. Stride 3 is sem_apply_stiffness. Stride 4

@@ -49,13 +49,13 @@ struct sem_ctx {
   int npatch = 0, pmax_nodes = 0, ptables = 0;
   int stall_test = 0;               // SEM_OPT_SWEEP_STALL_TEST (one-shot)
   int fuse_newmark = 2;             // SEM_OPT_FUSED_NEWMARK: Newmark update in the patch sweep
-                                    // (1 on, 0 off, 2 on for a single shot)
+                                    // (0 off, 1 and 2 on)
   int shot_pairs = 2;               // SEM_OPT_SHOT_PAIRS: 1 pairs, 0 one CTA a shot, 2 (default) by pair_rule
   PatchShape shape_opt{0, 0, 0};    // SEM_OPT_PATCH_SHAPE for the next sem_set_mesh (0: the order's)
   PatchShape shape{0, 0, 0};        // the bricks of the current mesh
   std::vector<PatchDesc> pdesc;     // host copy of the patch descriptors
   std::vector<int> last_patch;      // internal node -> the patch that touches it last
-  int assembly = 0;                 // SEM_OPT_ASSEMBLY: 0 patches, one launch per colour,
+  int assembly = 0;                 // SEM_OPT_ASSEMBLY: 0 patches in one launch and a rim pass,
                                     // 1 elements, 2 persistent patch sweep, 3 atomic ablation
   int slabs = 1;                    // spatial slabs of the sweep order
   int slabs_opt = 0;                // requested slab count (0 = automatic)
@@ -829,7 +829,7 @@ int sem_set_option(sem_ctx* c, int option, long long value) {
     case SEM_OPT_ASSEMBLY:
       if (value < 0 || value > 3)
         return fail(c, SEM_EINVAL,
-                    "assembly must be 0 (patch colours), 1 (elements), 2 (persistent patch sweep) or 3 (atomic "
+                    "assembly must be 0 (patches), 1 (elements), 2 (persistent patch sweep) or 3 (atomic "
                     "ablation)");
       c->assembly = static_cast<int>(value);
       drop_graph(c);
@@ -2157,8 +2157,9 @@ int sem_adjoint_begin(sem_ctx* c) {
 // SEM_OPT_FUSED_NEWMARK not 0).
 bool fused_adjoint(const sem_ctx* c) { return fused_sweep(c); }
 
-// One adjoint step: the sweep of lam with, at each node's last touch, the residual injection
-// and the leapfrog (or, unfused, the sweep, then the injection and leapfrog passes). G_dev is
+// One adjoint step: the sweep of lam and its rim pass with, where a node's force is complete, the
+// residual injection and the leapfrog (or, unfused, the sweep, then the injection and leapfrog
+// passes). G_dev is
 // the residual [nrec][3]; with idx it is taken from the device's adjoint counter (G_dev then
 // only says whether there is one).
 static int adjoint_sweep_step(sem_ctx* c, const float* G_dev, const DevCtl* idx, int back = 0) {
@@ -2208,9 +2209,9 @@ int sem_adjoint_accumulate(sem_ctx* c, const float* u_lo, const float* u_mid, co
   return SEM_OK;
 }
 
-// One adjoint step (sweep of lam, residual injection and leapfrog, sensitivity terms) with
-// its residual and snapshots named by the device's adjoint counter less k: the sweep of lam on the context's stream, the
-// sensitivity terms on the auxiliary stream as soon as the sweep is done, so that they overlap
+// One adjoint step (sweep of lam, residual injection and leapfrog, sensitivity terms) with its
+// residual and snapshots named by the device's adjoint counter less k: the sweep of lam and its
+// rim pass on the context's stream, the sensitivity terms on the auxiliary stream as soon as the sweep is done, so that they overlap
 // the next step's sweep. That sweep only writes the buffer of lam^{m+1}, which these terms do
 // not read; the sweep after it overwrites lam^{m-1}, so it waits for them (ev_sens ring).
 static int adjoint_indexed_step(sem_ctx* c, bool hasG, int k) {
@@ -2526,7 +2527,7 @@ void group_drop(sem_group* g) {
 }
 
 // Whether the group's steps can run as persistent sweeps: every context one shot on the
-// per-colour patch assembly, at most kMaxSweepColors patch colours.
+// patch assembly, at most kMaxSweepColors patch colours.
 bool group_persistent_ok(const sem_group* g) {
   if (g->mode != 1 || g->ctx.size() > static_cast<size_t>(kMaxGroupModels)) return false;
   for (const sem_ctx* c : g->ctx)

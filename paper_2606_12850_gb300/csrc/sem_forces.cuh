@@ -613,24 +613,23 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
 }
 
 // ---------------------------------------------------------------------------------------
-// Patch kernel (Sec. II-B stiffness action with the Sec. IV-C coloured assembly applied to
+// Patch kernels (Sec. II-B stiffness action with the Sec. IV-C coloured assembly applied to
 // patches of elements): one CTA per patch, a brick of up to PE neighbouring elements whose
-// records are consecutive; the launches of one sweep take the patch colours in order.
+// records are consecutive.
 //  0. bulk-prefetch the patch's records into L2, then wait for the previous grid;
-//  1. every team gathers its own elements' points through the records' ibool words, as the
-//     element kernel does (teams run independently; the nodes the patch's elements share
-//     are read once from DRAM and then from L1);
+//  1. every team gathers its own elements' points through the records' ibool words (teams run
+//     independently);
 //  2-3. every element's forces (team_element_forces);
-//  4a. each team adds the forces of its points that are alone at their patch node (inside
-//     one element of the patch: 512 of the 729 nodes of a 2 x 2 x 2 brick at NGLL 5) to the
-//     node, with no wait for the other teams;
-//  4b. after one CTA barrier, per shared patch node: the forces of the local points that
-//     meet there summed in the fixed order of the patch table (ascending element, then
-//     point; kPatchSlots slots per node read as one 16-byte word), then added to the node.
-//  A node is stored instead of added at its first touch in patch-colour order
-//  (kPatchFirstBit on the ibool word of the node's first local point in the patch).
-//  Patches of one colour share no node, so there are no atomics, and the order of every
-//  sum is fixed (bitwise reproducible results).
+//  4. after one CTA barrier, per patch node the forces of the local points that meet there are
+//     summed in the fixed order of the patch table (ascending element, then point; kPatchSlots
+//     slots per node read as one 16-byte word). What happens with the sums is the difference:
+//     the one-launch sweep (patch_forces_kernel, the default) completes the patch's inner nodes
+//     and leaves a partial sum per rim node for the rim pass; the persistent sweeps write nodes
+//     in place, a node stored at its first touch in patch-colour order (kPatchFirstBit on the
+//     ibool word of its first local point in the patch) and added to afterwards, first (4a) the
+//     points alone at their patch node, then (4b) the shared nodes.
+//  Patches of one colour share no node and a sum's parts come in colour order, so there are no
+//  atomics, and the order of every sum is fixed (bitwise reproducible results).
 // Shared memory: one ES-float workspace per element, as in the element kernel.
 // ---------------------------------------------------------------------------------------
 template <int N>
@@ -645,10 +644,9 @@ struct PatchCfg {
   // 0 one warp, 1 a named barrier over the team's warps, 2 the CTA
   static constexpr int KIND = TEAM == 32 ? 0 : TEAM < 256 ? 1 : 2;
   static constexpr int E = TEAM / NL;  // elements per team
-  // the default brick, in elements along the lattice x, y, z (any brick of PE elements runs
-  // the same kernel; GB300, 256 GLL intervals per side, one time step's fused sweep: at NGLL
-  // 5, 1x4x2 0.770 ms against 2x2x2 0.778 and 4x1x2 0.774; at NGLL 7, 1x2x2 0.805 against
-  // 2x2x1 0.810 and 2x1x2 0.811; at NGLL 9, 3x1x1 0.818 against 1x3x1 0.819 and 1x1x3 0.844)
+  // the order's brick, in elements along the lattice x, y, z (any brick of PE elements runs the
+  // same kernel; sem_tune_patch_shape measures them on a given mesh, a few per cent apart; at
+  // NGLL 5 larger meshes take another one, see patch_shape)
   static constexpr int BX = N == 2 ? 4 : N == 3 ? 3 : N == 4 ? 4 : N == 5 || N == 7 ? 1 : N <= 8 ? 2 : N == 9 ? 3 : 2;
   static constexpr int BY = N == 2 ? 4 : N == 3 ? 3 : N == 5 ? 4 : N <= 8 ? 2 : 1;
   static constexpr int BZ = N == 2 ? 4 : N == 3 ? 3 : N <= 5 || N == 7 ? 2 : 1;
@@ -975,8 +973,7 @@ __global__ void __launch_bounds__(PatchCfg<N>::T, PatchCfg<N>::MIN_BLOCKS)
 // 2k + 1 in .y), so one packed fma serves both shots, and every geometry and modulus value
 // read from the records serves both. The workspace is the single-shot layout with every
 // float widened to a pair (an element at twice its single-shot offset; u/F, eta and zeta
-// values as [NP][3] pairs, the ibool words at stride 2), so the patch tables' shared-memory
-// offsets apply doubled. Line owners throughout (Sec. II-B phases as in the single-shot core).
+// values as planes of pairs), so the patch tables' shared-memory offsets apply doubled. Line owners throughout (Sec. II-B phases as in the single-shot core).
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float2 bcast2(float s) { return make_float2(s, s); }
 __device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
@@ -1350,7 +1347,7 @@ __device__ __forceinline__ unsigned int prior_colour_count(const int* __restrict
 // in registers across patches). Returns the patch taken next, or -1 after a wait gave up.
 // When the previous colour had already finished as the patch began (the common case once a
 // colour is under way), the teams write their lone points as soon as their elements are
-// done, as in the per-colour kernel; otherwise one thread waits (bounded) first.
+// done; otherwise one thread waits (bounded) first.
 template <int N, bool LO>
 __device__ __noinline__ int sweep_one_patch(int P, const float* __restrict__ rec, const PatchDesc* __restrict__ desc,
                                             const uint16_t* __restrict__ slot_tab,

@@ -93,11 +93,14 @@ static int order_shape(int n, PatchShape* out) {
   return -1;
 }
 
-// The order's brick. At NGLL 5, meshes of some thousand elements and more take the cube of eight
-// instead, which has 386 rim nodes of 729 rather than 450 of 765: there the rim's traffic counts,
-// most with several shots and where the records no longer fit the 129 MB L2 (GB300, us a step,
-// 2 x 2 x 2 against 1 x 4 x 2: 40 x 36 x 44 170.1 / 174.2, 28^3 66.0 / 66.6, 20^3 25.5 / 25.4, with
-// 32 shots 593 / 604; 12^3 12.0 / 12.3, 8^3 9.15 / 8.69).
+// The order's brick. At NGLL 5, meshes from 4000 elements on take the cube of eight instead, which
+// has 386 rim nodes of 729 rather than 450 of 765: there the rim's traffic counts, most with
+// several shots and where the records no longer fit the 129 MB L2 (GB300, us a step, 2 x 2 x 2
+// against 1 x 4 x 2: 40 x 36 x 44 170.1 / 174.2, 28^3 65.6 / 66.6, 24^3 44.5 / 44.9, 20^3 with 32
+// shots 593 / 604). Below, and with one shot on meshes whose sides four divides, neither is the
+// faster throughout: 20^3 26.4 / 25.1, 18^3 19.0 / 21.2, 16^3 16.9 / 16.9, 14^3 14.2 / 15.4, 12^3
+// 12.7 / 12.5, 10^3 9.9 / 10.4, 8^3 8.69 / 8.63. The line is drawn where the cube is the safer of
+// the two on average; SEM_OPT_PATCH_SHAPE sets either.
 int patch_shape(int n, int nspec, PatchShape* out) {
   const int r = order_shape(n, out);
   if (r == 0 && n == 5 && nspec >= 4000) *out = PatchShape{2, 2, 2};
@@ -226,7 +229,7 @@ int launch_corrector(const DevProblem& p, void* stream) {
 // internal ids, so the fields stream, and neighbouring nodes of a face have neighbouring
 // partials. The entry and the node's state, which no sweep writes at the rim, are loaded
 // while the sweep drains. Bound by DRAM: 119 bytes a rim node (entry, partials, u, v, 1/M read,
-// u, v written), 56 us for the 2.8 M rim nodes of a 48^3 mesh at NGLL 5, 6.0 TB/s.
+// u, v written), 40 us for the 2.28 M rim nodes of a 48^3 mesh at NGLL 5, 6.0 TB/s.
 // ---------------------------------------------------------------------------------------
 template <bool MS, int NM>
 __global__ void __launch_bounds__(256) rim_combine_kernel(const RimLaunch R) {

@@ -134,7 +134,7 @@ int alloc_packed(sg_model* m) {
     m->pC.push_back(w);
     w += static_cast<size_t>(m->cout[st]) * m->cin[st] * 3;
     m->packed_train = m->packed_train && sgk::packed_backward_ok(m->cin[st], m->cout[st], m->up[st]);
-    sums = std::max(sums, static_cast<size_t>(152) * m->cin[st]);
+    sums = std::max(sums, static_cast<size_t>(sgk::kSms) * m->cin[st]);
   }
   sums = std::max(sums, B * 4 * ((m->out_l + 127) / 128) * m->out_c);
   for (int st = 0; m->packed_train && st < m->nstages; ++st) {

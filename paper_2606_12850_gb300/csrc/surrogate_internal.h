@@ -13,6 +13,8 @@ namespace sgk {
 
 using bf16 = __nv_bfloat16;
 
+constexpr int kSms = 152;  // GB300
+
 // How the products run. kind 0: warp-level mma.sync, 128/256 x 64 tiles. kind 1: tcgen05 with
 // the accumulator in tensor memory, 128 x 128 tiles. Both round the operands to bfloat16
 // (nearest even) and accumulate in float32. err: a device word that a kind-1 product sets to 1
@@ -100,7 +102,7 @@ int packed_loss(int B, int Ci, int K, int outC, int Lin, int in_dim, const bf16*
                 const Products& pr, cudaStream_t s);
 int packed_loss_blocks(int B, int outC, int Lin);
 // values the loss buffer holds: what mse_grad and packed_loss leave there for any batch up to B
-// (past 152 column blocks packed_loss has a CTA per 32 channels, more than kLossBlocks of them
+// (past kSms column blocks packed_loss has a CTA per 32 channels, more than kLossBlocks of them
 // from 19488 channels on)
 int loss_values(int B, int outC, int Lin);
 bool packed_backward_ok(int Ci, int Co, int up);
@@ -110,7 +112,7 @@ int pack_conv_t(int Ci, int Co, const bf16* W, bf16* Wt, cudaStream_t s);
 int packed_conv_wgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, const bf16* X, float* dW, float* ws,
                       const Products& pr, cudaStream_t s);
 // The gradient at the layer below: dz = dX gelu'(pre), packed (out, of a layer that upsamples by
-// out_up) or float32 [B][Ci][Lin] (out_f32), and its bias gradients db [Ci] (sums: scratch of 152
+// out_up) or float32 [B][Ci][Lin] (out_f32), and its bias gradients db [Ci] (sums: scratch of kSms
 // Ci floats; both null to leave them out)
 int packed_conv_dgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, const bf16* Wt, const float* pre,
                       bf16* out, int out_up, float* out_f32, float* sums, float* db, const Products& pr,

@@ -728,11 +728,11 @@ int grid_for(size_t n) {
 
 int tile_rows(int M) { return M >= 512 ? 256 : 128; }
 
-// CTAs that fill the GPU once: 152 SMs x resident CTAs of the product kernel
+// CTAs that fill the GPU once: its SMs x resident CTAs of the product kernel
 int splits_for(int M, int N, int K, int kind) {
   const int bm = kind == 1 ? TC_BM : tile_rows(M);
   const int bn = kind == 1 ? TC_BN : BN;
-  const int fill = kind == 1 ? 152 * 3 : 152 * 4;
+  const int fill = kind == 1 ? kSms * 3 : kSms * 4;
   const int tiles = ((M + bm - 1) / bm) * ((N + bn - 1) / bn);
   int s = (fill + tiles - 1) / tiles;
   const int kmax = (K + 255) / 256;

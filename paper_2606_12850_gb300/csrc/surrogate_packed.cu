@@ -1,9 +1,10 @@
-// The surrogate's forward and backward passes on packed activations (sm_103a): every layer's output is stored
-// once, as the bfloat16 values the next product rounds its operand to, in the core-matrix
-// layout that tcgen05 reads, so staging an operand is a few bulk copies and no thread converts
-// or rearranges anything between layers. The float32 pre-activations are stored only where the
-// backward pass needs them. Products, their K order, bias, activation and contraction are those
-// of the general kernels (surrogate_kernels.cu), so results are the same bit for bit.
+// The surrogate's forward and backward passes on packed activations (sm_103a): every layer's
+// output is stored once, as the bfloat16 values the next product rounds its operand to, in the
+// core-matrix layout that tcgen05 reads, so staging an operand is a few bulk copies and no thread
+// converts or rearranges anything between layers. The float32 pre-activations are stored only
+// where the backward pass needs them. The forward products, their K order, bias, activation and
+// contraction are those of the general tcgen05 kernels (surrogate_kernels.cu), and so are its
+// results, bit for bit; gradients differ from theirs in the order of float32 sums.
 //
 // The same layout is K-major for the forward products and the data gradients (rows = times,
 // K = channels) and MN-major for the weight gradients (K = times), where a tap's shift along
@@ -1020,10 +1021,10 @@ int conv_stages(int Ci, int N) {
   while (st >= 2 && conv_smem(Ci, N, st) > kSmemLimit) --st;
   return st;
 }
-// one CTA per SM (152), the same number for every column block
+// one CTA per SM, the same number for every column block
 int conv_grid(int B, int blocks, int Lin) {
   const long long tiles = static_cast<long long>(B) * ((Lin + kRows - 1) / kRows);
-  return blocks * static_cast<int>(std::max<long long>(1, std::min<long long>(152 / blocks, tiles)));
+  return blocks * static_cast<int>(std::max<long long>(1, std::min<long long>(kSms / blocks, tiles)));
 }
 int grid1(size_t n) { return static_cast<int>(std::min<size_t>((n + 255) / 256, 65535)); }
 
@@ -1197,7 +1198,7 @@ int packed_conv_wgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, co
   a.stall_test = pr.stall_test;
   const int ot = (Co + kRows - 1) / kRows;
   const size_t mn = static_cast<size_t>(Co) * Ci * 3;
-  a.splits = std::max(1, std::min({B, 152 / ot, static_cast<int>(ws ? pr.ws_floats / mn : 1)}));
+  a.splits = std::max(1, std::min({B, kSms / ot, static_cast<int>(ws ? pr.ws_floats / mn : 1)}));
   a.dst = a.splits > 1 ? ws : dW;
   const int smem = wgrad_smem(Ci, up, wgrad_stages(Ci, up));
   a.stages = wgrad_stages(Ci, up);
@@ -1233,7 +1234,7 @@ int packed_conv_dgrad(int B, int Ci, int Co, int Lin, int up, const bf16* dZ, co
   a.stall_test = pr.stall_test;
   a.stages = dgrad_stages(Ci, up);
   const int smem = dgrad_smem(Ci, up, a.stages);
-  const int items = B * ((Lin + 2 * kRows - 1) / (2 * kRows)), grid = std::min(152, items);
+  const int items = B * ((Lin + 2 * kRows - 1) / (2 * kRows)), grid = std::min(kSms, items);
   const cudaError_t e = up == 2 ? raise_smem(packed_dgrad_kernel<2>) : raise_smem(packed_dgrad_kernel<1>);
   if (e != cudaSuccess) return static_cast<int>(e);
   if (up == 2)
