@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(256) dense_kernel(const DenseArgs a) {
 // back). The default network's forward pass of 4096 samples in chunks of 256, GB300: 16.6 ms
 // with the general kernels (tc_conv_kernel 12.2, contraction 4.4, dense 2.0), 3.6 ms now, 880
 // TFLOP/s of products; one sample 69 against 27 us, bound by the latency of seven launches.
-// Training: the epilogue goes on to the error against the target, its square (squares16), dy = 2 (y - t) / n, and the packed bfloat16
+// Training: the epilogue goes on to the error against the target, its square (SquareSum), dy = 2 (y - t) / n, and the packed bfloat16
 // gradient x_k dy of every contracted copy; y and dy themselves are not stored (258 us for 256
 // samples, where the convolution, contraction, loss and expansion kernels took 1.7 ms).
 struct ConvArgs {
@@ -304,24 +304,34 @@ __device__ __forceinline__ float warp_sums16(float (&v)[16], int lane) {
 // lane's bits 4 .. 1
 __device__ __forceinline__ int warp_sums16_index(int lane) { return lane >> 1; }
 
-// Sum of the squares of 16 errors. A float32 pair takes them (each square exact as a pair, the
-// sum to about 2^-46) where its range holds them: from 2^-78, below which the low halves of the
-// squares that count would underflow, to float32's largest. Other groups (also all zeros, and
-// NaN) are summed in float64, whose units are too few to take every group.
-__device__ __forceinline__ double squares16(const float (&e)[16]) {
+// A sum of squared errors. A float32 pair takes the squares of 16 errors (each square exact as a
+// pair, the sum to about 2^-46) where its range holds them: their sum from 2^-78, below which the
+// low halves of the squares that count would underflow, to 2^100, which leaves room for every
+// thread's share. Other groups (also all zeros, and NaN) are summed in float64, whose units are too
+// few to take every group (with only the sums over the groups in float64 a training step of the
+// default network took 1448 us, 1435 like this).
+struct SquareSum {
   float hi = 0.f, lo = 0.f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const float sq = e[i] * e[i], sq_lo = fmaf(e[i], e[i], -sq);
-    const float s = hi + sq, z = s - hi;  // two-sum
-    lo += ((hi - (s - z)) + (sq - z)) + sq_lo;
-    hi = s;
+  double wide = 0.0;
+  __device__ __forceinline__ static void two_sum(float& hi, float& lo, float s, float l) {
+    const float t = hi + s, z = t - hi;
+    lo += ((hi - (t - z)) + (s - z)) + l;
+    hi = t;
   }
-  if (hi >= 0x1p-78f && hi <= 0x1.fffffep127f) return static_cast<double>(hi) + static_cast<double>(lo);
-  double d = 0.0;
-  for (int i = 0; i < 16; ++i) d += static_cast<double>(e[i]) * e[i];
-  return d;
-}
+  __device__ __forceinline__ void add16(const float (&e)[16]) {
+    float s = 0.f, l = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float sq = e[i] * e[i];
+      two_sum(s, l, sq, fmaf(e[i], e[i], -sq));
+    }
+    if (s >= 0x1p-78f && s <= 0x1p100f)
+      two_sum(hi, lo, s, l);
+    else
+      for (int i = 0; i < 16; ++i) wide += static_cast<double>(e[i]) * e[i];
+  }
+  __device__ __forceinline__ double value() const { return wide + (static_cast<double>(hi) + static_cast<double>(lo)); }
+};
 
 enum { kHidden = 0, kAnswer = 1, kTrain = 2 };
 
@@ -433,7 +443,7 @@ __global__ void __launch_bounds__(320, 1) packed_conv_kernel(const ConvArgs a) {
   } else {
     const int q = warp & 3, h = (warp - 2) >> 2;
     const uint32_t lanes = static_cast<uint32_t>(q * 32) << 16;
-    double loss = 0.0;
+    SquareSum squares;
     for (int tile = first; tile < ntiles; tile += step, ++issued) {
       const int buf = issued & 1;
       const int b = tile / ntt, s = (tile - b * ntt) * kRows + q * 32 + lane;
@@ -474,7 +484,7 @@ __global__ void __launch_bounds__(320, 1) packed_conv_kernel(const ConvArgs a) {
           if (s < a.Lin) {
 #pragma unroll
             for (int i = 0; i < 16; ++i) sum[i] -= t[i];
-            loss += squares16(sum);
+            squares.add16(sum);
 #pragma unroll
             for (int i = 0; i < 16; ++i) sum[i] *= a.scale;
             const int row = 1 + s, g0 = (32 * nb + 16 * h) / 8, gs = a.outC / 8;
@@ -532,6 +542,7 @@ __global__ void __launch_bounds__(320, 1) packed_conv_kernel(const ConvArgs a) {
       }
     }
     if constexpr (KIND == kTrain) {
+      double loss = squares.value();
 #pragma unroll
       for (int off = 16; off >= 1; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
       if (lane == 0) reinterpret_cast<volatile double*>(sloss)[warp - 2] = loss;
