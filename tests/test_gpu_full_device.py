@@ -1,6 +1,7 @@
 """Calls that need no device memory of their own, or can do without the part they lack, on a device
 that other arrays fill up."""
 import contextlib
+import gc
 
 import numpy as np
 import pytest
@@ -24,6 +25,7 @@ def library():
 def full_device(leave=0):
     """Within it, other arrays hold the free device memory but for ``leave`` bytes and less than 12 MB
     more (smaller arrays would come from segments of 20 MB)."""
+    gc.collect()  # contexts of earlier tests, held by tracebacks, must not give memory back within it
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     held = []
