@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(ForceCfg<N>::T, ForceCfg<N>::MIN_BLOCKS)
         if constexpr (CALLER)
           q[r] = load_node3(u + 3 * static_cast<size_t>(__ldg(perm + g)));
         else
-          q[r] = __ldcg(reinterpret_cast<const float4*>(u) + field_slot(nglob, S, g, shot_of((base + r * TEAM) / NP)));
+          q[r] = load_node4(reinterpret_cast<const float4*>(u) + field_slot(nglob, S, g, shot_of((base + r * TEAM) / NP)));
       }
     }
 #pragma unroll

@@ -19,9 +19,15 @@ __device__ __forceinline__ void allow_dependent_grid() { asm volatile("griddepco
 
 // A wavefield the previous launch may have written is read only after that wait and never through
 // the read-only path (__ldg), which is for data no one writes while the kernel runs, its start
-// before the wait included: float4 nodes by __ldcg, the nodes of caller arrays [nglob][3] by
-// plain loads (volatile, so that they stay behind the wait), whose three words share L1 lines
-// (f = -K u on 44 x 36 x 40 elements at NGLL 5: 167 us, with __ldcg 180).
+// before the wait included: float4 nodes by __ldcg in the patch kernels, by plain loads (volatile,
+// so that they stay behind the wait) in the element kernel; so too the nodes of caller arrays
+// [nglob][3], whose three words share L1 lines (f = -K u on 44 x 36 x 40 elements at NGLL 5: 167
+// us, with __ldcg 180).
+__device__ __forceinline__ float4 load_node4(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ float4 load_node3(const float* p) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   asm volatile("ld.global.f32 %0, [%1];" : "=f"(v.x) : "l"(p) : "memory");
