@@ -2211,9 +2211,10 @@ int sem_adjoint_accumulate(sem_ctx* c, const float* u_lo, const float* u_mid, co
 
 // One adjoint step (sweep of lam, residual injection and leapfrog, sensitivity terms) with its
 // residual and snapshots named by the device's adjoint counter less k: the sweep of lam and its
-// rim pass on the context's stream, the sensitivity terms on the auxiliary stream as soon as the sweep is done, so that they overlap
-// the next step's sweep. That sweep only writes the buffer of lam^{m+1}, which these terms do
-// not read; the sweep after it overwrites lam^{m-1}, so it waits for them (ev_sens ring).
+// rim pass on the context's stream, the sensitivity terms on the auxiliary stream as soon as the
+// sweep is done, so that they overlap the next step's sweep. That sweep only writes the buffer of
+// lam^{m+1}, which these terms do not read; the sweep after it overwrites lam^{m-1}, so it waits
+// for them (ev_sens ring).
 static int adjoint_indexed_step(sem_ctx* c, bool hasG, int k) {
   if (k >= 2) SEM_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_sens[k & 1], 0));
   // (with the counter the residual comes from it; the pointer only marks that there is one)

@@ -263,9 +263,10 @@ __global__ void __launch_bounds__(256) dense_kernel(const DenseArgs a) {
 // back). The default network's forward pass of 4096 samples in chunks of 256, GB300: 16.6 ms
 // with the general kernels (tc_conv_kernel 12.2, contraction 4.4, dense 2.0), 3.6 ms now, 880
 // TFLOP/s of products; one sample 69 against 27 us, bound by the latency of seven launches.
-// Training: the epilogue goes on to the error against the target, its square (SquareSum), dy = 2 (y - t) / n, and the packed bfloat16
-// gradient x_k dy of every contracted copy; y and dy themselves are not stored (258 us for 256
-// samples, where the convolution, contraction, loss and expansion kernels took 1.7 ms).
+// Training: the epilogue goes on to the error against the target, its square (SquareSum), dy = 2
+// (y - t) / n, and the packed bfloat16 gradient x_k dy of every contracted copy; y and dy
+// themselves are not stored (258 us for 256 samples, where the convolution, contraction, loss and
+// expansion kernels took 1.7 ms).
 struct ConvArgs {
   int B, Ci, Lin, Lpi, N, stages, blocks;
   const bf16* in;   // packed [B][Ci/8][Lpi][8]
